@@ -517,7 +517,7 @@ pic_status pic_measure_link(void* host, uint64_t bytes, void* cuda_stream, doubl
  *  cuda_stream  stream to run on (NULL = legacy default stream); the call
  *           synchronises it before returning.
  *  iters, rel_res  optional host outputs: iterations and ||r|| / ||b||.
- * Its scratch (569,792 doubles: 4.56 MB = 4.35 MiB) is one fixed array
+ * Its scratch (647,184 doubles: 5.18 MB = 4.94 MiB) is one fixed array
  * inside the library, held on every GPU that loads the library until the
  * process exits. The first call
  * on a device looks up that array's device address (cudaGetSymbolAddress)

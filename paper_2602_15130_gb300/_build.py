@@ -41,7 +41,7 @@ def _stale(target: Path, deps) -> bool:
 
 def build_library(force: bool = False, verbose: bool = False) -> Path:
     BUILD.mkdir(exist_ok=True)
-    headers = [CSRC / "pic_internal.cuh", CSRC / "mixed_common.cuh", CSRC / "ntc_fp64.cuh", PKG.parent / "include" / "pic.h"]
+    headers = [CSRC / "pic_internal.cuh", CSRC / "mixed_common.cuh", CSRC / "ntc_fp64.cuh", CSRC / "grid_exchange.cuh", PKG.parent / "include" / "pic.h"]
     cc = nvcc()
     jobs = []
     for src in SOURCES:

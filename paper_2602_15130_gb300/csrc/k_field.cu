@@ -1,22 +1,21 @@
 // Field solve of Eq. poisson_mms on the periodic node mesh:
 //   rhs : rho at nodes from the per-cell CIC partials, b = rho/eps0 -
 //         Lap phi^M - rho^M/eps0 and per-block partial sums of b;
-//   cg  : one cooperative persistent kernel: b -= mean(b), conjugate
-//         gradients on -Lap_h phi = b (7-point, warm start, three grid
-//         barriers per iteration: p update, q = A p with p.q, x/r update
-//         with r.r), zero-mean projection and E = -grad_h phi by central
-//         differences.
+//   cg  : one cooperative persistent kernel: conjugate gradients on
+//         -Lap_h phi = b - mean(b) (7-point, warm start), zero-mean
+//         projection and E = -grad_h phi by central differences.
 // All reductions are per-block partials combined in a fixed order, so a
-// solve is deterministic for a given grid. Grid barriers are bounded: a
-// wait that exceeds ~2 s of SM clock sets a timeout flag and the kernel
-// returns.
+// solve is deterministic for a given grid. Waits over the grid are bounded
+// (grid_exchange.cuh).
+#include <type_traits>
+
+#include "grid_exchange.cuh"
 #include "pic_internal.cuh"
 
 namespace pic {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr long long kBarrierCycles = 4000000000LL;
 
 inline int blocks_for(int64_t n, int t = kThreads) {
   int64_t b = (n + t - 1) / t;
@@ -139,71 +138,28 @@ struct CgArgs {
   int n;
   int64_t ncell;
   double inv_h2, two_h;
-  double *b, *x, *r, *p0, *p1, *q;
-  const double* rhs_part;
+  const double* b;
+  double *x, *r, *p0, *p1, *q;
+  const double* rhs_part;  // block partial sums of b, or nullptr: summed here
   int rhs_blocks;
-  double* red;  // [4][gridDim.x]
-  unsigned int* bar;
-  int* info;    // [0] iterations [1] status (1 = no convergence) [2] timeout
+  GridSlot* slots;         // exchange_slots(gridDim.x) of them
+  unsigned launch;         // the launch's number: never zero, never the same twice on these slots
+  int* info;    // [0] iterations [1] status (1 = no convergence) [2] number of a launch that timed out
   int* flags;   // sticky context flags
   double* res;
-  int skip_block = -1;  // failure injection: this block leaves before its first barrier
+  int skip_block = -1;  // failure injection: this block leaves before its first exchange
   double tol;
   int maxit;
   double *E0, *E1, *E2;
   long long* hist = nullptr;  // per-step history row: [0] iterations
 };
 
-// Grid barrier for a cooperative grid, bounded in time.
-__device__ __forceinline__ bool grid_barrier(unsigned int* bar, int* info, int* flags) {
-  // monotonic arrival counter (zero at launch): the k-th barrier of the
-  // launch is passed once the counter reaches k gridDim.x; the wait is
-  // bounded, after which the timeout flag is set and every block returns
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int arrived = atomicAdd(bar, 1u) + 1u;
-    const unsigned int target = (arrived + gridDim.x - 1u) / gridDim.x * gridDim.x;
-    ok = 1;
-    const long long t0 = clock64();
-    while (*(volatile unsigned int*)bar < target) {
-      if (clock64() - t0 > kBarrierCycles) {
-        atomicOr(info + 2, 1);
-        atomicOr(flags, 4);
-        ok = 0;
-        break;
-      }
-    }
-    __threadfence();
-    if (ok && *((volatile int*)(info + 2))) ok = 0;
-  }
-  __syncthreads();
-  return ok != 0;
-}
-
-// total of gridDim.x partials in fixed order, in every thread
-__device__ __forceinline__ double grid_total(const double* part, int m, double* sh) {
-  const int lane = threadIdx.x & 31;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double s = 0.0;
-    for (int i = lane; i < m; i += 32) s += ((volatile const double*)part)[i];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) sh[0] = s;
-  }
-  __syncthreads();
-  return sh[0];
-}
-
-// the six periodic neighbours of node id = i + n (j + n k), 32-bit indices
-// (n^3 < 2^31): x+, x-, y+, y-, z+, z-
+// periodic neighbours of node id = i + n (j + n k), 32-bit indices (n^3 <
+// 2^31): x+, x-, y+, y-, z+, z-
 struct Nbr {
   int xp, xm, yp, ym, zp, zm;
 };
-__device__ __forceinline__ Nbr neighbours(int id, int n, int nn) {
-  const int i = id % n, j = (id / n) % n, k = id / nn;
+__device__ __forceinline__ Nbr neighbours(int id, int i, int j, int k, int n, int nn) {
   Nbr b;
   b.xp = i == n - 1 ? id - (n - 1) : id + 1;
   b.xm = i == 0 ? id + (n - 1) : id - 1;
@@ -214,126 +170,245 @@ __device__ __forceinline__ Nbr neighbours(int id, int n, int nn) {
   return b;
 }
 
-// One block per SM of 1024 threads keeps the grid barriers and the
-// per-block partial sums short.
-constexpr int kCgThreads = 1024;
+// Launch shape of the solve. The FP64 pipe does two lanes per SM and clock,
+// so a warp's FP64 instruction holds it for 19 cycles (measured): the nodes are spread
+// over every SM, one block each, with as few threads as hold them (32 at
+// least), npt nodes a thread in registers (1, 2, 4 or 8; 0: more than that,
+// the vectors stay in memory).
+constexpr int kCgThreads = 512;
 
+struct CgShape {
+  int npt, threads, grid;
+};
+inline CgShape cg_shape(int64_t m, int sms) {
+  CgShape s;
+  if (sms > kMaxExchangeBlocks) sms = kMaxExchangeBlocks;
+  const int64_t per = (m + sms - 1) / sms;  // nodes an SM
+  s.npt = per <= kCgThreads ? 1 : per <= 2 * kCgThreads ? 2 : per <= 4 * kCgThreads ? 4 : per <= 8 * kCgThreads ? 8 : 0;
+  if (s.npt == 0) {
+    s.threads = kCgThreads;
+    s.grid = sms;
+    return s;
+  }
+  s.threads = (int)(((per + s.npt - 1) / s.npt + 31) / 32 * 32);
+  s.grid = (int)((m + (int64_t)s.npt * s.threads - 1) / ((int64_t)s.npt * s.threads));
+  return s;
+}
+
+// Conjugate gradients, the textbook recurrence. What bounds a small solve is
+// the two reductions over the grid that an iteration cannot do without:
+//  - a reduction and the barrier that goes with it are one exchange
+//    (grid_exchange.cuh), and inside a block the FP64 additions are done by
+//    one warp (a shuffle tree in every warp costs warps x 5 x 19 cycles of
+//    the FP64 pipe);
+//  - p's update needs no barrier of its own where a thread holds one node
+//    (m <= 512 nodes an SM): every thread forms its neighbours' new p from
+//    their r and old p (the same arithmetic, p double-buffered). From two
+//    nodes a thread on, those six extra FP64 operations a node cost more
+//    than the third exchange.
+// Per iteration at 32^3, 48^3 and 64^3 nodes, with the solve's launch: 11.9,
+// 17.8 and 23 us before (256- or 1024-thread blocks, an atomic-counter
+// barrier, three barriers, shuffle trees in every warp), 9.1, 11.4 and 15 us
+// now, two thirds of it in the exchanges.
+
+// The stopping rule ||r|| <= thresh = tol ||b||: the squares decide where
+// they are clearly apart (an FP64 square root takes 600 cycles).
+__device__ __forceinline__ bool done(double bb, double rr, double thresh, double lo2, double hi2) {
+  if (bb == 0.0 || rr < lo2) return true;
+  if (rr > hi2) return false;
+  return sqrt(rr) <= thresh;
+}
+
+template <int NPT>
 __global__ void __launch_bounds__(kCgThreads) k_cg(CgArgs a) {
-  __shared__ double sh[40];
+  constexpr bool kRegs = NPT > 0, kRecompute = NPT == 1;
+  constexpr int kN = kRegs ? NPT : 1;
+  __shared__ double sh[2 * kCgThreads];
   __shared__ double scal[2];  // scalars formed once per block by thread 0
-  __shared__ int stop;
-  const int n = a.n, nn = a.n * a.n;
-  const int m = (int)a.ncell;
-  const int stride = gridDim.x * blockDim.x;
-  const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const int G = gridDim.x;
-  int ph = 0;  // alternating reduction slots
-  auto slot = [&](int q) { return a.red + (size_t)q * 2 * G; };
+  __shared__ int stop, ok_sh;
   // the others then wait for an arrival that never comes, until the bound
   if ((int)blockIdx.x == a.skip_block) return;
+  const int n = a.n, nn = a.n * a.n;
+  const int m = (int)a.ncell;
+  const int t = threadIdx.x, T = blockDim.x, G = gridDim.x;
+  const int chunk = kRegs ? NPT * T : (m + G - 1) / G;
+  const int64_t lo64 = (int64_t)blockIdx.x * chunk;
+  const int lo = (int)(lo64 < m ? lo64 : m), hi = lo64 + chunk < m ? (int)(lo64 + chunk) : m;
+  GridExchange X{a.slots, G, a.launch, 0u, a.info + 2, a.flags, &ok_sh};
+  double xr[kN], rr_[kN], pr[kN], qr[kN];
+  int ijk[kN];  // the node's coordinates, 10 bits each
+  // f(k, id, i, j, l) for every node of the thread: register slot k, node id
+  // with coordinates (i, j, l)
+  auto each = [&](auto f) {
+    if constexpr (kRegs) {
+#pragma unroll
+      for (int k = 0; k < kN; ++k) {
+        const int id = lo + t + k * T;
+        if (id < hi) f(k, id, ijk[k] & 1023, (ijk[k] >> 10) & 1023, ijk[k] >> 20);
+      }
+    } else {
+      for (int id = lo + t; id < hi; id += T) f(0, id, id % n, (id / n) % n, id / nn);
+    }
+  };
+  if constexpr (kRegs) {
+#pragma unroll
+    for (int k = 0; k < kN; ++k) {
+      const int id = lo + t + k * T;
+      ijk[k] = (id % n) | ((id / n) % n) << 10 | (id / nn) << 20;
+    }
+  }
+  double tot[2];
 
-  // phase 0: zero-mean b, r = b - A x, ||r||^2 and ||b||^2
-  const double mean_b = grid_total(a.rhs_part, a.rhs_blocks, sh) / (double)m;
-  double rr_loc = 0.0, bb_loc = 0.0;
-  for (int id = t0; id < m; id += stride) {
-    const Nbr q = neighbours(id, n, nn);
-    const double bv = a.b[id] - mean_b;
-    a.b[id] = bv;
-    const double* x = a.x;
-    const double nb = x[q.xp] + x[q.xm] + x[q.yp] + x[q.ym] + x[q.zp] + x[q.zm];
-    const double Ax = (6.0 * x[id] - nb) * a.inv_h2;
-    const double rv = bv - Ax;
-    a.r[id] = rv;
-    rr_loc += rv * rv;
-    bb_loc += bv * bv;
-  }
-  {
-    const double s1 = block_sum(rr_loc, sh);
-    if (threadIdx.x == 0) slot(ph)[blockIdx.x] = s1;
-    const double s2 = block_sum(bb_loc, sh);
-    if (threadIdx.x == 0) slot(ph)[G + blockIdx.x] = s2;
-  }
-  if (!grid_barrier(a.bar, a.info, a.flags)) return;
-  double rr = grid_total(slot(ph), G, sh);
-  const double bb = grid_total(slot(ph) + G, G, sh);
-  ph ^= 1;
-  double beta = 0.0;
-  int it = 0, status = 0;
-  double* p = a.p0;
-  const double thresh = a.tol * sqrt(bb);
-  while (true) {
-    if (threadIdx.x == 0) stop = (bb == 0.0 || sqrt(rr) <= thresh) ? 1 : (it >= a.maxit ? 2 : 0);
+  // the mean of b
+  if (a.rhs_part) {
+    if (t < 32) {
+      double s = 0.0;
+      for (int i = t; i < a.rhs_blocks; i += 32) s += a.rhs_part[i];
+      s = warp_sum_d(s);
+      if (t == 0) scal[0] = s / (double)m;
+    }
     __syncthreads();
+  } else {
+    double s = 0.0;
+    each([&](int, int id, int, int, int) { s += a.b[id]; });
+    X.sum<1, false>(&s, tot, sh);
+    if (t == 0) scal[0] = tot[0] / (double)m;
+    __syncthreads();
+    if (!ok_sh) return;
+  }
+  const double mean_b = scal[0];
+  // r = b - A x, ||r||^2 and ||b||^2
+  double loc[2] = {0.0, 0.0};
+  each([&](int k, int id, int i, int j, int l) {
+    const Nbr q = neighbours(id, i, j, l, n, nn);
+    const double bv = a.b[id] - mean_b;
+    const double* x = a.x;
+    const double xc = x[id];
+    const double nb = x[q.xp] + x[q.xm] + x[q.yp] + x[q.ym] + x[q.zp] + x[q.zm];
+    const double rv = bv - (6.0 * xc - nb) * a.inv_h2;
+    a.r[id] = rv;
+    if constexpr (kRegs) {
+      xr[k] = xc;
+      rr_[k] = rv;
+    }
+    loc[0] += rv * rv;
+    loc[1] += bv * bv;
+  });
+  double rr = 0.0, bb = 0.0, thresh = 0.0, lo2 = 0.0, hi2 = 0.0;  // thread 0
+  int it = 0, status = 0;
+  // every sum ends with thread 0's scalars published by one block barrier
+  X.sum<2, true>(loc, tot, sh);
+  if (t == 0) {
+    rr = tot[0];
+    bb = tot[1];
+    thresh = a.tol * sqrt(bb);
+    lo2 = thresh * thresh * (1.0 - 1e-12);
+    hi2 = thresh * thresh * (1.0 + 1e-12);
+    stop = done(bb, rr, thresh, lo2, hi2) ? 1 : (it >= a.maxit ? 2 : 0);
+  }
+  __syncthreads();
+  if (!ok_sh) return;
+  double beta = 0.0;
+  double *p = a.p0, *p_new = kRecompute ? a.p1 : a.p0;
+  while (true) {
     if (stop == 1) break;
     if (stop == 2) { status = 1; break; }
-    // p = r + beta p
-    if (it == 0) {
-      for (int id = t0; id < m; id += stride) p[id] = a.r[id];
+    // p = r + beta p, then q = A p and p.q
+    double pq = 0.0;
+    if constexpr (kRecompute) {
+      each([&](int k, int id, int i, int j, int l) {
+        const Nbr q = neighbours(id, i, j, l, n, nn);
+        const double* r = a.r;
+        const double pc = it == 0 ? rr_[k] : rr_[k] + beta * pr[k];
+        double v[6] = {__ldcg(r + q.xp), __ldcg(r + q.xm), __ldcg(r + q.yp),
+                       __ldcg(r + q.ym), __ldcg(r + q.zp), __ldcg(r + q.zm)};
+        if (it > 0) {
+          const double o[6] = {__ldcg(p + q.xp), __ldcg(p + q.xm), __ldcg(p + q.yp),
+                               __ldcg(p + q.ym), __ldcg(p + q.zp), __ldcg(p + q.zm)};
+#pragma unroll
+          for (int e = 0; e < 6; ++e) v[e] = v[e] + beta * o[e];
+        }
+        p_new[id] = pc;
+        pr[k] = pc;
+        const double qv = (6.0 * pc - (v[0] + v[1] + v[2] + v[3] + v[4] + v[5])) * a.inv_h2;
+        qr[k] = qv;
+        pq += pc * qv;
+      });
+      double* s = p;
+      p = p_new;
+      p_new = s;
     } else {
-      for (int id = t0; id < m; id += stride) p[id] = a.r[id] + beta * p[id];
+      each([&](int k, int id, int, int, int) {
+        const double rv = kRegs ? rr_[k] : a.r[id];
+        const double pc = it == 0 ? rv : rv + beta * (kRegs ? pr[k] : p[id]);
+        p[id] = pc;
+        if constexpr (kRegs) pr[k] = pc;
+      });
+      X.sum<0, true>(nullptr, nullptr, sh);
+      __syncthreads();
+      if (!ok_sh) return;
+      each([&](int k, int id, int i, int j, int l) {
+        const Nbr q = neighbours(id, i, j, l, n, nn);
+        const double nb = __ldcg(p + q.xp) + __ldcg(p + q.xm) + __ldcg(p + q.yp) + __ldcg(p + q.ym) +
+                          __ldcg(p + q.zp) + __ldcg(p + q.zm);
+        const double pc = kRegs ? pr[k] : p[id];
+        const double qv = (6.0 * pc - nb) * a.inv_h2;
+        if constexpr (kRegs) qr[k] = qv;
+        else a.q[id] = qv;
+        pq += pc * qv;
+      });
     }
-    if (!grid_barrier(a.bar, a.info, a.flags)) return;
-    // q = A p, p.q
-    double pq_loc = 0.0;
-    for (int id = t0; id < m; id += stride) {
-      const Nbr q = neighbours(id, n, nn);
-      const double nb = p[q.xp] + p[q.xm] + p[q.yp] + p[q.ym] + p[q.zp] + p[q.zm];
-      const double pc = p[id];
-      const double qv = (6.0 * pc - nb) * a.inv_h2;
-      a.q[id] = qv;
-      pq_loc += pc * qv;
-    }
-    {
-      const double s = block_sum(pq_loc, sh);
-      if (threadIdx.x == 0) slot(ph)[blockIdx.x] = s;
-    }
-    if (!grid_barrier(a.bar, a.info, a.flags)) return;
-    const double pq = grid_total(slot(ph), G, sh);
-    ph ^= 1;
-    if (threadIdx.x == 0) scal[0] = rr / pq;
+    X.sum<1, false>(&pq, tot, sh);
+    if (t == 0) scal[0] = rr / tot[0];
     __syncthreads();
+    if (!ok_sh) return;
     const double alpha = scal[0];
-    double rn_loc = 0.0;
-    for (int id = t0; id < m; id += stride) {
-      a.x[id] += alpha * p[id];
-      const double rv = a.r[id] - alpha * a.q[id];
-      a.r[id] = rv;
-      rn_loc += rv * rv;
-    }
-    {
-      const double s = block_sum(rn_loc, sh);
-      if (threadIdx.x == 0) slot(ph)[blockIdx.x] = s;
-    }
-    if (!grid_barrier(a.bar, a.info, a.flags)) return;
-    const double rr_new = grid_total(slot(ph), G, sh);
-    ph ^= 1;
+    double rn = 0.0;
+    each([&](int k, int id, int, int, int) {
+      if constexpr (kRegs) {
+        xr[k] += alpha * pr[k];
+        rr_[k] = rr_[k] - alpha * qr[k];
+        a.r[id] = rr_[k];
+        rn += rr_[k] * rr_[k];
+      } else {
+        a.x[id] += alpha * p[id];
+        const double rv = a.r[id] - alpha * a.q[id];
+        a.r[id] = rv;
+        rn += rv * rv;
+      }
+    });
     ++it;
-    if (threadIdx.x == 0) scal[1] = rr_new / rr;
+    X.sum<1, kRecompute>(&rn, tot, sh);  // with r (and p) for the neighbours' p
+    if (t == 0) {
+      scal[1] = tot[0] / rr;
+      rr = tot[0];
+      stop = done(bb, rr, thresh, lo2, hi2) ? 1 : (it >= a.maxit ? 2 : 0);
+    }
     __syncthreads();
+    if (!ok_sh) return;
     beta = scal[1];
-    rr = rr_new;
   }
   // zero-mean projection
   double xs = 0.0;
-  for (int id = t0; id < m; id += stride) xs += a.x[id];
-  {
-    const double s = block_sum(xs, sh);
-    if (threadIdx.x == 0) slot(ph)[blockIdx.x] = s;
-  }
-  if (!grid_barrier(a.bar, a.info, a.flags)) return;
-  const double mean_x = grid_total(slot(ph), G, sh) / (double)m;
-  ph ^= 1;
-  for (int id = t0; id < m; id += stride) a.x[id] -= mean_x;
-  if (!grid_barrier(a.bar, a.info, a.flags)) return;
+  each([&](int k, int id, int, int, int) { xs += kRegs ? xr[k] : a.x[id]; });
+  X.sum<1, false>(&xs, tot, sh);
+  if (t == 0) scal[0] = tot[0] / (double)m;
+  __syncthreads();
+  if (!ok_sh) return;
+  const double mean_x = scal[0];
+  each([&](int k, int id, int, int, int) { a.x[id] = (kRegs ? xr[k] : a.x[id]) - mean_x; });
+  X.sum<0, true>(nullptr, nullptr, sh);
+  __syncthreads();
+  if (!ok_sh) return;
   // E = -grad_h phi, second-order central differences
-  for (int id = t0; id < m; id += stride) {
-    const Nbr q = neighbours(id, n, nn);
+  each([&](int, int id, int i, int j, int l) {
+    const Nbr q = neighbours(id, i, j, l, n, nn);
     const double* x = a.x;
-    a.E0[id] = -(x[q.xp] - x[q.xm]) / a.two_h;
-    a.E1[id] = -(x[q.yp] - x[q.ym]) / a.two_h;
-    a.E2[id] = -(x[q.zp] - x[q.zm]) / a.two_h;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.E0[id] = -(__ldcg(x + q.xp) - __ldcg(x + q.xm)) / a.two_h;
+    a.E1[id] = -(__ldcg(x + q.yp) - __ldcg(x + q.ym)) / a.two_h;
+    a.E2[id] = -(__ldcg(x + q.zp) - __ldcg(x + q.zm)) / a.two_h;
+  });
+  if (blockIdx.x == 0 && t == 0) {
     a.info[0] = it;
     a.info[1] = status;
     if (a.hist) a.hist[0] = it;
@@ -341,6 +416,215 @@ __global__ void __launch_bounds__(kCgThreads) k_cg(CgArgs a) {
     if (status) atomicOr(a.flags, 2);
     atomicMax(a.flags + 1, it);
   }
+}
+
+const void* cg_kernel(int npt) {
+  return npt == 1   ? (const void*)k_cg<1>
+         : npt == 2 ? (const void*)k_cg<2>
+         : npt == 4 ? (const void*)k_cg<4>
+         : npt == 8 ? (const void*)k_cg<8>
+                    : (const void*)k_cg<0>;
+}
+
+// The solve on one cluster of 16 blocks, one node a thread, for meshes of at
+// most 8,192 nodes (n <= 20): a block's p lives in its shared memory,
+// neighbours in other blocks are read there, and a sum over the cluster is
+// 16 stores into every block's shared memory and one cluster barrier (400
+// cycles; 2,080 with the sums, where an exchange over the whole grid takes
+// 5,000). With more nodes the cluster's 16 FP64 pipes take longer than the
+// exchanges over all SMs cost: per iteration at 8^3 and 24^3 nodes (there
+// two nodes a thread) 4.4 and 7.9 us against 6.2 and 7.4 us on the grid.
+constexpr int kClusterBlocks = 16;
+constexpr int64_t kClusterNodes = (int64_t)kClusterBlocks * kCgThreads;
+
+__device__ __forceinline__ uint32_t cluster_address(const void* shared, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(shared)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ double ld_cluster(uint32_t a) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kCgThreads) k_cg_cluster(CgArgs a) {
+  __shared__ double sh[2 * kCgThreads];
+  __shared__ double ps[kCgThreads];                      // this block's p
+  __shared__ double part[2][2][kClusterBlocks];          // every block's partials, alternating
+  __shared__ double scal[2];
+  __shared__ int stop;
+  const int n = a.n, nn = a.n * a.n, m = (int)a.ncell;
+  const int t = threadIdx.x, T = blockDim.x;
+  const int id = (int)blockIdx.x * T + t;
+  const bool own = id < m;
+  uint32_t nbr[6];  // the neighbours' p: x+, x-, y+, y-, z+, z-
+  {
+    const Nbr q = neighbours(id, id % n, (id / n) % n, id / nn, n, nn);
+    const int o[6] = {q.xp, q.xm, q.yp, q.ym, q.zp, q.zm};
+#pragma unroll
+    for (int e = 0; e < 6; ++e) nbr[e] = own ? cluster_address(ps + o[e] % T, (uint32_t)(o[e] / T)) : 0u;
+  }
+  auto nbr_sum = [&]() {
+    double v[6];
+#pragma unroll
+    for (int e = 0; e < 6; ++e) v[e] = ld_cluster(nbr[e]);
+    return v[0] + v[1] + v[2] + v[3] + v[4] + v[5];
+  };
+  // Totals over the cluster of two values per thread (or one), in warp 0;
+  // the caller follows with a __syncthreads.
+  int set = 0;
+  double tot[2];
+  auto sum = [&](auto two, double u, double v) {
+    constexpr int kV = decltype(two)::value ? 2 : 1;
+    set ^= 1;
+    sh[t] = u;
+    if (kV == 2) sh[T + t] = v;
+    __syncthreads();
+    if (t < 32) {
+#pragma unroll
+      for (int q = 0; q < kV; ++q) {
+        double s = sh[q * T + t];
+        for (int w = t + 32; w < T; w += 32) s += sh[q * T + w];
+        s = warp_sum_d(s);
+        if (t < kClusterBlocks) st_cluster(cluster_address(&part[set][q][blockIdx.x], (uint32_t)t), s);
+      }
+    }
+    cluster_barrier();
+    if (t < 32) {
+#pragma unroll
+      for (int q = 0; q < kV; ++q) {
+        double s = part[set][q][t & (kClusterBlocks - 1)];
+#pragma unroll
+        for (int off = kClusterBlocks / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        tot[q] = s;
+      }
+    }
+  };
+
+  cluster_barrier();  // every block's shared memory is there
+  if (a.rhs_part) {
+    if (t < 32) {
+      double s = 0.0;
+      for (int i = t; i < a.rhs_blocks; i += 32) s += a.rhs_part[i];
+      s = warp_sum_d(s);
+      if (t == 0) scal[0] = s / (double)m;
+    }
+  } else {
+    sum(std::false_type{}, own ? a.b[id] : 0.0, 0.0);
+    if (t == 0) scal[0] = tot[0] / (double)m;
+  }
+  __syncthreads();
+  const double mean_b = scal[0];
+  // r = b - A x
+  double xr = 0.0, rv = 0.0, pr = 0.0, qr = 0.0, bv = 0.0;
+  if (own) {
+    xr = a.x[id];
+    ps[t] = xr;
+  }
+  cluster_barrier();
+  if (own) {
+    bv = a.b[id] - mean_b;
+    rv = bv - (6.0 * xr - nbr_sum()) * a.inv_h2;
+  }
+  double rr = 0.0, bb = 0.0, thresh = 0.0, lo2 = 0.0, hi2 = 0.0;  // thread 0
+  int it = 0, status = 0;
+  sum(std::true_type{}, rv * rv, bv * bv);
+  if (t == 0) {
+    rr = tot[0];
+    bb = tot[1];
+    thresh = a.tol * sqrt(bb);
+    lo2 = thresh * thresh * (1.0 - 1e-12);
+    hi2 = thresh * thresh * (1.0 + 1e-12);
+    stop = done(bb, rr, thresh, lo2, hi2) ? 1 : (it >= a.maxit ? 2 : 0);
+  }
+  __syncthreads();
+  double beta = 0.0;
+  while (true) {
+    if (stop == 1) break;
+    if (stop == 2) { status = 1; break; }
+    if (own) {
+      pr = it == 0 ? rv : rv + beta * pr;
+      ps[t] = pr;
+    }
+    cluster_barrier();
+    if (own) qr = (6.0 * pr - nbr_sum()) * a.inv_h2;
+    sum(std::false_type{}, pr * qr, 0.0);
+    if (t == 0) scal[0] = rr / tot[0];
+    __syncthreads();
+    const double alpha = scal[0];
+    if (own) {
+      xr += alpha * pr;
+      rv = rv - alpha * qr;
+    }
+    ++it;
+    sum(std::false_type{}, rv * rv, 0.0);
+    if (t == 0) {
+      scal[1] = tot[0] / rr;
+      rr = tot[0];
+      stop = done(bb, rr, thresh, lo2, hi2) ? 1 : (it >= a.maxit ? 2 : 0);
+    }
+    __syncthreads();
+    beta = scal[1];
+  }
+  // zero-mean projection and E
+  sum(std::false_type{}, xr, 0.0);
+  if (t == 0) scal[0] = tot[0] / (double)m;
+  __syncthreads();
+  const double mean_x = scal[0];
+  if (own) {
+    a.x[id] = xr - mean_x;
+    ps[t] = xr - mean_x;
+  }
+  cluster_barrier();
+  if (own) {
+    a.E0[id] = -(ld_cluster(nbr[0]) - ld_cluster(nbr[1])) / a.two_h;
+    a.E1[id] = -(ld_cluster(nbr[2]) - ld_cluster(nbr[3])) / a.two_h;
+    a.E2[id] = -(ld_cluster(nbr[4]) - ld_cluster(nbr[5])) / a.two_h;
+  }
+  if (blockIdx.x == 0 && t == 0) {
+    a.info[0] = it;
+    a.info[1] = status;
+    if (a.hist) a.hist[0] = it;
+    a.res[0] = bb > 0.0 ? sqrt(rr) / sqrt(bb) : 0.0;
+    if (status) atomicOr(a.flags, 2);
+    atomicMax(a.flags + 1, it);
+  }
+  cluster_barrier();  // no block leaves while another reads its shared memory
+}
+
+// Launch the solve: one cluster where the mesh is small, else a cooperative
+// grid over the SMs (always with a failure injection, whose wait is bounded
+// there).
+cudaError_t launch_solve(const CgArgs& args, int sms, cudaStream_t stream) {
+  CgArgs a = args;
+  void* argv[] = {&a};
+  if (a.ncell <= kClusterNodes && a.skip_block < 0) {
+    const int64_t per = (a.ncell + kClusterBlocks - 1) / kClusterBlocks;
+    const void* fn = (const void*)k_cg_cluster;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClusterBlocks;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterBlocks);
+    cfg.blockDim = dim3((unsigned)((per + 31) / 32 * 32));
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, argv);
+  }
+  const CgShape s = cg_shape(a.ncell, sms);
+  return cudaLaunchCooperativeKernel(cg_kernel(s.npt), dim3(s.grid), dim3(s.threads), argv, 0, stream);
 }
 
 struct StoreFieldArgs {
@@ -399,10 +683,11 @@ cudaError_t launch_rhs(pic_ctx* c, double t) {
   return cudaGetLastError();
 }
 
-int cg_threads() { return kCgThreads; }
-const void* cg_kernel_ptr() { return (const void*)k_cg; }
+int cg_blocks(int64_t m, int sms) { return cg_shape(m, sms).grid; }
+// bytes of the exchange inboxes a context of this grid holds
+size_t cg_slot_bytes(int grid) { return exchange_slots((size_t)grid) * sizeof(GridSlot); }
 
-cudaError_t launch_cg_on(pic_ctx* c, double* b, double* x, const double* rhs_part, int rhs_blocks, double* E0,
+cudaError_t launch_cg_on(pic_ctx* c, const double* b, double* x, const double* rhs_part, int rhs_blocks, double* E0,
                          double* E1, double* E2) {
   CgArgs a;
   a.n = c->P.n;
@@ -417,8 +702,8 @@ cudaError_t launch_cg_on(pic_ctx* c, double* b, double* x, const double* rhs_par
   a.q = c->cg_q;
   a.rhs_part = rhs_part;
   a.rhs_blocks = rhs_blocks;
-  a.red = c->cg_red;
-  a.bar = c->cg_bar;
+  a.slots = reinterpret_cast<GridSlot*>(c->cg_red);
+  a.launch = ++c->cg_launch;
   a.info = c->cg_info;
   a.flags = c->flags;
   a.res = c->cg_res;
@@ -430,13 +715,8 @@ cudaError_t launch_cg_on(pic_ctx* c, double* b, double* x, const double* rhs_par
   a.skip_block = c->stall_next_cg ? c->cg_grid - 1 : -1;
   a.hist = c->hist_row;
   c->stall_next_cg = false;
-  cudaError_t e = cudaMemsetAsync(c->cg_bar, 0, 2 * sizeof(unsigned int), c->stream);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(c->cg_info, 0, 3 * sizeof(int), c->stream);
-  if (e != cudaSuccess) return e;
-  void* args[] = {&a};
   prof_begin(c);
-  e = cudaLaunchCooperativeKernel((const void*)k_cg, dim3(c->cg_grid), dim3(kCgThreads), args, 0, c->stream);
+  cudaError_t e = launch_solve(a, c->num_sms, c->stream);
   prof_end(c, KC_CG);
   c->launches++;
   if (e != cudaSuccess) return e;
@@ -484,29 +764,16 @@ namespace pic {
 namespace {
 
 constexpr int64_t kNoallocMaxNodes = 48 * 48 * 48;   // largest mesh: 48^3 nodes
-constexpr int kNoallocMaxGrid = 4096;                  // cooperative blocks
-constexpr int64_t kNoallocPartBlocks = (kNoallocMaxNodes + kThreads - 1) / kThreads;
-// layout in doubles: b copy, r, p0, p1, q [5 N]; partial sums of b; CG
-// reduction slots [4 grid]; 16 words of barrier / status / residual
-constexpr int64_t kNoallocDoubles = 5 * kNoallocMaxNodes + kNoallocPartBlocks + 4 * kNoallocMaxGrid + 16;
+// layout in doubles: r, p0, p1, q [4 N]; the exchange slots (two doubles
+// each); 16 words of status / residual
+constexpr int64_t kNoallocSlots = exchange_slots(kMaxExchangeBlocks);
+constexpr int64_t kNoallocDoubles = 4 * kNoallocMaxNodes + 2 * kNoallocSlots + 16;
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocDoubles];
 
 std::mutex g_noalloc_mutex;
 double* g_noalloc_ptr[64] = {nullptr};
-
-// copy b into the scratch and write per-block partial sums for its mean
-__global__ void __launch_bounds__(kThreads) k_noalloc_prep(const double* b, double* bcopy, double* part, int64_t m) {
-  __shared__ double sh[40];
-  const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double v = 0.0;
-  if (id < m) {
-    v = b[id];
-    bcopy[id] = v;
-  }
-  const double tot = block_sum(v, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
+unsigned g_noalloc_launch[64] = {0};
 
 }  // namespace
 }  // namespace pic
@@ -538,6 +805,7 @@ extern "C" pic_status pic_poisson_solve_noalloc(int32_t n, const double* b, doub
   }
   // one-time set-up per device: the scratch array's device address
   double* base = nullptr;
+  unsigned launch = 0;
   {
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
     if (!g_noalloc_ptr[dev]) {
@@ -549,22 +817,16 @@ extern "C" pic_status pic_poisson_solve_noalloc(int32_t n, const double* b, doub
       g_noalloc_ptr[dev] = (double*)p;
     }
     base = g_noalloc_ptr[dev];
+    launch = ++g_noalloc_launch[dev];
   }
-  int sms = 0, occ = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg, kThreads, 0) != cudaSuccess || occ < 1) {
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
     return PIC_ECUDA;
   }
-  int64_t grid = (m + kThreads - 1) / kThreads;
-  if (grid > (int64_t)occ * sms) grid = (int64_t)occ * sms;
-  if (grid > kNoallocMaxGrid) grid = kNoallocMaxGrid;
-  const int part_blocks = (int)((m + kThreads - 1) / kThreads);
 
-  double* bcopy = base;
-  double* part = base + 5 * kNoallocMaxNodes;
-  double* red = part + kNoallocPartBlocks;
-  int* words = (int*)(red + 4 * kNoallocMaxGrid);   // [0,1] barrier, [2..4] info, [5,6] flags
+  double* slots = base + 4 * kNoallocMaxNodes;
+  int* words = (int*)(slots + 2 * kNoallocSlots);   // [0..2] info, [4,5] flags
   double* res = (double*)(words + 8);
 
   CgArgs a;
@@ -572,37 +834,30 @@ extern "C" pic_status pic_poisson_solve_noalloc(int32_t n, const double* b, doub
   a.ncell = m;
   a.inv_h2 = (double)n * (double)n;
   a.two_h = 2.0 * (1.0 / (double)n);
-  a.b = bcopy;
+  a.b = b;
   a.x = phi;
-  a.r = base + kNoallocMaxNodes;
-  a.p0 = base + 2 * kNoallocMaxNodes;
-  a.p1 = base + 3 * kNoallocMaxNodes;
-  a.q = base + 4 * kNoallocMaxNodes;
-  a.rhs_part = part;
-  a.rhs_blocks = part_blocks;
-  a.red = red;
-  a.bar = (unsigned int*)words;
-  a.info = words + 2;
-  a.flags = words + 5;
+  a.r = base;
+  a.p0 = base + kNoallocMaxNodes;
+  a.p1 = base + 2 * kNoallocMaxNodes;
+  a.q = base + 3 * kNoallocMaxNodes;
+  a.rhs_part = nullptr;
+  a.rhs_blocks = 0;
+  a.slots = reinterpret_cast<GridSlot*>(slots);
+  a.launch = launch;
+  a.info = words;
+  a.flags = words + 4;
   a.res = res;
   a.tol = tol;
   a.maxit = maxit;
   a.E0 = E;
   a.E1 = E + m;
   a.E2 = E + 2 * m;
-  // the array keeps the last call's contents: clear the barrier and status words
+  // the array keeps the last call's contents: clear the status words
   cudaError_t e = cudaMemsetAsync(words, 0, 8 * sizeof(int), stream);
-  if (e == cudaSuccess) {
-    k_noalloc_prep<<<part_blocks, kThreads, 0, stream>>>(b, bcopy, part, m);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) {
-    void* args[] = {&a};
-    e = cudaLaunchCooperativeKernel((const void*)k_cg, dim3((unsigned)grid), dim3(kThreads), args, 0, stream);
-  }
-  int info[5] = {0, 0, 0, 0, 0};
+  if (e == cudaSuccess) e = launch_solve(a, sms, stream);
+  int info[3] = {0, 0, 0};
   double r = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(info, words + 2, 5 * sizeof(int), cudaMemcpyDeviceToHost, stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(info, words, sizeof(info), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&r, res, sizeof(double), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {

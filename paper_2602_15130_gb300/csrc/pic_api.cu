@@ -14,8 +14,8 @@
 namespace pic {
 int dsmc_threads();
 const void* dsmc_kernel_ptr(bool verify);
-int cg_threads();
-const void* cg_kernel_ptr();
+int cg_blocks(int64_t m, int sms);
+size_t cg_slot_bytes(int grid);
 int64_t scan_blocks_needed(int64_t ncell);
 int rhs_blocks_needed(int64_t ncell);
 int err_blocks_needed(int64_t np, int64_t ncell);
@@ -352,7 +352,7 @@ void for_each_buffer(pic_ctx* c, F f) {
   f((void**)&c->corner, 8 * nc * 8);
   f((void**)&c->rho, nc * 8);
   f((void**)&c->rhs_part, (size_t)c->rhs_blocks * 8);
-  f((void**)&c->cg_red, (size_t)4 * c->cg_grid * 8);
+  f((void**)&c->cg_red, cg_slot_bytes(c->cg_grid));
   f((void**)&c->cg_bar, 64);
   f((void**)&c->cg_info, 64);
   f((void**)&c->cg_res, 64);
@@ -838,17 +838,19 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
   c->scan_nblocks = scan_blocks_needed(c->P.ncell);
   c->rhs_blocks = rhs_blocks_needed(c->P.ncell);
   c->err_blocks = err_blocks_needed(c->P.np, c->P.ncell);
-  int occ = 0;
-  const void* cg_fn = c->mixed ? cg32_kernel_ptr() : cg_kernel_ptr();
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cg_fn, cg_threads(), 0);
-  if (e != cudaSuccess || occ < 1) {
-    cudaGetLastError();
-    delete c;
-    return PIC_ECUDA;
+  if (c->mixed) {
+    int occ = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cg32_kernel_ptr(), cg32_threads(), 0);
+    if (e != cudaSuccess || occ < 1) {
+      cudaGetLastError();
+      delete c;
+      return PIC_ECUDA;
+    }
+    const int64_t need = (c->P.ncell + cg32_threads() - 1) / cg32_threads();
+    c->cg_grid = (int)(need < (int64_t)occ * c->num_sms ? need : (int64_t)occ * c->num_sms);
+  } else {
+    c->cg_grid = cg_blocks(c->P.ncell, c->num_sms);
   }
-  c->cg_block = cg_threads();
-  int64_t cg_need = (c->P.ncell + c->cg_block - 1) / c->cg_block;
-  c->cg_grid = (int)(cg_need < (int64_t)occ * c->num_sms ? cg_need : (int64_t)occ * c->num_sms);
   if (c->cg_grid < 1) c->cg_grid = 1;
   // the precision form's Poisson solve: CG preconditioned by a multigrid
   // V-cycle on meshes of 2^k >= 16 nodes per edge, plain CG otherwise
@@ -925,6 +927,7 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
   if (e == cudaSuccess) e = cudaMemsetAsync(c->counters, 0, 64, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 0, 64, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->cg_info, 0, 64, c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->cg_red, 0, cg_slot_bytes(c->cg_grid), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->cg_res, 0, 64, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
@@ -1159,7 +1162,8 @@ pic_status pic_get_state(pic_ctx* c, double* x, double* v) {
 }
 
 pic_status pic_inject_barrier_stall(pic_ctx* c) {
-  if (!c || (c->nrep == 0 && c->cg_grid < 2)) return PIC_EINVAL;
+  // meshes of up to 1024 nodes are refused in either form
+  if (!c || (c->nrep == 0 && (c->cg_grid < 2 || c->P.ncell <= 1024))) return PIC_EINVAL;
   c->stall_next_cg = true;
   return PIC_OK;
 }

@@ -633,10 +633,11 @@ struct pic_ctx {
   double* cg_p[2];
   double* cg_q;
   double* cg_red;   // reduction slots
-  unsigned int* cg_bar;  // grid barrier words
-  int* cg_info;     // [0] iterations, [1] status (0 ok, 1 noconv, 2 timeout)
+  unsigned int* cg_bar;  // grid barrier words (precision form)
+  unsigned cg_launch;    // solves launched on the reduction slots (FP64 form)
+  int* cg_info;     // [0] iterations, [1] status (0 ok, 1 noconv), [2] timeout
   double* cg_res;   // relative residual
-  int cg_grid, cg_block;
+  int cg_grid;
   bool stall_next_cg;  // failure injection: the next CG launch has one block leave before its first barrier
 
   // G^{-1} knot tables (FP64 and FP32)
@@ -756,7 +757,7 @@ cudaError_t launch_rhs(pic_ctx* c, double t);
 cudaError_t launch_cg(pic_ctx* c);             // CG + zero-mean + E
 // the FP64 CG on caller buffers: solves -Lap_h x = b - mean(b) (warm start
 // from x, mean removed from x) and writes E = -grad_h x
-cudaError_t launch_cg_on(pic_ctx* c, double* b, double* x, const double* rhs_part, int rhs_blocks, double* E0,
+cudaError_t launch_cg_on(pic_ctx* c, const double* b, double* x, const double* rhs_part, int rhs_blocks, double* E0,
                          double* E1, double* E2);
 using StepHook = std::function<cudaError_t(int)>;
 cudaError_t step_fp64(pic_ctx* c, int64_t n, const StepHook* hook);
