@@ -574,10 +574,17 @@ pic_status cuda_err(cudaError_t e) {
 
 double tval(const pic_ctx* c, double steps) { return c->t0 + steps * c->cfg.dt; }
 
+// blocks of the collision adjoint: its warps share the forward kernel's
+// overlay, so there are no more of them
+int adj_dsmc_grid(const pic_ctx* c) {
+  const int g = (int)((int64_t)c->dsmc_grid * (c->dsmc_block / 32) / (kAdjDsmcThreads / 32));
+  return g < 1 ? 1 : g;
+}
+
 pic_status ensure_buffers(pic_ctx* c, int seg, int ncp) {
   AdjointBuffers* B = c->adj;
   const size_t np3 = 3 * (size_t)c->P.np, nc = (size_t)c->P.ncell;
-  const size_t lanes = (size_t)c->dsmc_grid * (c->dsmc_block / 32) * 32;
+  const size_t lanes = (size_t)adj_dsmc_grid(c) * kAdjDsmcThreads;
   if (B && B->seg >= seg && B->ncp >= ncp && B->np3 == np3) return PIC_OK;
   adjoint_free(c);
   B = new (std::nothrow) AdjointBuffers();
@@ -648,12 +655,13 @@ cudaError_t collide_adjoint(pic_ctx* c, uint32_t c0, const double* lam, double* 
   a.max_rec = B.max_rec;
   a.ngroups = c->dsmc_groups;
   a.flags = c->flags;
-  if (c->dsmc_smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_dsmc_adj, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)c->dsmc_smem);
+  const size_t smem = (size_t)(kAdjDsmcThreads / 32) * 32 * c->bm_words * 4;
+  if (smem > 48 * 1024) {
+    cudaError_t e =
+        cudaFuncSetAttribute((const void*)k_dsmc_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_dsmc_adj<<<c->dsmc_grid, kAdjDsmcThreads, c->dsmc_smem, c->stream>>>(a);
+  k_dsmc_adj<<<adj_dsmc_grid(c), kAdjDsmcThreads, smem, c->stream>>>(a);
   c->launches++;
   return cudaGetLastError();
 }

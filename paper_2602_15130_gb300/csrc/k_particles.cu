@@ -127,11 +127,34 @@ __global__ void __launch_bounds__(kThreads) k_store_dv(StoreDvArgs a) {
 // K-averaged NTC collisions. One warp serves a group of G consecutive cells;
 // lane l runs outcome (chunk Kc + l % Kc) of cell (l / Kc) of the group,
 // sequentially over its candidate pairs with in-place updates (Algorithm 1).
-// The lane's working velocities live in a private overlay slot in global
-// memory (L1-resident in practice), valid where the lane's bitmap in shared
-// memory has the particle's bit; untouched particles are read from v.
-// After __syncwarp the warp sums each particle's per-outcome changes in
-// ascending outcome order and divides by K.
+// Then the lanes take the cells' particles: each adds its particle's changes
+// in ascending outcome order and forms the analytic source.
+//
+// What bounds it is the FP64 pipe (two lanes an SM and clock), so as little
+// as possible runs there, and that by full warps:
+//  - the accept test runs in FP32 on a copy of the group's velocities in
+//    shared memory, with a bound on its error; the one candidate in a
+//    million it cannot decide is decided in FP64 as the paper writes it
+//    (ntc_decide64), so every decision is the FP64 one;
+//  - one candidate in eight is accepted: the lanes only test their
+//    candidates and put the accepted pairs into a queue of the warp, which is
+//    scattered 32 pairs at a time, whichever lanes they came from. A
+//    candidate whose p or q is changed by a queued pair of its lane waits;
+//  - the source's R(a) comes from a table of degree-7 polynomials in a^2
+//    (hs_R64) instead of an exponential, an error function, a square root
+//    and a division.
+// Before, with the test and the source in FP64 and each lane scattering its
+// own pairs, the FP64 pipe was 85% busy; a call now takes 0.36 ms instead of
+// 1.36 (32^3 cells of 32, K = 16; 168 FP64 instructions per 32 particles,
+// the pipe 95% busy), 0.53 instead of 2.97 (12^3 cells of 101, K = 243) and
+// 98 us instead of 158 (8^3 cells of 8, K = 16: latency of the few warps).
+//
+// Working velocities: bit l of mask[p] says that lane l has changed particle
+// p of its cell. The first kList changed particles of a lane keep their
+// velocity in a list in shared memory, any further ones in the lane's
+// particle-indexed overlay in global memory. One word per lane holds the low
+// bytes of its list's indices (0xff: unused), so that in cells of up to 255
+// particles an entry is found by one zero-byte search.
 // --------------------------------------------------------------------------
 struct DsmcArgs {
   Params P;
@@ -141,8 +164,14 @@ struct DsmcArgs {
   double *dv0, *dv1, *dv2;  // out: <dv> - <dv^M>, or <dv> when m0 != nullptr
   double *m0, *m1, *m2;     // out (optional): <dv^M>
   double* overlay;
-  int max_ppc, bm_words, G, Kc, nchunks;
+  int max_ppc, G, Kc, nchunks;
+  int stage;                // particles of a group whose velocities are staged
   int64_t ngroups;
+  // parts > 1: a group's chunks of outcomes are shared by that many warps,
+  // which leave their sums in partial ([parts][3][N_p]) for k_dsmc_merge
+  int parts;
+  double* partial;
+  unsigned long long* queue;  // next (group, part) to take (zero at launch), or nullptr: a grid stride
   unsigned long long* counters;
   int* flags;
   double vh[3];             // PIC_DIST_PAPER: f_v scales at the call's time
@@ -150,26 +179,401 @@ struct DsmcArgs {
   long long* hist;          // per-step history row: [1] candidates, [2] collisions, [3] g > g_max
 };
 
-constexpr int kDsmcThreads = 128;
+// one warp a block: a launch of few groups still reaches every SM
+constexpr int kDsmcThreads = 32;
+constexpr int kList = 4;
+constexpr int kOverlay = 7;     // slot number of a particle in the overlay
+constexpr int kByteCell = 255;  // largest cell the byte keys are exact for
+// accepted pairs queued before they are scattered: a pass takes 32, and a
+// candidate adds at most 32 to a queue of 31
+constexpr int kQueue = 64;
+
+struct ListEntry {
+  double v[3];
+  long long p;
+};
+// A warp's shared memory; behind it the FP32 velocities [stage] and the
+// masks [max_ppc].
+struct Warp64 {
+  ListEntry list[kList * 32];  // entry k of lane l at 32 k + l
+  // p | q << 16; lane | slots of p and q << 8, 16 | kOld*; epsilon word; chi
+  // word, or candidate + 1 with kChiSlot
+  uint4 queue[kQueue];
+  uint32_t keys[32];
+  int len[32];
+};
+// of a queue entry: the slot of p or q held its velocity before; its chi word
+// is still to be drawn
+constexpr uint32_t kOldP = 1u << 24, kOldQ = 1u << 25, kChiSlot = 1u << 26;
+
+struct Counts64 {
+  uint32_t cand, coll, gmax, tie;  // per lane, flushed before they can overflow
+};
+constexpr uint32_t kFlushAt = 1u << 30;  // an outcome adds less than 2^31
+
+__device__ __forceinline__ int key_find(uint32_t keys, int p) {
+  const uint32_t x = keys ^ (((uint32_t)p & 0xffu) * 0x01010101u);
+  const uint32_t z = (x - 0x01010101u) & ~x & 0x80808080u;
+  return z ? (__ffs((int)z) - 8) >> 3 : -1;
+}
+__device__ __forceinline__ int list_find(const ListEntry* wl, int t, int p) {
+  int k = -1;
+#pragma unroll
+  for (int i = 0; i < kList; ++i)
+    if (i < t && wl[32 * i].p == p) k = i;
+  return k;
+}
+
+// The accept decision of one candidate in FP64, as the paper writes it
+// (U < sigma(g) g / (sigma g)_max), with the near-tie and g > g_max flags.
+__device__ __noinline__ int ntc_decide64(const Params& P, uint32_t w, double dx, double dy, double dz) {
+  const double g2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+  const double g = __dsqrt_rn(g2);
+  const double ratio = P.n_sigma == 0 ? __ddiv_rn(__dmul_rn(P.sigma0, g), P.sg_max)
+                                      : __ddiv_rn(sigma_g(P, g2), P.sg_max);
+  const double U = unif32(w);
+  return (U < ratio ? 1 : 0) | (fabs(U - ratio) < 1e-12 ? 2 : 0) | (g > P.gmax ? 4 : 0);
+}
+
+// FP32 constants of the test
+struct Test32 {
+  float gmax, gmax2, sgmax, s0, s1, s2;
+  float tie;  // what a near tie (1e-12 in U) amounts to where U is below 1e-6
+  int n_sigma;
+};
+
+// The same decision from FP32 velocities (each the FP64 one rounded): 0 or
+// 1, or -1 where FP64 has to decide. With S = sum (v_p^2 + v_q^2) the
+// components' differences are off by at most 2^-23 (|v_p| + |v_q|), g^2 by
+// less than 2^-20 S, and the squared threshold by less than 2^-20 of itself;
+// the margin is twice both. g^2 near or above g_max^2 is left to FP64 too
+// (its flag), and so is anything not finite (no comparison with it holds).
+// Odd-power sigma: the same through its derivative.
+__device__ __forceinline__ int ntc_test32(const Test32& T, uint32_t w, const float4& a, const float4& b) {
+  const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
+  const float g2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+  const float S = a.w + b.w;  // |v_p|^2 + |v_q|^2
+  const float U = fmaf((float)w, 0x1p-32f, 0x1p-33f);
+  const float e2 = fmaf(0x1p-19f, S, T.tie);
+  float lhs, rhs, margin;
+  if (T.n_sigma == 0) {
+    const float ug = U * T.gmax;
+    lhs = ug * ug;
+    rhs = g2;
+    margin = fmaf(0x1p-19f, lhs, e2);
+  } else {
+    lhs = U * T.sgmax;
+    rhs = fmaf(fmaf(T.s2, g2, T.s1), g2, T.s0);
+    const float d = fmaf(2.f * fabsf(T.s2), g2 + e2, fabsf(T.s1));
+    margin = fmaf(d, e2, fmaf(0x1p-19f, lhs + fabsf(T.s0) + g2 * d, T.tie));
+  }
+  if (fabsf(lhs - rhs) > margin && g2 + e2 < T.gmax2) return lhs < rhs ? 1 : 0;
+  return -1;
+}
+
+// R(a) of hs_R at u = a^2: polynomials of degree 7 on intervals of 1/8 up to
+// kR64Max (interpolation error below 1e-17), the closed form beyond.
+__device__ __forceinline__ double hs_R64(const Params& P, double u) {
+  if (!(u < (double)kR64Max)) return hs_R(P, sqrt(u));
+  const double t = u * (double)kR64PerUnit;
+  const double r = floor_small(t);
+  const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1)) + 4 * (int)r;
+  const double x = t - r - 0.5;
+  const double2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
+  return fma(fma(fma(fma(fma(fma(fma(q3.y, x, q3.x), x, q2.y), x, q2.x), x, q1.y), x, q1.x), x, q0.y), x, q0.x);
+}
+
+// Algorithm 1 for the warp's (cell, outcome) lanes: outcome o of cell `cell`
+// (particles off .. off + c - 1) where run is set.
+template <bool kVerify>
+__device__ __forceinline__ void ntc_warp64(const DsmcArgs& a, const Test32& T, uint32_t cell, uint32_t o, int off,
+                                           int c, bool run, int lane, Warp64& W, const float4* stage, int gs,
+                                           uint32_t* mask, double* wov, Counts64& cnt) {
+  const Params& P = a.P;
+  const DLog& lg = a.lg;
+  const uint32_t c0 = a.c0;
+  const bool log_all = kVerify && lg.mode == PIC_DLOG_ALL;
+  long long npairs = 0;
+  U4 bchi{0u, 0u, 0u, 0u}, b0{0u, 0u, 0u, 0u};
+  if (run) {
+    // the chi stream (c0, cell, slot, (o << 8) | 1): word 0 of slot 0 is the
+    // N_pairs uniform, word (s + 1) mod 4 of slot (s + 1) / 4 the chi of
+    // candidate s
+    bchi = philox(c0, cell, 0u, (o << 8) | 1u, P.key0, P.key1);
+    const double base = __dmul_rn(__dmul_rn((double)((long long)c * (long long)(c - 1)), P.pmax), 0.5);
+    npairs = (long long)floor(__dadd_rn(base, unif32(bchi.x)));
+    if (log_all) dlog_put(lg, c0, cell, o, -1, -1, -1, (int)npairs, PIC_DLOG_NPAIRS);
+    if (npairs > 0) {
+      // candidate s: block (c0, cell, s, o << 8) = (p, q, accept, epsilon)
+      b0 = philox(c0, cell, 0u, o << 8, P.key0, P.key1);
+      if (npairs > 0x7fffffffll) npairs = 0x7fffffffll;
+      cnt.cand += (uint32_t)npairs;
+    } else {
+      npairs = 0;
+    }
+  }
+  const uint32_t bit = 1u << lane;
+  double* const ov = wov + (size_t)lane * a.max_ppc * 3;
+  uint32_t keys = 0xffffffffu;   // low bytes of the list's indices
+  int t = 0;                     // list entries
+  bool spilled = false;          // some particle is in the overlay
+  uint32_t waiting = 0u;         // bit k + 1: a queued pair will write slot k
+  int s = 0, qn = 0;
+  bool stuck = false;
+  const int np = (int)npairs;
+  // slot of particle x of this lane, or -1
+  auto find = [&](int x) {
+    int k = key_find(keys, x);
+    if (c > kByteCell && k >= 0 && !(k < t && W.list[32 * k + lane].p == x)) k = list_find(W.list + lane, t, x);
+    if (spilled && k < 0 && (mask[x] & bit)) k = kOverlay;
+    return k;
+  };
+  // a slot for a particle that has none
+  auto new_slot = [&](int x) {
+    atomicOr(mask + x, bit);
+    if (t == kList) {
+      spilled = true;
+      return kOverlay;
+    }
+    keys ^= (~(uint32_t)x & 0xffu) << (8 * t);
+    W.list[32 * t + lane].p = x;
+    return t++;
+  };
+  // working velocity of particle x in slot k (-1: none) of lane l, whose
+  // cell's first particle is `at`
+  auto velocity = [&](int x, int k, int l, int at, double* v) {
+    if (k < 0) {
+      v[0] = a.v0[at + x]; v[1] = a.v1[at + x]; v[2] = a.v2[at + x];
+    } else {
+      const double* e = k < kList ? W.list[32 * k + l].v : wov + ((size_t)l * a.max_ppc + x) * 3;
+      v[0] = e[0]; v[1] = e[1]; v[2] = e[2];
+    }
+  };
+  auto rounded = [](const double* v) {
+    float4 f = make_float4((float)v[0], (float)v[1], (float)v[2], 0.f);
+    f.w = fmaf(f.x, f.x, fmaf(f.y, f.y, f.z * f.z));
+    return f;
+  };
+  for (;;) {
+    const bool go = s < np && !stuck;
+    const int able = __popc(__ballot_sync(0xffffffffu, go));
+    if (able <= 4 * __popc(__ballot_sync(0xffffffffu, stuck)) || qn >= 32) {
+      if (qn == 0) break;  // no lane is stuck without a queued pair
+      // scatter the queue
+      __syncwarp();
+      for (int e0 = 0; e0 < qn; e0 += 32) {
+        const int e = e0 + lane;
+        uint4 ec = make_uint4(0u, 0u, 0u, 0u);
+        if (e < qn) ec = W.queue[e];
+        const int owner = (int)(ec.y & 31u);
+        // the owner's cell, outcome and first particle
+        const uint32_t ocell = __shfl_sync(0xffffffffu, cell, owner), oo = __shfl_sync(0xffffffffu, o, owner);
+        const int ooff = __shfl_sync(0xffffffffu, off, owner);
+        if (e < qn) {
+          const int p = (int)(ec.x & 0xffffu), q = (int)(ec.x >> 16);
+          const int kp = (int)((ec.y >> 8) & 15u), kq = (int)((ec.y >> 16) & 15u);
+          double vp[3], vq[3];
+          velocity(p, ec.y & kOldP ? kp : -1, owner, ooff, vp);
+          velocity(q, ec.y & kOldQ ? kq : -1, owner, ooff, vq);
+          uint32_t wchi = ec.w;
+          if (ec.y & kChiSlot) {
+            const U4 b = philox(c0, ocell, ec.w >> 2, (oo << 8) | 1u, P.key0, P.key1);
+            const uint32_t js = ec.w & 3u;
+            wchi = js == 0u ? b.x : js == 1u ? b.y : js == 2u ? b.z : b.w;
+          }
+          const double dx = __dsub_rn(vp[0], vq[0]), dy = __dsub_rn(vp[1], vq[1]), dz = __dsub_rn(vp[2], vq[2]);
+          const double g =
+              __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
+          double* wp = kp < kList ? W.list[32 * kp + owner].v : wov + ((size_t)owner * a.max_ppc + p) * 3;
+          double* wq = kq < kList ? W.list[32 * kq + owner].v : wov + ((size_t)owner * a.max_ppc + q) * 3;
+          if (kVerify && (P.verify & PIC_VERIFY_ERROR2)) {
+            // injected Error 2: swap with probability 1/2 (coin = chi draw)
+            const bool swap = unif32(wchi) < 0.5;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              wp[d] = swap ? vq[d] : vp[d];
+              wq[d] = swap ? vp[d] : vq[d];
+            }
+          } else {
+            double se, ce;
+            sincospi(2.0 * unif32(ec.z), &se, &ce);
+            double uchi = unif32(wchi);
+            if (kVerify && (P.verify & PIC_VERIFY_ANISO)) uchi = aniso_u(uchi);
+            const double cchi = __dsub_rn(1.0, __dmul_rn(2.0, uchi));
+            const double schi = __dsqrt_rn(__dsub_rn(1.0, __dmul_rn(cchi, cchi)));
+            const double nv[3] = {__dmul_rn(ce, schi), __dmul_rn(se, schi), cchi};
+            const bool err1 = kVerify && (P.verify & PIC_VERIFY_ERROR1);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              const double gp = __dmul_rn(g, nv[d]);
+              // Eq. v_cm; injected Error 1 flips the sign of v_q
+              const double cm = __dmul_rn(err1 ? __dsub_rn(vp[d], vq[d]) : __dadd_rn(vp[d], vq[d]), 0.5);
+              wp[d] = fma(gp, 0.5, cm);
+              wq[d] = fma(gp, -0.5, cm);
+            }
+          }
+          if (kVerify && P.ang_hist)
+            record_angles(P.ang_hist, (P.verify & PIC_VERIFY_ANISO) != 0, g, __dsub_rn(wp[0], wq[0]),
+                          __dsub_rn(wp[1], wq[1]), __dsub_rn(wp[2], wq[2]));
+        }
+      }
+      __syncwarp();
+      qn = 0;
+      waiting = 0u;
+      stuck = false;
+      continue;
+    }
+    bool accept = false;
+    uint32_t p = 0u, q = 0u, ww = 0u;
+    int kp = -1, kq = -1;
+    if (go) {
+      p = draw_index(b0.x, (uint32_t)c);
+      // q uniform over the other c - 1 particles: the distribution of
+      // drawing again until q != p
+      q = draw_index(b0.y, (uint32_t)(c - 1));
+      q += q >= p ? 1u : 0u;
+      kp = find((int)p);
+      kq = find((int)q);
+      stuck = ((waiting >> (kp + 1) | waiting >> (kq + 1)) & 1u) != 0u;
+      if (!stuck) {
+        const uint32_t wz = b0.z;
+        ww = b0.w;
+        ++s;
+        if (s < np) b0 = philox(c0, cell, (uint32_t)s, o << 8, P.key0, P.key1);
+        int d = -1;
+        if (stage && kp < 0 && kq < 0) {
+          d = ntc_test32(T, wz, stage[off - gs + (int)p], stage[off - gs + (int)q]);
+        } else {
+          double vp[3], vq[3];
+          velocity((int)p, kp, lane, off, vp);
+          velocity((int)q, kq, lane, off, vq);
+          d = ntc_test32(T, wz, rounded(vp), rounded(vq));
+        }
+        if (d < 0) {
+          double vp[3], vq[3];
+          velocity((int)p, kp, lane, off, vp);
+          velocity((int)q, kq, lane, off, vq);
+          d = ntc_decide64(P, wz, __dsub_rn(vp[0], vq[0]), __dsub_rn(vp[1], vq[1]), __dsub_rn(vp[2], vq[2]));
+        }
+        if (d & 4) ++cnt.gmax;
+        if (d & 2) ++cnt.tie;
+        accept = (d & 1) != 0;
+        if (log_all || ((d & 2) && lg.mode != PIC_DLOG_OFF))
+          dlog_put(lg, c0, cell, o, s - 1, (int)p, (int)q, accept ? 1 : 0, d & 2 ? PIC_DLOG_TIE : 0);
+      }
+    }
+    const unsigned acc = __ballot_sync(0xffffffffu, accept);
+    if (accept) {
+      uint32_t info = (uint32_t)lane | (kp >= 0 ? kOldP : 0u) | (kq >= 0 ? kOldQ : 0u) | (s > 3 ? kChiSlot : 0u);
+      if (kp < 0) kp = new_slot((int)p);
+      if (kq < 0) kq = new_slot((int)q);
+      waiting |= 2u << kp | 2u << kq;
+      info |= (uint32_t)kp << 8 | (uint32_t)kq << 16;
+      const uint32_t wchi = s == 1 ? bchi.y : s == 2 ? bchi.z : s == 3 ? bchi.w : (uint32_t)s;
+      W.queue[qn + __popc(acc & (bit - 1u))] = make_uint4(p | q << 16, info, ww, wchi);
+      ++cnt.coll;
+    }
+    qn += __popc(acc);
+  }
+  W.keys[lane] = keys;
+  W.len[lane] = t;
+  __syncwarp();
+}
+
+// the warp's counts into the launch's totals
+__device__ __forceinline__ void flush_counts(const DsmcArgs& a, Counts64& cnt, int lane) {
+  const uint32_t v[4] = {cnt.cand, cnt.coll, cnt.gmax, cnt.tie};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const unsigned long long lo = __reduce_add_sync(0xffffffffu, v[k] & 0xffffu);
+    const unsigned long long hi = __reduce_add_sync(0xffffffffu, v[k] >> 16);
+    const unsigned long long tot = lo + (hi << 16);
+    if (lane == 0 && tot) {
+      atomicAdd(a.counters + k, tot);
+      if (a.hist && k < 3) atomicAdd((unsigned long long*)a.hist + 1 + k, tot);
+    }
+  }
+  cnt = {0u, 0u, 0u, 0u};
+}
+
+// the outputs of particle j (velocity w) of a cell of cc, from the sum of its
+// changes over the outcomes
+__device__ __forceinline__ void dsmc_finish(const DsmcArgs& a, int64_t j, int cc, const double* w, const double* acc,
+                                            double invK) {
+  const Params& P = a.P;
+  double so[3];
+  if (P.n_sigma == 0) {
+    // Eq. vel_change_1c
+    const double mx = P.vmean[0] - w[0], my = P.vmean[1] - w[1], mz = P.vmean[2] - w[2];
+    const double u = fma(mx, mx, fma(my, my, mz * mz)) * (P.inv_vsig * P.inv_vsig);
+    const double f = P.src_pref * (double)(cc - 1) * P.vsig * hs_R64(P, u);
+    so[0] = f * mx; so[1] = f * my; so[2] = f * mz;
+  } else {
+    odd_source(P, a.vh, w[0], w[1], w[2], cc, so);
+  }
+  if (a.m0) {
+    a.dv0[j] = acc[0] * invK; a.dv1[j] = acc[1] * invK; a.dv2[j] = acc[2] * invK;
+    a.m0[j] = so[0]; a.m1[j] = so[1]; a.m2[j] = so[2];
+  } else {
+    a.dv0[j] = fma(acc[0], invK, -so[0]);
+    a.dv1[j] = fma(acc[1], invK, -so[1]);
+    a.dv2[j] = fma(acc[2], invK, -so[2]);
+  }
+}
+
+// the parts' sums, in order, and the source: one warp a cell
+constexpr int kMergeThreads = 128;
+__global__ void __launch_bounds__(kMergeThreads) k_dsmc_merge(DsmcArgs a) {
+  const int lane = threadIdx.x & 31;
+  const int64_t cell = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (cell >= a.P.ncell) return;
+  const int32_t s = a.start[cell], e = a.start[cell + 1];
+  const double invK = 1.0 / (double)a.P.K;
+  for (int32_t j = s + lane; j < e; j += 32) {
+    double acc[3] = {0.0, 0.0, 0.0};
+    for (int k = 0; k < a.parts; ++k)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) acc[d] += a.partial[((int64_t)3 * k + d) * a.P.np + j];
+    const double w[3] = {a.v0[j], a.v1[j], a.v2[j]};
+    dsmc_finish(a, j, e - s, w, acc, invK);
+  }
+}
 
 template <bool kVerify>
-__global__ void __launch_bounds__(kDsmcThreads) k_dsmc(DsmcArgs a) {
-  extern __shared__ uint32_t smem[];
+__global__ void __launch_bounds__(kDsmcThreads, 16) k_dsmc(DsmcArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
   const Params& P = a.P;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int wpb = blockDim.x >> 5;
-  const int64_t gwarp = (int64_t)blockIdx.x * wpb + wib;
-  const int64_t nwarps = (int64_t)gridDim.x * wpb;
-  uint32_t* wbm = smem + (size_t)wib * 32 * a.bm_words;     // warp's 32 bitmaps
-  uint32_t* bm = wbm + (size_t)lane * a.bm_words;            // this lane's
-  double* wov = a.overlay + (size_t)gwarp * 32 * a.max_ppc * 3;
-  double* ov = wov + (size_t)lane * a.max_ppc * 3;
-  for (int i = 0; i < a.bm_words; ++i) bm[i] = 0u;
+  const int lane = threadIdx.x;
+  Warp64& W = *reinterpret_cast<Warp64*>(smem);
+  float4* const staged = reinterpret_cast<float4*>(&W + 1);
+  uint32_t* const mask = reinterpret_cast<uint32_t*>(staged + a.stage);
+  double* wov = a.overlay + (size_t)blockIdx.x * 32 * a.max_ppc * 3;
+  for (int i = lane; i < a.max_ppc; i += 32) mask[i] = 0u;
   __syncwarp();
-  LaneCounts cnt = {0, 0, 0, 0};
-  const bool separate = a.m0 != nullptr;
+  Counts64 cnt = {0u, 0u, 0u, 0u};
+  const double invK = 1.0 / (double)P.K;
+  const Test32 T = {(float)P.gmax, (float)(P.gmax * P.gmax), (float)P.sg_max, (float)P.sigma_n[0],
+                    (float)P.sigma_n[1], (float)P.sigma_n[2],
+                    P.n_sigma == 0 ? (float)(2e-18 * P.gmax * P.gmax) : (float)(2e-12 * P.sg_max), P.n_sigma};
 
-  for (int64_t grp = gwarp; grp < a.ngroups; grp += nwarps) {
+  for (int64_t take = blockIdx.x;; take += gridDim.x) {
+    int64_t item = take;
+    if (a.queue) {
+      unsigned long long q = 0;
+      if (lane == 0) q = atomicAdd(a.queue, 1ull);
+      item = (int64_t)__shfl_sync(0xffffffffu, q, 0);
+    }
+    if (item >= a.ngroups * a.parts) break;  // warp-uniform
+    const int64_t grp = item / a.parts;
+    const int part = (int)(item % a.parts);
+    const int ch0 = (int)((int64_t)a.nchunks * part / a.parts), ch1 = (int)((int64_t)a.nchunks * (part + 1) / a.parts);
+    // where the sums over the part's outcomes are kept
+    double *d0 = a.dv0, *d1 = a.dv1, *d2 = a.dv2;
+    if (a.parts > 1) {
+      d0 = a.partial + (int64_t)3 * part * P.np;
+      d1 = d0 + P.np;
+      d2 = d1 + P.np;
+    }
     const int64_t cell0 = grp * a.G;
     const int ncl = (int)min((int64_t)a.G, P.ncell - cell0);  // cells in this group
     const int mycl = lane / a.Kc;
@@ -179,90 +583,67 @@ __global__ void __launch_bounds__(kDsmcThreads) k_dsmc(DsmcArgs a) {
       s = a.start[cell0 + mycl];
       c = a.start[cell0 + mycl + 1] - s;
     }
-    const int32_t gs = a.start[cell0], ge = a.start[cell0 + ncl];
-    for (int ch = 0; ch < a.nchunks; ++ch) {
+    const int cmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)c);
+    const int32_t gs = a.start[cell0], gn = a.start[cell0 + ncl] - gs;
+    const bool use_stage = gn <= a.stage;
+    __syncwarp();
+    if (use_stage)
+      for (int i = lane; i < gn; i += 32) {
+        const float x = (float)a.v0[gs + i], y = (float)a.v1[gs + i], z = (float)a.v2[gs + i];
+        staged[i] = make_float4(x, y, z, fmaf(x, x, fmaf(y, y, z * z)));
+      }
+    __syncwarp();
+    for (int ch = ch0; ch < ch1; ++ch) {
       const int o = ch * a.Kc + lane % a.Kc;
       bool run = lane_cell && o < P.K && c >= 2;
       if (run && c > a.max_ppc) {
         atomicOr(a.flags, 1);
         run = false;
       }
-      if (run)
-      {
-        NoRecord none;
-        ntc_outcome<kVerify>(P, a.c0, (uint32_t)(cell0 + mycl), (uint32_t)o, c, a.v0 + s, a.v1 + s, a.v2 + s,
-                             bm, ov, cnt, none, a.lg);
-      }
-      __syncwarp();
+      ntc_warp64<kVerify>(a, T, (uint32_t)(cell0 + mycl), (uint32_t)o, s, c, run, lane, W,
+                          use_stage ? staged : nullptr, gs, mask, wov, cnt);
       // sum this chunk's changes per particle in ascending outcome order
-      const bool last = ch == a.nchunks - 1;
-      for (int32_t j = gs + lane; j < ge; j += 32) {
-        int cl = 0;
-        while (cl + 1 < ncl && a.start[cell0 + cl + 1] <= j) ++cl;
-        const int32_t cs = a.start[cell0 + cl];
-        const int cc = a.start[cell0 + cl + 1] - cs;
-        const int jj = j - cs;
-        double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0;
-        if (ch > 0) { acc0 = a.dv0[j]; acc1 = a.dv1[j]; acc2 = a.dv2[j]; }
-        if (cc >= 2 && cc <= a.max_ppc) {
-          const double w0 = a.v0[j], w1 = a.v1[j], w2 = a.v2[j];
-          for (int k = 0; k < a.Kc; ++k) {
-            if (ch * a.Kc + k >= P.K) break;
-            const int L = cl * a.Kc + k;
-            if ((wbm[(size_t)L * a.bm_words + (jj >> 5)] >> (jj & 31)) & 1u) {
-              const double* W = wov + ((size_t)L * a.max_ppc + jj) * 3;
-              acc0 = __dadd_rn(acc0, __dsub_rn(W[0], w0));
-              acc1 = __dadd_rn(acc1, __dsub_rn(W[1], w1));
-              acc2 = __dadd_rn(acc2, __dsub_rn(W[2], w2));
-            }
-          }
+      const bool last = ch == a.nchunks - 1 && a.parts == 1;
+      const uint32_t kseg = a.Kc == 32 ? 0xffffffffu : ((1u << a.Kc) - 1u);
+      for (int jb = 0; jb < cmax; jb += 32) {
+        const int jj = jb + lane;
+        // cells above max_ppc have no masks (and no collisions)
+        uint32_t word = 0u;
+        if (jj < a.max_ppc) {
+          word = mask[jj];
+          mask[jj] = 0u;
         }
-        if (!last) {
-          a.dv0[j] = acc0; a.dv1[j] = acc1; a.dv2[j] = acc2;
-        } else {
-          const double K = (double)P.K;
-          const double m0 = acc0 != 0.0 ? acc0 / K : 0.0, m1 = acc1 != 0.0 ? acc1 / K : 0.0,
-                       m2 = acc2 != 0.0 ? acc2 / K : 0.0;
-          double s0, s1, s2;
-          if (P.n_sigma == 0) {
-            hs_source(P, a.v0[j], a.v1[j], a.v2[j], cc, &s0, &s1, &s2);
-          } else {
-            double so[3];
-            odd_source(P, a.vh, a.v0[j], a.v1[j], a.v2[j], cc, so);
-            s0 = so[0]; s1 = so[1]; s2 = so[2];
+        for (int cl = 0; cl < ncl; ++cl) {
+          const int32_t cs = __shfl_sync(0xffffffffu, s, cl * a.Kc);
+          const int cc = __shfl_sync(0xffffffffu, c, cl * a.Kc);
+          if (jj >= cc) continue;
+          uint32_t mine = word & (kseg << (cl * a.Kc));
+          if (!last && ch > ch0 && !mine) continue;  // nothing to add
+          const int32_t j = cs + jj;
+          const double w[3] = {a.v0[j], a.v1[j], a.v2[j]};
+          double acc[3] = {0.0, 0.0, 0.0};
+          if (ch > ch0) { acc[0] = d0[j]; acc[1] = d1[j]; acc[2] = d2[j]; }
+          while (mine) {
+            const int l = __ffs((int)mine) - 1;
+            mine &= mine - 1u;
+            // lane l's working velocity of particle jj: its list, else its overlay
+            const int k = cc <= kByteCell ? key_find(W.keys[l], jj) : list_find(W.list + l, W.len[l], jj);
+            const double* e = k >= 0 ? W.list[32 * k + l].v : wov + ((size_t)l * a.max_ppc + jj) * 3;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) acc[d] = __dadd_rn(acc[d], __dsub_rn(e[d], w[d]));
           }
-          if (separate) {
-            a.dv0[j] = m0; a.dv1[j] = m1; a.dv2[j] = m2;
-            a.m0[j] = s0; a.m1[j] = s1; a.m2[j] = s2;
+          if (last) {
+            dsmc_finish(a, j, cc, w, acc, invK);
           } else {
-            a.dv0[j] = m0 - s0; a.dv1[j] = m1 - s1; a.dv2[j] = m2 - s2;
+            d0[j] = acc[0]; d1[j] = acc[1]; d2[j] = acc[2];
           }
         }
       }
       __syncwarp();
-      if (run)
-        for (int i = 0; i < (c + 31) / 32; ++i) bm[i] = 0u;
-      __syncwarp();
+      if (__any_sync(0xffffffffu, cnt.cand >= kFlushAt)) flush_counts(a, cnt, lane);
     }
   }
-  // warp totals, one atomic per counter per warp
-  for (int off = 16; off > 0; off >>= 1) {
-    cnt.cand += __shfl_down_sync(0xffffffffu, cnt.cand, off);
-    cnt.coll += __shfl_down_sync(0xffffffffu, cnt.coll, off);
-    cnt.gmax += __shfl_down_sync(0xffffffffu, cnt.gmax, off);
-    cnt.tie += __shfl_down_sync(0xffffffffu, cnt.tie, off);
-  }
-  if (lane == 0) {
-    if (cnt.cand) atomicAdd(a.counters + 0, cnt.cand);
-    if (cnt.coll) atomicAdd(a.counters + 1, cnt.coll);
-    if (cnt.gmax) atomicAdd(a.counters + 2, cnt.gmax);
-    if (cnt.tie) atomicAdd(a.counters + 3, cnt.tie);
-    if (a.hist) {
-      if (cnt.cand) atomicAdd((unsigned long long*)a.hist + 1, cnt.cand);
-      if (cnt.coll) atomicAdd((unsigned long long*)a.hist + 2, cnt.coll);
-      if (cnt.gmax) atomicAdd((unsigned long long*)a.hist + 3, cnt.gmax);
-    }
-  }
+  flush_counts(a, cnt, lane);
 }
 
 // --------------------------------------------------------------------------
@@ -570,26 +951,41 @@ cudaError_t launch_dsmc(pic_ctx* c, uint32_t c0, bool separate, double t_src) {
   else { a.m0 = a.m1 = a.m2 = nullptr; }
   a.overlay = c->overlay;
   a.max_ppc = c->cfg.max_ppc;
-  a.bm_words = c->bm_words;
   a.G = c->dsmc_G;
   a.Kc = c->dsmc_Kc;
   a.nchunks = (c->P.K + c->dsmc_Kc - 1) / c->dsmc_Kc;
+  a.stage = c->dsmc_stage;
   a.ngroups = c->dsmc_groups;
+  a.parts = c->dsmc_parts;
+  a.partial = c->dsmc_partial;
+  // more work than warps: taken from a queue, since a cell's work varies
+  a.queue = a.ngroups * a.parts > c->dsmc_grid ? c->dsmc_queue : nullptr;
   a.counters = c->counters;
   a.flags = c->flags;
   a.lg = DLog{c->dlog, c->dlog_n, (long long)c->dlog_cap, c->dlog ? c->dlog_mode : 0};
   a.hist = c->hist_row;
   prof_begin(c);
+  if (a.queue) {
+    const cudaError_t eq = cudaMemsetAsync(c->dsmc_queue, 0, 8, c->stream);
+    if (eq != cudaSuccess) return eq;
+  }
   if (c->P.verify || a.lg.mode == PIC_DLOG_ALL)
     k_dsmc<true><<<c->dsmc_grid, kDsmcThreads, c->dsmc_smem, c->stream>>>(a);
   else
     k_dsmc<false><<<c->dsmc_grid, kDsmcThreads, c->dsmc_smem, c->stream>>>(a);
+  if (a.parts > 1) {
+    k_dsmc_merge<<<blocks_for(32 * c->P.ncell, kMergeThreads), kMergeThreads, 0, c->stream>>>(a);
+    c->launches++;
+  }
   prof_end(c, KC_DSMC);
   c->launches++;
   return cudaGetLastError();
 }
 
 int dsmc_threads() { return kDsmcThreads; }
+size_t dsmc_smem_bytes(int max_ppc, int stage) {
+  return sizeof(Warp64) + (size_t)stage * sizeof(float4) + (size_t)max_ppc * 4;
+}
 const void* dsmc_kernel_ptr(bool verify) {
   return verify ? (const void*)k_dsmc<true> : (const void*)k_dsmc<false>;
 }

@@ -7,12 +7,14 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <memory>
 #include <new>
 
 #include "pic_internal.cuh"
 
 namespace pic {
 int dsmc_threads();
+size_t dsmc_smem_bytes(int max_ppc, int stage);
 const void* dsmc_kernel_ptr(bool verify);
 int cg_blocks(int64_t m, int sms);
 size_t cg_slot_bytes(int grid);
@@ -93,6 +95,8 @@ using namespace pic;
 namespace {
 
 constexpr int kGinvM = 1024;
+constexpr int kDsmcStageMax = 1024;
+constexpr size_t kDsmcPartialBytes = size_t(1) << 29;
 
 // Knots of G^{-1}, G(y) = y - a cos(2 pi y), a = A/(2 pi), at T_k = k/M:
 // y_k by Newton in FP64 (converged to |dy| < 1e-16) and the slope
@@ -128,6 +132,52 @@ void hs_R_host(double a, const double* ser, double* R, double* dR) {
   const double s = sqrt(2.0 / kPi), e = exp(-0.5 * a * a), f = erf(a / sqrt(2.0));
   *R = s * (1.0 + 1.0 / (a * a)) * e + (a + 2.0 / a - 1.0 / (a * a * a)) * f;
   *dR = s * e * (1.0 / a - 3.0 / (a * a * a)) + (1.0 - 2.0 / (a * a) + 3.0 / (a * a * a * a)) * f;
+}
+
+// FP64 table of R(a) as a function of u = a^2 (hs_R64): on each interval the
+// polynomial of degree 7 in x = 8 u - k - 1/2 through its Chebyshev nodes,
+// from extended-precision values of the closed form (of the even series below
+// u = 1/4). R is entire in u, and the interpolation error is below 1e-17.
+void hs_R64_table(double* out) {
+  constexpr int kN = 8;
+  typedef long double real;
+  const real pi = 3.14159265358979323846264338327950288L;
+  auto R = [&](real u) -> real {
+    const real s = sqrtl(2.0L / pi);
+    if (u < 0.25L) {
+      // sum_j c_j u^j with c_j = d_j + d_{j+1} + e_{j-1} + 2 e_j - e_{j+1}
+      // (series_coefficients), d_k = (-1/2)^k / k!, e_k = d_k / (2 k + 1)
+      real d[26];
+      d[0] = 1.0L;
+      for (int k = 1; k < 26; ++k) d[k] = d[k - 1] * (-0.5L / k);
+      real acc = 0.0L;
+      for (int j = 24; j >= 0; --j) {
+        const real em = j > 0 ? d[j - 1] / (2 * j - 1) : 0.0L;
+        acc = acc * u + d[j] + d[j + 1] + em + 2.0L * d[j] / (2 * j + 1) - d[j + 1] / (2 * j + 3);
+      }
+      return s * acc;
+    }
+    const real a = sqrtl(u);
+    return s * (1.0L + 1.0L / u) * expl(-0.5L * u) + (a + 2.0L / a - 1.0L / (a * u)) * erfl(a / sqrtl(2.0L));
+  };
+  for (int k = 0; k < kR64Max * kR64PerUnit; ++k) {
+    // divided differences at the nodes x_i in [-1/2, 1/2], then monomials
+    real x[kN], f[kN];
+    for (int i = 0; i < kN; ++i) {
+      x[i] = 0.5L * cosl(pi * (2 * i + 1) / (2 * kN));
+      f[i] = R(((real)k + 0.5L + x[i]) / kR64PerUnit);
+    }
+    for (int j = 1; j < kN; ++j)
+      for (int i = kN - 1; i >= j; --i) f[i] = (f[i] - f[i - 1]) / (x[i] - x[i - j]);
+    real c[kN];
+    for (int i = 0; i < kN; ++i) c[i] = 0.0L;
+    c[0] = f[kN - 1];
+    for (int i = kN - 2; i >= 0; --i) {
+      for (int j = kN - 1; j > 0; --j) c[j] = c[j - 1] - x[i] * c[j];
+      c[0] = f[i] - x[i] * c[0];
+    }
+    for (int j = 0; j < kN; ++j) out[kN * k + j] = (double)c[j];
+  }
 }
 
 // FP32 tables of the precision form: the knots of G^{-1} (y_k, dy/dT) and
@@ -312,6 +362,7 @@ void for_each_buffer(pic_ctx* c, F f) {
     f((void**)&c->cg_p[1], nc * 8);
     f((void**)&c->cg_q, nc * 8);
     f((void**)&c->overlay, lanes * 8);
+    if (c->dsmc_parts > 1) f((void**)&c->dsmc_partial, (size_t)c->dsmc_parts * 3 * np * 8);
   } else {
     for (int b = 0; b < 2; ++b) {
       f((void**)&c->cell32[b], np * 4);
@@ -362,7 +413,7 @@ void for_each_buffer(pic_ctx* c, F f) {
   f((void**)&c->flags, 64);
   f((void**)&c->err_part, (size_t)c->err_blocks * 14 * 8);
   f((void**)&c->err_out, 14 * 8);
-  f((void**)&c->ginv, (size_t)(kGinvM + 1) * 2 * 8);
+  f((void**)&c->ginv, ((size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles)) * 8);
   f((void**)&c->ginv_f, (size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4);
   if (c->nrep == 0 && (c->cfg.verify & PIC_VERIFY_ANGLES)) {
     f((void**)&c->ang_hist, (size_t)2 * PIC_ANGLE_BINS * 8);
@@ -866,14 +917,35 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
   c->bm_words = c->cfg.max_ppc / 32;
   c->dsmc_block = c->mixed ? dsmc32_threads() : dsmc_threads();
   const void* dsmc_fn = c->mixed ? dsmc32_kernel_ptr(c->P.verify != 0) : dsmc_kernel_ptr(c->P.verify != 0);
-  c->dsmc_smem = c->mixed ? dsmc32_smem_bytes(c->bm_words) : (size_t)(c->dsmc_block / 32) * 32 * c->bm_words * 4;
+  if (c->mixed) {
+    c->dsmc_smem = dsmc32_smem_bytes(c->bm_words);
+  } else {
+    // the FP32 copy of a group's velocities: room for twice its mean; larger
+    // groups are tested from their FP64 velocities
+    const double want = 2.0 * (double)c->P.np / (double)c->P.ncell * c->dsmc_G + 64.0;
+    c->dsmc_stage = want < kDsmcStageMax ? ((int)want + 31) / 32 * 32 : kDsmcStageMax;
+    c->dsmc_smem = dsmc_smem_bytes(c->cfg.max_ppc, c->dsmc_stage);
+  }
+  // the logging and verification variant may be launched as well
   if (c->dsmc_smem > 48 * 1024) {
     e = cudaFuncSetAttribute(dsmc_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dsmc_smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(c->mixed ? dsmc32_kernel_ptr(true) : dsmc_kernel_ptr(true),
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dsmc_smem);
     if (e != cudaSuccess) {
       cudaGetLastError();
       delete c;
       return PIC_EINVAL;
     }
+  }
+  // max_ppc in the FP64 form: 16 bytes of it in a block's shared memory (the
+  // pathwise adjoint's bitmaps)
+  int optin = 0;
+  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+  if (e != cudaSuccess || (!c->mixed && (size_t)16 * c->cfg.max_ppc > (size_t)optin)) {
+    cudaGetLastError();
+    delete c;
+    return e != cudaSuccess ? PIC_ECUDA : PIC_EINVAL;
   }
   int docc = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&docc, dsmc_fn, c->dsmc_block, c->dsmc_smem);
@@ -883,7 +955,20 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     return PIC_ECUDA;
   }
   const int64_t wpb = c->dsmc_block / 32;
-  int64_t dgrid = (c->dsmc_groups + wpb - 1) / wpb;
+  c->dsmc_parts = 1;
+  if (!c->mixed) {
+    // a cell's work grows with the square of its particles, so the launch
+    // wants several items a warp: a group's chunks of outcomes are shared by
+    // parts until there are four (the 12^3 level of Table 1, 1,728 cells of
+    // 101 on 2,432 warps, K = 243: 0.96 ms a call by whole cells, 0.53 ms in
+    // five parts, of which the merge takes 10 us)
+    const int64_t nchunks = (K + c->dsmc_Kc - 1) / c->dsmc_Kc;
+    int64_t parts = 4 * (int64_t)docc * c->num_sms / c->dsmc_groups;
+    if (parts > nchunks) parts = nchunks;
+    while (parts > 1 && (size_t)parts * 24 * (size_t)c->P.np > kDsmcPartialBytes) --parts;
+    c->dsmc_parts = parts < 1 ? 1 : (int)parts;
+  }
+  int64_t dgrid = (c->dsmc_groups * c->dsmc_parts + wpb - 1) / wpb;
   if (dgrid > (int64_t)docc * c->num_sms) dgrid = (int64_t)docc * c->num_sms;
   c->dsmc_grid = (int)(dgrid < 1 ? 1 : dgrid);
   if (c->cfg.K == 0) c->dsmc_grid = 1;
@@ -899,7 +984,8 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     return PIC_ENOMEM;
   }
   {
-    double* tab = (double*)malloc((size_t)(kGinvM + 1) * 2 * 8);
+    const size_t tab_doubles = (size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles);
+    double* tab = (double*)malloc(tab_doubles * 8);
     float* tabf = (float*)malloc((size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4);
     if (!tab || !tabf) {
       free(tab);
@@ -909,7 +995,16 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     }
     ginv_table(c->cfg.fx_amp, tab);
     ginv_table_f(tab, tabf);
-    e = cudaMemcpy(c->ginv, tab, (size_t)(kGinvM + 1) * 2 * 8, cudaMemcpyHostToDevice);
+    if (!c->mixed) {
+      // the same for every context: formed once
+      static const std::unique_ptr<double[]> r64 = [] {
+        std::unique_ptr<double[]> t(new double[kR64Doubles]);
+        hs_R64_table(t.get());
+        return t;
+      }();
+      memcpy(tab + (kGinvM + 1) * 2, r64.get(), sizeof(double) * kR64Doubles);
+    }
+    e = cudaMemcpy(c->ginv, tab, tab_doubles * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->ginv_f, tabf, (size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4,
                                          cudaMemcpyHostToDevice);
     free(tab);

@@ -21,6 +21,10 @@ constexpr int kRTabM = 512;
 // steps of the per-step history (pic_get_step_history)
 constexpr int kHistSteps = 4096;
 constexpr float kRTabAmax = 8.f;
+// FP64 table of R at u = a^2 in [0, kR64Max): kR64PerUnit polynomials of
+// degree 7 a unit of u, behind the FP64 G^{-1} knots
+constexpr int kR64Max = 64, kR64PerUnit = 8;
+constexpr int kR64Doubles = 8 * kR64Max * kR64PerUnit;
 
 // ---------------------------------------------------------------------------
 // Everything a kernel needs to know about the problem, passed by value.
@@ -416,6 +420,13 @@ __device__ __forceinline__ void e_manufactured(const Params& P, const TimeTerms&
   *ez = -tt.em_amp * s0 * s1 * c2;
 }
 
+// floor of 0 <= t < 2^31 without a conversion instruction (FP64 conversions
+// run on the FP64 pipe, as an addition does)
+__device__ __forceinline__ double floor_small(double t) {
+  const double r = __dadd_rd(t, 0x1p52);
+  return __dsub_rn(r, 0x1p52);
+}
+
 // R(a): E_{X ~ N(m, s^2 I)} |X| X = s R(|m|/s) m (hard spheres, Gaussian f_v).
 __device__ __forceinline__ double hs_R(const Params& P, double a) {
   const double a2 = a * a;
@@ -428,17 +439,6 @@ __device__ __forceinline__ double hs_R(const Params& P, double a) {
   const double ia = 1.0 / a, ia2 = ia * ia;
   const double sq2pi = 0.79788456080286535588;  // sqrt(2/pi)
   return sq2pi * (1.0 + ia2) * exp(-0.5 * a2) + (a + 2.0 * ia - ia2 * ia) * erf(a * 0.70710678118654752440);
-}
-
-// <Delta v^M> of Eq. vel_change_1c for a particle of velocity v in a cell of c.
-__device__ __forceinline__ void hs_source(const Params& P, double vx, double vy, double vz, int c,
-                                          double* sx, double* sy, double* sz) {
-  const double mx = P.vmean[0] - vx, my = P.vmean[1] - vy, mz = P.vmean[2] - vz;
-  const double a = sqrt(mx * mx + my * my + mz * mz) * P.inv_vsig;
-  const double f = P.src_pref * (double)(c - 1) * P.vsig * hs_R(P, a);
-  *sx = f * mx;
-  *sy = f * my;
-  *sz = f * mz;
 }
 
 // Cells above kBigCell particles are ranked by a block-level bitonic sort
@@ -647,6 +647,9 @@ struct pic_ctx {
   // collisions
   double* overlay;  // per-lane working velocities
   int dsmc_grid, dsmc_block, dsmc_G, dsmc_Kc, bm_words;
+  int dsmc_stage;   // FP64 form: particles of a cell group staged in shared memory
+  int dsmc_parts;   // FP64 form: warps that share a group's outcomes, and their sums [parts][3][N_p]
+  double* dsmc_partial;
   int64_t dsmc_groups;
   size_t dsmc_smem;
   pic::AdjointBuffers* adj;      // pathwise-adjoint working set, allocated on first use
