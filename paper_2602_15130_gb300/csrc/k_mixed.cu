@@ -21,30 +21,165 @@ inline int blocks_for(int64_t n, int t = kThreads) {
   return (int)(b < 1 ? 1 : b);
 }
 
-// --------------------------------------------------------------- sampling --
+// ------------------------------------------------- sampling and state load --
+// Where a state in pid order goes: as arrays into the current buffer, or,
+// for the sort that follows, as 32-byte records (o0 o1 o2 v0 | v1 v2 pid -),
+// either straight into per-cell bins ([ncell][bin_cap], arrival rank r at
+// slot r; a rank at or above bin_cap sets *bin_over) or in pid order with
+// cell keys and arrival ranks. v^M depends only on the pid: it is kept by pid
+// (m0 m1 m2 -) and joins the particle in the sort.
+//
+// A record is one aligned sector (two with v^M). At 134M particles a load of
+// rows in device memory takes 3.5 ms, bound by the random sectors: records of
+// 48 bytes (which share sectors), written in pid order as well as into the
+// bins, with v^M gathered through the inverse of the old order, took 20.4.
+struct Put32 {
+  float4* rec;
+  float4* bins;
+  int64_t bin_cap;
+  int words;      // float4 a binned record: 2, or 4 with v^M
+  int* bin_over;
+  int32_t *key, *rank, *count;
+  int32_t* cell;  // arrays (rec and bins null)
+  float *o0, *o1, *o2, *v0, *v1, *v2, *m0, *m1, *m2;
+  uint32_t* pid;
+};
+
+// one 32-byte store: a whole sector in one transaction (two 16-byte stores
+// reach L2 as two partial writes: 5.8 ms instead of 3.5 for 134M random
+// records)
+__device__ __forceinline__ void store_record(float4* p, const float4& a, const float4& b) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+               "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+               : "memory");
+}
+
+__device__ __forceinline__ void put32(const Put32& a, int64_t i, int32_t cell, const float* o, const float* v,
+                                      const float4& m) {
+  if (a.rec || a.bins) {
+    // neighbours in pid order lie in unrelated cells: one atomic each
+    const int32_t rk = atomicAdd(a.count + cell, 1);
+    float4* q = a.rec + 2 * i;
+    if (a.bins) {
+      if (rk >= a.bin_cap) {
+        *a.bin_over = 1;
+        return;
+      }
+      q = a.bins + a.words * ((int64_t)cell * a.bin_cap + rk);
+      if (a.words == 4) store_record(q + 2, m, make_float4(0.f, 0.f, 0.f, 0.f));
+    } else {
+      a.key[i] = cell;
+      a.rank[i] = rk;
+    }
+    store_record(q, make_float4(o[0], o[1], o[2], v[0]),
+                 make_float4(v[1], v[2], __uint_as_float((uint32_t)i), 0.f));
+    return;
+  }
+  a.cell[i] = cell;
+  a.o0[i] = o[0]; a.o1[i] = o[1]; a.o2[i] = o[2];
+  a.v0[i] = v[0]; a.v1[i] = v[1]; a.v2[i] = v[2];
+  a.m0[i] = m.x; a.m1[i] = m.y; a.m2[i] = m.z;
+  a.pid[i] = (uint32_t)i;
+}
+
 struct Sample32Args {
   Params P;
   TimeTerms tt;
-  int64_t row0, row_end;  // the particles (pids) this launch takes
-  const double *xs, *vs;  // optional caller state (pid order, [N][3] each; device or mapped host)
-  // optional v^M (tau for the paper's f_v) to keep: a context's sorted
-  // arrays, read for pid i at vslot[i] (the inverse sort permutation)
-  const int32_t* vslot;
-  const float *vin0, *vin1, *vin2;
-  // optional: the state as 48-byte records in pid order (o0 o1 o2 v0 | v1 v2
-  // m0 m1 | m2 cell pid -) with its cell keys and in-cell arrival ranks,
-  // instead of the structure-of-arrays buffers (a state load followed by
-  // the sort: its gather reads the records at random)
-  float4* rec = nullptr;
-  int32_t *key = nullptr, *rank = nullptr, *count = nullptr;
-  // optional, with rec: the records also binned by cell ([ncell][bin_cap],
-  // arrival rank r at slot r); a rank at or above bin_cap sets *bin_over
-  float4* bins = nullptr;
-  int64_t bin_cap = 0;
-  int* bin_over = nullptr;
-  int32_t* cell;
-  float *o0, *o1, *o2, *v0, *v1, *v2, *m0, *m1, *m2;
-  uint32_t* pid;
+  float4* vm;      // out: v^M (tau for the paper's f_v) by pid
+  int state;       // 0: v^M only
+  Put32 put;
+};
+
+__global__ void __launch_bounds__(kThreads) k_sample32(Sample32Args a) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const Params& P = a.P;
+  if (i >= P.np) return;
+  const U4 b0 = sample_block(P, (uint64_t)i, 0), b1 = sample_block(P, (uint64_t)i, 1),
+           b2 = sample_block(P, (uint64_t)i, 2);
+  const double xi[6] = {unif52(b0.x, b0.y), unif52(b0.z, b0.w), unif52(b1.x, b1.y),
+                        unif52(b1.z, b1.w), unif52(b2.x, b2.y), unif52(b2.z, b2.w)};
+  const bool paper = P.dist == PIC_DIST_PAPER;
+  double vm[3];
+  for (int d = 0; d < 3; ++d) vm[d] = paper ? tau_inv(xi[3 + d]) : P.vmean[d] + P.vsig * normcdfinv(xi[3 + d]);
+  const float4 m = make_float4((float)vm[0], (float)vm[1], (float)vm[2], 0.f);
+  a.vm[i] = m;
+  if (!a.state) return;
+  const int n = P.n;
+  int ci[3];
+  float off[3], vf[3];
+  for (int d = 0; d < 3; ++d) {
+    double s, cc;
+    const double x = wrap_unit(paper ? xm_solve_gen(a.tt, d, xi[d], &s, &cc) : xm_solve(P, a.tt, xi[d], &s));
+    vf[d] = (float)(paper ? vm[d] * a.tt.vh[d] : vm[d]);
+    ci[d] = cell_coord(x, n);
+    const float o = (float)fma(x, (double)n, -(double)ci[d]);
+    off[d] = o >= 1.f ? 0x1.fffffep-1f : (o < 0.f ? 0.f : o);
+  }
+  put32(a.put, i, ci[0] + n * (ci[1] + n * ci[2]), off, vf, m);
+}
+
+// The FP64 conversions of the state's rows with integer arithmetic, bit for
+// bit: an FP64 instruction takes a warp 19 cycles of the SM's pipe, and the
+// 21 of a load and 15 of a store took 5.4 and 3.9 ms at 134M particles.
+//
+// (float)x, to nearest
+__device__ __forceinline__ float to_f32(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const uint32_t e = (uint32_t)(b >> 52) & 0x7ffu;
+  if (e - 898u > 1149u - 898u) return (float)x;  // not a normal float (or zero)
+  const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+  return __uint_as_float(((uint32_t)(b >> 32) & 0x80000000u) | ((uint32_t)(r >> 29) - (896u << 23)));
+}
+// (double)f
+__device__ __forceinline__ double to_f64(float f) {
+  const uint32_t b = __float_as_uint(f);
+  const uint32_t e = (b >> 23) & 255u;
+  if (e - 1u > 253u) return (double)f;  // zero, subnormal or not finite
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+// cell and offset of a coordinate, as cell_coord and k_sample32 form them:
+// floor(x n) with x n rounded to FP64; x n - floor(x n) in one rounding (an
+// FMA), then to FP32; both clamped
+__device__ __forceinline__ int split_coord(double x, int n, float* off) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const uint32_t e = (uint32_t)(b >> 52);  // sign and exponent
+  int c;
+  float o;
+  if (e - 1023u + 120u < 120u) {  // 2^-120 <= x < 1
+    const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) * (unsigned long long)n;
+    const int sh = 1075 - (int)e;  // x n = m 2^-sh, exactly
+    unsigned long long r = m;      // rounded to 53 bits
+    const int over = 11 - __clzll((long long)m);
+    if (over > 0) r = (m + ((1ull << (over - 1)) - 1ull) + ((m >> over) & 1ull)) >> over << over;
+    c = sh < 64 ? (int)(r >> sh) : 0;
+    if (c >= n) c = n - 1;
+    const long long f = sh < 64 ? (long long)(m - ((unsigned long long)c << sh)) : (long long)m;
+    o = 0.f;
+    if (f > 0) {
+      const int lz = __clzll(f);
+      unsigned long long g = (unsigned long long)f << lz;
+      // to 53 bits, then to 24
+      g = g >= 0xfffffffffffffc00ull ? 0xffffffffffffffffull : (g + 0x3ffull + ((g >> 11) & 1ull)) & ~0x7ffull;
+      uint32_t q = (uint32_t)(g >> 40);
+      const unsigned long long rest = g & 0xffffffffffull;
+      q += rest > 0x8000000000ull || (rest == 0x8000000000ull && (q & 1u)) ? 1u : 0u;
+      // g 2^(-sh - lz) with 24 bits q: q 2^(40 - sh - lz)
+      o = __uint_as_float(((uint32_t)(189 - sh - lz) << 23) + q);
+    }
+  } else {
+    c = cell_coord(x, n);
+    o = (float)fma(x, (double)n, -(double)c);
+  }
+  *off = o >= 1.f ? 0x1.fffffep-1f : (o < 0.f ? 0.f : o);
+  return c;
+}
+
+struct Load32Args {
+  int n;
+  int64_t np;
+  const double *xs, *vs;  // the caller's state (pid order, [N][3] each; device or mapped host)
+  const float4* vm;       // v^M by pid
+  Put32 put;
 };
 
 // A caller's state ([N][3] rows, in place in pinned host memory over
@@ -52,95 +187,36 @@ struct Sample32Args {
 // into shared memory (16-byte loads where the rows allow), so each byte
 // crosses the link once; a thread's three components are then three
 // shared-memory reads.
-__global__ void __launch_bounds__(kThreads) k_sample32(Sample32Args a) {
+__global__ void __launch_bounds__(kThreads) k_load32(Load32Args a) {
   __shared__ __align__(16) double sxs[3 * kThreads], svs[3 * kThreads];
-  const int64_t base = a.row0 + (int64_t)blockIdx.x * kThreads;
+  const int64_t base = (int64_t)blockIdx.x * kThreads;
   const int64_t i = base + threadIdx.x;
-  const Params& P = a.P;
-  if (a.xs) {
-    const int64_t rows = a.row_end - base < kThreads ? a.row_end - base : kThreads;
-    const double* gx = a.xs + 3 * base;
-    const double* gv = a.vs + 3 * base;
-    if (rows == kThreads && ((reinterpret_cast<uintptr_t>(gx) | reinterpret_cast<uintptr_t>(gv)) & 15) == 0) {
-      for (int k = threadIdx.x; k < 3 * kThreads / 2; k += kThreads) {
-        reinterpret_cast<double2*>(sxs)[k] = reinterpret_cast<const double2*>(gx)[k];
-        reinterpret_cast<double2*>(svs)[k] = reinterpret_cast<const double2*>(gv)[k];
-      }
-    } else {
-      for (int64_t k = threadIdx.x; k < 3 * rows; k += kThreads) {
-        sxs[k] = gx[k];
-        svs[k] = gv[k];
-      }
+  const int64_t rows = a.np - base < kThreads ? a.np - base : kThreads;
+  const double* gx = a.xs + 3 * base;
+  const double* gv = a.vs + 3 * base;
+  if (rows == kThreads && ((reinterpret_cast<uintptr_t>(gx) | reinterpret_cast<uintptr_t>(gv)) & 15) == 0) {
+    for (int k = threadIdx.x; k < 3 * kThreads / 2; k += kThreads) {
+      reinterpret_cast<double2*>(sxs)[k] = reinterpret_cast<const double2*>(gx)[k];
+      reinterpret_cast<double2*>(svs)[k] = reinterpret_cast<const double2*>(gv)[k];
     }
-    __syncthreads();
-  }
-  if (i >= a.row_end) return;
-  double xi[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  const bool given_vm = a.vslot != nullptr;
-  const int32_t vj = given_vm ? a.vslot[i] : 0;
-  if (!a.xs || !given_vm) {
-    const U4 b0 = sample_block(P, (uint64_t)i, 0), b1 = sample_block(P, (uint64_t)i, 1),
-             b2 = sample_block(P, (uint64_t)i, 2);
-    xi[0] = unif52(b0.x, b0.y); xi[1] = unif52(b0.z, b0.w); xi[2] = unif52(b1.x, b1.y);
-    xi[3] = unif52(b1.z, b1.w); xi[4] = unif52(b2.x, b2.y); xi[5] = unif52(b2.z, b2.w);
-  }
-  const float* vin[3] = {a.vin0, a.vin1, a.vin2};
-  double x[3], v[3], vm[3];
-  const bool paper = P.dist == PIC_DIST_PAPER;
-  for (int d = 0; d < 3; ++d) {
-    double s, cc;
-    // the paper's f_v: the v^M array holds tau, v^M(t) = vh(t) tau; a state
-    // loaded into a context that already holds one keeps its v^M values
-    if (given_vm)
-      vm[d] = (double)vin[d][vj];
-    else
-      vm[d] = paper ? tau_inv(xi[3 + d]) : P.vmean[d] + P.vsig * normcdfinv(xi[3 + d]);
-    if (a.xs) {
-      x[d] = sxs[3 * threadIdx.x + d];
-      v[d] = svs[3 * threadIdx.x + d];
-    } else if (paper) {
-      x[d] = wrap_unit(xm_solve_gen(a.tt, d, xi[d], &s, &cc));
-      v[d] = vm[d] * a.tt.vh[d];
-    } else {
-      x[d] = wrap_unit(xm_solve(P, a.tt, xi[d], &s));
-      v[d] = vm[d];
+  } else {
+    for (int64_t k = threadIdx.x; k < 3 * rows; k += kThreads) {
+      sxs[k] = gx[k];
+      svs[k] = gv[k];
     }
   }
-  const int n = P.n;
+  __syncthreads();
+  if (i >= a.np) return;
   int ci[3];
-  float off[3];
+  float off[3], v[3];
+#pragma unroll
   for (int d = 0; d < 3; ++d) {
-    ci[d] = cell_coord(x[d], n);
-    float o = (float)(x[d] * (double)n - (double)ci[d]);
-    off[d] = o >= 1.f ? 0x1.fffffep-1f : (o < 0.f ? 0.f : o);
+    ci[d] = split_coord(sxs[3 * threadIdx.x + d], a.n, &off[d]);
+    v[d] = to_f32(svs[3 * threadIdx.x + d]);
   }
-  const int32_t cell = ci[0] + n * (ci[1] + n * ci[2]);
-  if (a.rec) {
-    const float4 r0 = make_float4(off[0], off[1], off[2], (float)v[0]);
-    const float4 r1 = make_float4((float)v[1], (float)v[2], (float)vm[0], (float)vm[1]);
-    const float4 r2 = make_float4((float)vm[2], __int_as_float(cell), __uint_as_float((uint32_t)i), 0.f);
-    float4* r = a.rec + 3 * i;
-    r[0] = r0; r[1] = r1; r[2] = r2;
-    a.key[i] = cell;
-    const int32_t rk = cell_slot(a.count, cell);
-    a.rank[i] = rk;
-    if (a.bins) {
-      // random 48-byte stores into HBM, while the load itself waits on the
-      // host link
-      if (rk < a.bin_cap) {
-        float4* q = a.bins + 3 * ((int64_t)cell * a.bin_cap + rk);
-        q[0] = r0; q[1] = r1; q[2] = r2;
-      } else {
-        *a.bin_over = 1;
-      }
-    }
-    return;
-  }
-  a.cell[i] = cell;
-  a.o0[i] = off[0]; a.o1[i] = off[1]; a.o2[i] = off[2];
-  a.v0[i] = (float)v[0]; a.v1[i] = (float)v[1]; a.v2[i] = (float)v[2];
-  a.m0[i] = (float)vm[0]; a.m1[i] = (float)vm[1]; a.m2[i] = (float)vm[2];
-  a.pid[i] = (uint32_t)i;
+  float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!a.put.rec && !(a.put.bins && a.put.words == 2)) m = a.vm[i];
+  put32(a.put, i, ci[0] + a.n * (ci[1] + a.n * ci[2]), off, v, m);
 }
 
 struct Keys32Args {
@@ -184,6 +260,29 @@ __global__ void __launch_bounds__(kThreads) k_store_state32(Store32Args a) {
   vs[3 * p] = a.v0[j]; vs[3 * p + 1] = a.v1[j]; vs[3 * p + 2] = a.v2[j];
 }
 
+// The state in pid order, for a destination the kernels write in place.
+// Into device memory: the particles are scattered as 32-byte records (o0 o1
+// o2 v0 | v1 v2 cell -), one whole sector each, to their pid's place, and the
+// rows formed from consecutive records. Gathering by the inverse permutation
+// touches seven sectors a particle: 19.7 ms and 2.7 for the permutation at
+// 134M particles, 3.5 and 3.0 by records. Into host memory the rows are bound
+// by the link (33 ms there) and hide the gather; the inverse permutation,
+// which is less work beside them than the records, goes ahead by windows.
+struct ToPid32Args {
+  int64_t np;
+  const int32_t* cell;
+  const float *o0, *o1, *o2, *v0, *v1, *v2;
+  const uint32_t* pid;
+  float4* rec;
+};
+
+__global__ void __launch_bounds__(kThreads) k_to_pid32(ToPid32Args a) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= a.np) return;
+  store_record(a.rec + 2 * (int64_t)a.pid[j], make_float4(a.o0[j], a.o1[j], a.o2[j], a.v0[j]),
+               make_float4(a.v1[j], a.v2[j], __int_as_float(a.cell[j]), 0.f));
+}
+
 // Inverse of the sort permutation: the slot of every pid, in passes over
 // windows of kInvWindow pids. Each pass streams every pid and writes only
 // the slots of its window, so its random 4-byte stores land in a span L2
@@ -223,32 +322,66 @@ __global__ void __launch_bounds__(kThreads) k_inv_perm32_gs(InvPerm32Args a) {
   }
 }
 
-// The state in pid order for a destination the kernel writes in place
-// (device memory, or pinned host memory reached over NVLink-C2C): each
-// thread gathers one pid through the inverse permutation, the block's rows
-// go through shared memory, and the stores cover contiguous spans. Same
-// arithmetic as k_store_state32. Rows row0 .. row_end - 1.
+// Rows row0 .. row_end - 1 (pids), from the records or (rec null) through
+// the inverse permutation; they go through shared memory, so that the stores
+// cover contiguous spans. Same values as k_store_state32 (integer
+// conversions; the cell index plus the offset is the only FP64 sum, and the
+// product with h = 2^-k an exponent).
 struct StoreByPid32Args {
   int64_t row0, row_end;
-  int n;
+  int n, log2n;
   double h;
+  const float4* rec;
   const int32_t *slot, *cell;
   const float *o0, *o1, *o2, *v0, *v1, *v2;
   double *x, *v;
 };
+__device__ __forceinline__ double small_int(int c) {  // 0 <= c < 2^20
+  if (c == 0) return 0.0;
+  const int e = 31 - __clz(c);
+  return __hiloint2double(((1023 + e) << 20) + ((c << (20 - e)) & 0xfffff), 0);
+}
 
 __global__ void __launch_bounds__(kThreads) k_store_state32_by_pid(StoreByPid32Args a) {
   __shared__ __align__(16) double sx[3 * kThreads], sv[3 * kThreads];
   const int64_t base = a.row0 + (int64_t)blockIdx.x * kThreads;
   const int t = threadIdx.x;
   if (base + t < a.row_end) {
-    const int64_t j = a.slot[base + t];
-    const int n = a.n, c = a.cell[j];
-    const int ci = c % n, cj = (c / n) % n, ck = c / (n * n);
-    sx[3 * t] = ((double)ci + (double)a.o0[j]) * a.h;
-    sx[3 * t + 1] = ((double)cj + (double)a.o1[j]) * a.h;
-    sx[3 * t + 2] = ((double)ck + (double)a.o2[j]) * a.h;
-    sv[3 * t] = a.v0[j]; sv[3 * t + 1] = a.v1[j]; sv[3 * t + 2] = a.v2[j];
+    float o[3], v[3];
+    int c;
+    if (a.rec) {
+      const float4 r0 = a.rec[2 * (base + t)], r1 = a.rec[2 * (base + t) + 1];
+      o[0] = r0.x; o[1] = r0.y; o[2] = r0.z;
+      v[0] = r0.w; v[1] = r1.x; v[2] = r1.y;
+      c = __float_as_int(r1.z);
+    } else {
+      const int64_t j = a.slot[base + t];
+      o[0] = a.o0[j]; o[1] = a.o1[j]; o[2] = a.o2[j];
+      v[0] = a.v0[j]; v[1] = a.v1[j]; v[2] = a.v2[j];
+      c = a.cell[j];
+    }
+    int ci[3];
+    if (a.log2n >= 0) {
+      ci[0] = c & (a.n - 1);
+      ci[1] = (c >> a.log2n) & (a.n - 1);
+      ci[2] = c >> (2 * a.log2n);
+    } else {
+      ci[0] = c % a.n;
+      ci[1] = (c / a.n) % a.n;
+      ci[2] = c / (a.n * a.n);
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double y = small_int(ci[d]) + to_f64(o[d]);
+      const int hi = __double2hiint(y);
+      // the product with h = 2^-log2n by its exponent (y is zero, at least
+      // 2^-149, or not finite)
+      if (a.log2n >= 0 && hi != 0 && (hi & 0x7ff00000) != 0x7ff00000)
+        sx[3 * t + d] = __hiloint2double(hi - (a.log2n << 20), __double2loint(y));
+      else
+        sx[3 * t + d] = y * a.h;
+      sv[3 * t + d] = to_f64(v[d]);
+    }
   }
   __syncthreads();
   const int64_t rows = a.row_end - base < kThreads ? a.row_end - base : kThreads;
@@ -1651,92 +1784,73 @@ __global__ void __launch_bounds__(kThreads) k_store_dv32(StoreDv32Args a) {
 }  // namespace
 
 // ============================================================== launches ==
-// The inverse of a sort permutation (slot[pid[j]] = j) by windows of
-// kInvWindow pids, each window's pass on the context's auxiliary stream
-// (higher priority) ahead of consume(lo, hi), which the caller launches on
-// the context's stream for the rows (pids) lo .. hi - 1 of a load or store
-// that waits on the host link: window r's pass runs beside the consumer of
-// window r - 1. Only the first pass is not hidden; it takes a grid of one
-// thread per pid, the later ones two blocks per SM, so that they do not
-// hold the SMs the consumer needs (full-grid passes there took every SM a
-// consumer block freed, and the two kernels took turns).
-template <class Consume>
-cudaError_t inverse_by_windows(pic_ctx* c, const uint32_t* pid, Consume consume) {
-  cudaError_t e = ensure_aux_stream(c);
-  if (e != cudaSuccess) return e;
-  InvPerm32Args ia;
-  ia.np = c->P.np;
-  ia.pid = pid;
-  ia.slot = c->perm;
-  // the auxiliary stream starts after the work already on the context's
-  e = cudaEventRecord(c->aux_fork, c->stream);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->aux, c->aux_fork, 0);
-  for (int64_t lo = 0; lo < ia.np && e == cudaSuccess; lo += kInvWindow) {
-    ia.lo = lo;
-    ia.hi = lo + kInvWindow < ia.np ? lo + kInvWindow : ia.np;
-    if (lo == 0)
-      k_inv_perm32<<<blocks_for(ia.np), kThreads, 0, c->aux>>>(ia);
-    else
-      k_inv_perm32_gs<<<2 * c->num_sms, kThreads, 0, c->aux>>>(ia);
-    c->launches++;
-    // the wait takes the record made just before it, so one event serves
-    // every window
-    e = cudaEventRecord(c->aux_join, c->aux);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->aux_join, 0);
-    if (e == cudaSuccess) consume(ia.lo, ia.hi);
+static Put32 put_target(pic_ctx* c, LoadTarget target) {
+  Put32 a{};
+  if (target == LoadTarget::kArrays) {
+    const int b = c->cur;
+    a.cell = c->cell32[b];
+    a.o0 = c->off[b][0]; a.o1 = c->off[b][1]; a.o2 = c->off[b][2];
+    a.v0 = c->vf[b][0]; a.v1 = c->vf[b][1]; a.v2 = c->vf[b][2];
+    a.m0 = c->vmf[b][0]; a.m1 = c->vmf[b][1]; a.m2 = c->vmf[b][2];
+    a.pid = c->pid[b];
+    return a;
   }
-  return e == cudaSuccess ? cudaGetLastError() : e;
-}
-
-cudaError_t launch_sample32(pic_ctx* c, double t0, const double* x, const double* v, int held, bool to_records) {
-  Sample32Args a;
-  a.P = c->P;
-  a.tt = time_terms(c->P, t0);
-  a.row0 = 0;
-  a.row_end = c->P.np;
-  a.xs = x;
-  a.vs = v;
-  a.vslot = held >= 0 ? c->perm : nullptr;
-  a.vin0 = held >= 0 ? c->vmf[held][0] : nullptr;
-  a.vin1 = held >= 0 ? c->vmf[held][1] : nullptr;
-  a.vin2 = held >= 0 ? c->vmf[held][2] : nullptr;
-  const int b = c->cur;
-  a.cell = c->cell32[b];
-  a.o0 = c->off[b][0]; a.o1 = c->off[b][1]; a.o2 = c->off[b][2];
-  a.v0 = c->vf[b][0]; a.v1 = c->vf[b][1]; a.v2 = c->vf[b][2];
-  a.m0 = c->vmf[b][0]; a.m1 = c->vmf[b][1]; a.m2 = c->vmf[b][2];
-  a.pid = c->pid[b];
-  if (to_records) {
+  a.count = c->count;
+  if (target == LoadTarget::kBins) {
+    a.bins = c->bins;
+    a.bin_cap = c->bin_cap;
+    a.words = c->bin_words = 2;
+    a.bin_over = c->bin_over;
+  } else {
     a.rec = reinterpret_cast<float4*>(c->stage);
     a.key = c->key;
     a.rank = c->rank;
-    a.count = c->count;
-    if (c->bins) {
-      a.bins = c->bins;
-      a.bin_cap = c->bin_cap;
-      a.bin_over = c->bin_over;
-    }
   }
-  if (held < 0 || c->inv_valid) {
-    prof_begin(c);
-    k_sample32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(a);
-    prof_end(c, x ? KC_OTHER : KC_SAMPLE);
-    c->launches++;
-    return cudaGetLastError();
-  }
-  // v^M read through the inverse of the held state's permutation, formed
-  // by windows ahead of the load of the same rows (pids)
+  return a;
+}
+
+cudaError_t launch_sample32(pic_ctx* c, double t0, LoadTarget target) {
+  Sample32Args a;
+  a.P = c->P;
+  a.tt = time_terms(c->P, t0);
+  a.vm = c->vm_by_pid;
+  a.state = 1;
+  a.put = put_target(c, target);
   prof_begin(c);
-  const cudaError_t e = inverse_by_windows(c, c->pid[held], [&](int64_t lo, int64_t hi) {
-    a.row0 = lo;
-    a.row_end = hi;
-    k_sample32<<<blocks_for(hi - lo), kThreads, 0, c->stream>>>(a);
+  k_sample32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(a);
+  prof_end(c, KC_SAMPLE);
+  c->launches++;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_load32(pic_ctx* c, const double* x, const double* v, LoadTarget target, bool host) {
+  prof_begin(c);
+  if (!c->sampled) {
+    // the context's first state: v^M of every pid
+    Sample32Args s;
+    s.P = c->P;
+    s.tt = time_terms(c->P, 0.0);
+    s.vm = c->vm_by_pid;
+    s.state = 0;
+    s.put = Put32{};
+    k_sample32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(s);
     c->launches++;
-  });
+  }
+  Load32Args a;
+  a.n = c->P.n;
+  a.np = c->P.np;
+  a.xs = x;
+  a.vs = v;
+  a.vm = c->vm_by_pid;
+  a.put = put_target(c, target);
+  // v^M in the binned record where the load waits on the host link: 1.3 ms
+  // less for the sort at 134M particles, but 2.3 ms more for the load's
+  // stores, which only the link hides
+  if (host && target == LoadTarget::kBins) c->bin_words = a.put.words = c->bin_words_max;
+  k_load32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(a);
   prof_end(c, KC_OTHER);
-  // perm now holds the inverse of the held state's order, which the sort
-  // that follows replaces
-  return e;
+  c->launches++;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_keys32(pic_ctx* c) {
@@ -1772,6 +1886,8 @@ cudaError_t launch_gather32(pic_ctx* c) {
   g.spid = c->pid[o];  // written in arrival order by the scatter
   if (c->rec_state) {
     g.rec = c->bin_state ? c->bins : reinterpret_cast<const float4*>(c->stage);
+    g.vm = c->vm_by_pid;
+    g.rec_words = c->bin_state ? c->bin_words : 2;
     g.bin_cap = c->bin_state ? c->bin_cap : 0;
     g.spid = nullptr;  // the pids come with the records
   }
@@ -2026,19 +2142,55 @@ cudaError_t launch_store_state32(pic_ctx* c, double* xv, int32_t* cell_of_pid) {
   return cudaGetLastError();
 }
 
-// x, v [N_p][3] in pid order written in place (device or mapped pinned host
-// memory, 8-byte aligned); the inverse permutation goes into the sort's
-// free permutation buffer
+// The inverse of a sort permutation (slot[pid[j]] = j) by windows of
+// kInvWindow pids, each window's pass on the context's auxiliary stream
+// (higher priority) ahead of consume(lo, hi), which the caller launches on
+// the context's stream for the rows (pids) lo .. hi - 1 of a store that
+// waits on the host link: window r's pass runs beside the consumer of
+// window r - 1. Only the first pass is not hidden; it takes a grid of one
+// thread per pid, the later ones two blocks per SM, so that they do not
+// hold the SMs the consumer needs (full-grid passes there took every SM a
+// consumer block freed, and the two kernels took turns).
+template <class Consume>
+cudaError_t inverse_by_windows(pic_ctx* c, const uint32_t* pid, Consume consume) {
+  cudaError_t e = ensure_aux_stream(c);
+  if (e != cudaSuccess) return e;
+  InvPerm32Args ia;
+  ia.np = c->P.np;
+  ia.pid = pid;
+  ia.slot = c->perm;
+  // the auxiliary stream starts after the work already on the context's
+  e = cudaEventRecord(c->aux_fork, c->stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->aux, c->aux_fork, 0);
+  for (int64_t lo = 0; lo < ia.np && e == cudaSuccess; lo += kInvWindow) {
+    ia.lo = lo;
+    ia.hi = lo + kInvWindow < ia.np ? lo + kInvWindow : ia.np;
+    if (lo == 0)
+      k_inv_perm32<<<blocks_for(ia.np), kThreads, 0, c->aux>>>(ia);
+    else
+      k_inv_perm32_gs<<<2 * c->num_sms, kThreads, 0, c->aux>>>(ia);
+    c->launches++;
+    // the wait takes the record made just before it, so one event serves
+    // every window
+    e = cudaEventRecord(c->aux_join, c->aux);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->aux_join, 0);
+    if (e == cudaSuccess) consume(ia.lo, ia.hi);
+  }
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
 
-// Into arrays in pid order used in place; without a valid inverse the
-// store goes by windows of the inverse.
-cudaError_t launch_store_state32_by_pid(pic_ctx* c, double* x, double* v) {
+// x, v [N_p][3] in pid order written in place (device memory, or mapped
+// pinned host memory: host; 8-byte aligned). The records take the staging
+// area, the inverse permutation the sort's free permutation buffer.
+cudaError_t launch_store_state32_by_pid(pic_ctx* c, double* x, double* v, bool host) {
   const int b = c->cur;
   StoreByPid32Args a;
   a.row0 = 0;
   a.row_end = c->P.np;
   a.n = c->P.n;
+  a.log2n = (c->P.n & (c->P.n - 1)) == 0 ? __builtin_ctz((unsigned)c->P.n) : -1;
   a.h = c->P.h;
+  a.rec = nullptr;
   a.slot = c->perm;
   a.cell = c->cell32[b];
   a.o0 = c->off[b][0]; a.o1 = c->off[b][1]; a.o2 = c->off[b][2];
@@ -2047,7 +2199,20 @@ cudaError_t launch_store_state32_by_pid(pic_ctx* c, double* x, double* v) {
   a.v = v;
   prof_begin(c);
   cudaError_t e;
-  if (c->inv_valid) {
+  if (!host) {
+    ToPid32Args s;
+    s.np = c->P.np;
+    s.cell = a.cell;
+    s.o0 = a.o0; s.o1 = a.o1; s.o2 = a.o2;
+    s.v0 = a.v0; s.v1 = a.v1; s.v2 = a.v2;
+    s.pid = c->pid[b];
+    s.rec = reinterpret_cast<float4*>(c->stage);
+    a.rec = s.rec;
+    k_to_pid32<<<blocks_for(s.np), kThreads, 0, c->stream>>>(s);
+    k_store_state32_by_pid<<<blocks_for(a.row_end), kThreads, 0, c->stream>>>(a);
+    c->launches += 2;
+    e = cudaGetLastError();
+  } else if (c->inv_valid) {
     k_store_state32_by_pid<<<blocks_for(a.row_end), kThreads, 0, c->stream>>>(a);
     c->launches++;
     e = cudaGetLastError();

@@ -365,7 +365,6 @@ cudaError_t launch_scan_scatter(pic_ctx* c) {
 }
 
 cudaError_t launch_sort(pic_ctx* c) {
-  c->inv_valid = false;
   const int64_t m = c->P.ncell;
   cudaError_t e = launch_scan_scatter(c);
   if (e != cudaSuccess) return e;

@@ -235,10 +235,13 @@ struct Gather32Args {
   double* corner;       // [8][ncell]
   int big_lo;             // cells above this count go to the block sort
   const uint32_t* spid;   // optional: pids in arrival order (slot s + e holds perm[s + e]'s pid)
-  // optional: the source as 48-byte records (o0 o1 o2 v0 | v1 v2 m0 m1 |
-  // m2 cell pid -) instead of in[] and pid_in: a random source read as
-  // records touches two 32-byte sectors a particle instead of nine
+  // optional: the source as records (o0 o1 o2 v0 | v1 v2 pid -) instead of
+  // in[] and pid_in, with v^M (m0 m1 m2 -) behind them (rec_words 4) or by
+  // pid in vm (rec_words 2): a random source read so touches two 32-byte
+  // sectors a particle instead of nine
   const float4* rec = nullptr;
+  const float4* vm = nullptr;
+  int rec_words = 2;
   // records binned by cell (rec holds [ncell][bin_cap] records, a cell's
   // arrival e at its slot e): each cell reads its own contiguous span, and
   // perm is not used
@@ -250,11 +253,12 @@ struct Gather32Args {
 template <bool kRec>
 __device__ __forceinline__ void gather_load32(const Gather32Args& a, const float4* rb, int32_t src, float* d) {
   if constexpr (kRec) {
-    const float4 r0 = __ldg(rb + 3 * (int64_t)src), r1 = __ldg(rb + 3 * (int64_t)src + 1),
-                 r2 = __ldg(rb + 3 * (int64_t)src + 2);
+    const float4* r = rb + a.rec_words * (int64_t)src;
+    const float4 r0 = __ldg(r), r1 = __ldg(r + 1);
+    const float4 m = __ldg(a.rec_words == 4 ? r + 2 : a.vm + __float_as_uint(r1.z));
     d[0] = r0.x; d[1] = r0.y; d[2] = r0.z; d[3] = r0.w;
-    d[4] = r1.x; d[5] = r1.y; d[6] = r1.z; d[7] = r1.w;
-    d[8] = r2.x;
+    d[4] = r1.x; d[5] = r1.y;
+    d[6] = m.x; d[7] = m.y; d[8] = m.z;
   } else {
 #pragma unroll
     for (int q = 0; q < 9; ++q) d[q] = a.in[q][src];
@@ -262,7 +266,7 @@ __device__ __forceinline__ void gather_load32(const Gather32Args& a, const float
 }
 template <bool kRec>
 __device__ __forceinline__ uint32_t gather_pid32(const Gather32Args& a, const float4* rb, int32_t src) {
-  if constexpr (kRec) return __float_as_uint(__ldg(rb + 3 * (int64_t)src + 2).z);
+  if constexpr (kRec) return __float_as_uint(__ldg(rb + a.rec_words * (int64_t)src + 1).z);
   else return a.pid_in[src];
 }
 
@@ -408,7 +412,7 @@ __device__ __forceinline__ void gather_cell32(const Gather32Args& a, int64_t cel
   if constexpr (kRec) {
     if (a.bin_cap > 0) {
       binned = true;
-      rb += 3 * cell * a.bin_cap;
+      rb += a.rec_words * cell * a.bin_cap;
     }
   }
   const int32_t nch = (cnt + 31) >> 5;  // warp-uniform

@@ -377,6 +377,7 @@ void for_each_buffer(pic_ctx* c, F f) {
       f((void**)&c->dvf[d], np * 4);
       if (c->nrep == 0) f((void**)&c->dvmf[d], np * 4);  // pic_collide_avg only
     }
+    if (c->nrep == 0) f((void**)&c->vm_by_pid, np * 16);
     f((void**)&c->Ef4, nc * 16);
     f((void**)&c->bf, nc * 4);
     f((void**)&c->phif, nc * 4);
@@ -450,6 +451,16 @@ T* in_place(const pic_ctx* c, T* p) {
   return nullptr;
 }
 
+// whether a caller array used in place is host memory
+bool in_host(const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeHost;
+}
+
 // Read and clear the sticky device flags of the work enqueued so far
 // (synchronises the stream).
 pic_status check_pending(pic_ctx* c) {
@@ -470,14 +481,12 @@ pic_status check_pending(pic_ctx* c) {
   return PIC_OK;
 }
 
-// sort by (cell, pid) from the current positions and solve the field at t
-// keys_done: the state load wrote the keys, ranks and counts itself
-// Bins for a state load's records, by cell: a capacity of four times the
-// mean particles per cell (a multiple of 32), if that is at most kBigCell
-// (larger cells take the block sort, which reads through perm), the bins
-// hold at most eight times the records (a sparse state on a fine mesh
+// Bins for the records of a state in pid order, by cell: a capacity of four
+// times the mean particles per cell (a multiple of 32), if that is at most
+// kBigCell (larger cells take the block sort, which reads through perm), the
+// bins hold at most eight times the records (a sparse state on a fine mesh
 // would mostly bin nothing) and take at most a quarter of the free device
-// memory. Tried once per context; without bins the loads take the scatter
+// memory. Tried once per context; without bins the states take the scatter
 // and a random gather.
 void ensure_bins(pic_ctx* c) {
   if (c->bin_tried) return;
@@ -486,13 +495,15 @@ void ensure_bins(pic_ctx* c) {
   const int64_t mean = (c->P.np + c->P.ncell - 1) / c->P.ncell;
   int64_t cap = (4 * mean + 31) / 32 * 32;
   if (cap > kBigCell) return;
-  const size_t bytes = (size_t)c->P.ncell * (size_t)cap * 48;
-  if (bytes > (size_t)8 * 48 * (size_t)c->P.np) return;
+  const size_t records = (size_t)c->P.ncell * (size_t)cap;
+  if (records > (size_t)8 * (size_t)c->P.np) return;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
     cudaGetLastError();
     return;
   }
+  c->bin_words_max = records * 64 <= free_b / 4 ? 4 : 2;
+  const size_t bytes = records * 16 * c->bin_words_max;
   if (bytes > free_b / 4) return;
   c->bins = (float4*)dev_alloc(c, bytes);
   c->bin_over = (int*)dev_alloc(c, sizeof(int));
@@ -506,6 +517,8 @@ void ensure_bins(pic_ctx* c) {
   c->bin_cap = cap;
 }
 
+// sort by (cell, pid) from the current positions and solve the field at t;
+// keys_done: the state was written with its keys, ranks and counts
 pic_status sort_and_field(pic_ctx* c, double t, bool keys_done = false) {
   c->lor_valid = false;
   if (!keys_done) CK(cudaMemsetAsync(c->count, 0, (size_t)c->P.ncell * 4, c->stream));
@@ -530,23 +543,29 @@ pic_status sort_and_field(pic_ctx* c, double t, bool keys_done = false) {
 double time_at(const pic_ctx* c, double steps) { return c->t0 + steps * c->cfg.dt; }
 
 // The precision form's state in pid order (sampled, or a caller's rows used
-// in place, keeping the v^M of a held state buffer) written by the sampling
-// kernel as records in the staging area and into the per-cell bins, then
-// sorted with its field: from the bins, or, when a cell outgrew its bin
-// (or there are no bins), by the scatter and a random gather of the
-// records. *binned: the sort read the bins.
-pic_status records_then_sort(pic_ctx* c, double t, const double* xs, const double* vs, int held, bool* binned) {
+// in place) written as records for the sort, and the sort with its field:
+// into the per-cell bins, and again as records in the staging area when a
+// cell outgrows its bin (or straight there without bins), which the sort
+// reads through a scatter and a random gather. *binned: the sort read the
+// bins.
+pic_status records_then_sort(pic_ctx* c, double t, const double* xs, const double* vs, bool* binned) {
   ensure_bins(c);
-  CK(cudaMemsetAsync(c->count, 0, (size_t)c->P.ncell * 4, c->stream));
-  if (c->bins) CK(cudaMemsetAsync(c->bin_over, 0, sizeof(int), c->stream));
-  CK(launch_sample32(c, t, xs, vs, held, true));
   *binned = false;
+  const bool host = xs && (in_host(xs) || in_host(vs));
+  auto write = [&](LoadTarget target) -> cudaError_t {
+    const cudaError_t e = cudaMemsetAsync(c->count, 0, (size_t)c->P.ncell * 4, c->stream);
+    if (e != cudaSuccess) return e;
+    return xs ? launch_load32(c, xs, vs, target, host) : launch_sample32(c, t, target);
+  };
   if (c->bins) {
+    CK(cudaMemsetAsync(c->bin_over, 0, sizeof(int), c->stream));
+    CK(write(LoadTarget::kBins));
     int over = 1;
     CK(cudaMemcpyAsync(&over, c->bin_over, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     *binned = over == 0;
   }
+  if (!*binned) CK(write(LoadTarget::kRecords));
   c->rec_state = true;
   c->bin_state = *binned;
   pic_status s = sort_and_field(c, t, true);
@@ -1074,7 +1093,7 @@ pic_status pic_sample_mms(pic_ctx* c, double t0) {
     // at random: through the records and the bins, as a state load
     CK(cudaMemsetAsync(c->phif, 0, (size_t)c->P.ncell * 4, c->stream));
     bool binned = false;
-    pic_status s = records_then_sort(c, t0, nullptr, nullptr, -1, &binned);
+    pic_status s = records_then_sort(c, t0, nullptr, nullptr, &binned);
     if (s != PIC_OK) return s;
     c->sampled = true;
     return check_pending(c);
@@ -1107,29 +1126,19 @@ pic_status pic_set_state(pic_ctx* c, const double* x, const double* v, double t0
   c->step = step;
   CK(restart_history(c));
   if (c->mixed) {
-    // v^M is a per-particle constant (tau for the paper's f_v): a context that
-    // already holds a state keeps its values, read through the inverse sort
-    // permutation by the load, instead of re-deriving them from xi in FP64.
-    // Caller arrays used in place leave the staging area free: the load then
-    // writes the state there as records, which the sort's random gather
-    // reads in two sectors a particle instead of nine.
+    // caller arrays used in place leave the staging area free: the state then
+    // goes to the sort as records
     const bool records = xs != c->stage && vs != c->stage + 3 * c->P.np;
     if (records) {
       bool binned = false;
-      pic_status s = records_then_sort(c, time_at(c, (double)step), xs, vs, c->sampled ? c->cur : -1, &binned);
+      pic_status s = records_then_sort(c, time_at(c, (double)step), xs, vs, &binned);
       if (s != PIC_OK) return s;
       if (binned) c->binned_loads++;
       c->sampled = true;
       return check_pending(c);
     }
-    if (c->sampled) {
-      const int src = c->cur;
-      c->cur = 1 - src;
-      CK(launch_sample32(c, time_at(c, (double)step), xs, vs, src));
-    } else {
-      c->cur = 0;
-      CK(launch_sample32(c, time_at(c, (double)step), xs, vs));
-    }
+    c->cur = 0;
+    CK(launch_load32(c, xs, vs, LoadTarget::kArrays, false));
   } else {
     c->cur = 0;
     CK(launch_load_state(c, xs, vs, time_at(c, (double)step)));
@@ -1242,7 +1251,8 @@ pic_status pic_get_state(pic_ctx* c, double* x, double* v) {
     double* xd = in_place(c, x);
     double* vd = in_place(c, v);
     if (xd && vd) {
-      CK(launch_store_state32_by_pid(c, xd, vd));
+      // host rows in either array: bound by the link
+      CK(launch_store_state32_by_pid(c, xd, vd, in_host(x) || in_host(v)));
       CK(cudaStreamSynchronize(c->stream));
       return PIC_OK;
     }

@@ -615,20 +615,24 @@ struct pic_ctx {
   double* dv[3];    // collision term per particle (sorted order)
   double* lor[3];   // dt q/m (E_p - E^M_p) of the last kick without drift
   bool lor_valid;   // lor matches the current order, positions and field
-  bool rec_state;   // the next sort reads the state from records in the staging area
-  // A state load's records binned by cell as well ([ncell][bin_cap]
-  // records; allocated at the first load that reads the caller's arrays
-  // in place, when they fit): the sort then reads each cell's records as
-  // one span, and skips its scatter, unless a cell outgrew its bin.
+  // precision form: v^M (tau for the paper's f_v) by pid, written with the
+  // context's first state
+  float4* vm_by_pid;
+  bool rec_state;   // the next sort reads the state from records, in the staging area or the bins
+  // Bins for the records of a state in pid order ([ncell][bin_cap]; allocated
+  // with the first state that is sampled or read in place, when they fit):
+  // the sort reads each cell's records as one span, and skips its scatter,
+  // unless a cell outgrows its bin.
   float4* bins;
   int64_t bin_cap;  // 0: no bins
+  int bin_words, bin_words_max;  // float4 a record (2, or 4 with v^M): of the current ones, and room for
   int* bin_over;    // device flag: some cell held more than bin_cap particles
   bool bin_tried;   // the bins' allocation was attempted
   bool bin_state;   // the next sort reads the records from the bins
   int64_t binned_loads;  // state loads sorted from the bins (pic_stats)
   bool inv_valid;   // perm holds the inverse of the current sort permutation
   // auxiliary stream (created at first use, higher priority) and its fork
-  // and join events: the inverse permutation overlaps the state store
+  // and join events: the inverse permutation overlaps a state store
   cudaStream_t aux;
   cudaEvent_t aux_fork, aux_join;
   // multigrid-preconditioned CG of the precision form (0 levels: plain CG)
@@ -818,14 +822,12 @@ cudaError_t launch_scan(pic_ctx* c);           // scan of counts into start
 cudaError_t launch_scan_scatter(pic_ctx* c);   // scan of counts + scatter into perm
 cudaError_t launch_err_final(pic_ctx* c, int nblocks);
 // precision form
-// held >= 0: the buffer of a state the context holds, whose v^M (tau) the
-// load keeps instead of recomputing them, read from its sorted arrays at
-// the inverse of its sort permutation (formed here when perm does not hold
-// it); to_records: write the state into the staging area as 48-byte records
-// with their cell keys and ranks (sort_and_field then skips the keys), for
-// a state load whose caller arrays are used in place
-cudaError_t launch_sample32(pic_ctx* c, double t0, const double* x, const double* v, int held = -1,
-                           bool to_records = false);
+// A state in pid order, sampled or read from a caller's rows, as arrays of
+// the current buffer, or for the sort that follows (which then needs no
+// keys) as records binned by cell or in the staging area
+enum class LoadTarget { kArrays, kBins, kRecords };
+cudaError_t launch_sample32(pic_ctx* c, double t0, LoadTarget target);
+cudaError_t launch_load32(pic_ctx* c, const double* x, const double* v, LoadTarget target, bool host);
 cudaError_t ensure_aux_stream(pic_ctx* c);    // the auxiliary stream and its events
 // the multigrid levels of an n^3 mesh (n a power of two >= 16, else 0) and
 // the floats their coarse levels need
@@ -853,7 +855,7 @@ void adjoint_free(pic_ctx* c);
 cudaError_t launch_cg32(pic_ctx* c);
 cudaError_t launch_errors32(pic_ctx* c, double t);
 cudaError_t launch_store_state32(pic_ctx* c, double* xv_dev, int32_t* cell_of_pid);
-cudaError_t launch_store_state32_by_pid(pic_ctx* c, double* x, double* v);
+cudaError_t launch_store_state32_by_pid(pic_ctx* c, double* x, double* v, bool host);
 cudaError_t launch_store_field32(pic_ctx* c, double* phi, double* E);
 cudaError_t launch_store_dv32(pic_ctx* c, double* dv, double* dvm);
 
