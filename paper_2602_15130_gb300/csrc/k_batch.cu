@@ -9,7 +9,7 @@
 //
 //  - sampling: binary search of the particle's replicate;
 //  - RHS: the node's replicate from rep_of_cell, FP64 manufactured terms;
-//  - CG: a team of blocks per replicate (one per 16,384 nodes, at most 32)
+//  - CG: a team of blocks per replicate (one per 1,024 to 16,384 nodes, at most 32)
 //    meeting at bounded per-replicate barriers, double-float inner products;
 //  - DSMC: a static list of (replicate, cell group) work items so warps of
 //    one launch serve replicates of different K and cell size;
@@ -182,10 +182,9 @@ __device__ __forceinline__ double block_df_total0(DF v, double* sh) {
   return t;
 }
 
-// A replicate's solve is split over a team of T blocks (cg_team_size: one
-// per kTeamNodes nodes, at most kTeamMax), part k owning a contiguous node
-// range. The team meets at bounded barriers on a per-replicate arrival
-// counter (the k-th barrier passes once the counter reaches k T), and its
+// A replicate's solve is split over a team of T blocks (cg_team_size), part k
+// owning a contiguous node range. The team meets at bounded barriers on a
+// per-replicate arrival counter (the k-th barrier passes once the counter reaches k T), and its
 // inner products are the parts' block totals summed by every part in part
 // order, so the iterates do not depend on which block runs which part or
 // on the block size. Thread 0 of each part keeps the FP64 scalars.
@@ -240,7 +239,7 @@ __device__ __forceinline__ double team_total(const BCgArgs& a, int rep, int part
 __device__ void cg_part(const BCgArgs& a, int rep, int part, double* sh, float* fsc, int& stop, int* ok_sh) {
   const BatchRep& B = a.reps[rep];
   const int n = B.f.n, nn = n * n, m = nn * n;
-  const int T = cg_team_size(m);
+  const int T = B.team;
   const int chunk = (m + T - 1) / T;
   const int lo = part * chunk, hi = min(m, lo + chunk);
   const int t0 = threadIdx.x < kCgWidth ? lo + (int)threadIdx.x : INT_MAX;
@@ -1091,7 +1090,7 @@ cudaError_t build_step_items(pic_ctx* c, int cand) {
             for (int64_t i = 0; i < nc; i += T.rhs_nodes) add(ph, r, i, i + T.rhs_nodes < nc ? i + T.rhs_nodes : nc);
             break;
           case BP_CG: {
-            const int T = cg_team_size((int)nc);  // the solve's team: consecutive items
+            const int T = B.team;  // the solve's team: consecutive items
             for (int k = 0; k < T; ++k) add(ph, r, k, T);
             break;
           }

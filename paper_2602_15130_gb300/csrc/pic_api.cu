@@ -1649,8 +1649,17 @@ pic_status pic_create_batch(const pic_config* cfgs, int32_t nrep, void* stream, 
   grab((void**)&c->cg_iters_rep, sizeof(int) * nrep);
   grab((void**)&c->cg_res_rep, sizeof(double) * nrep);
   grab((void**)&c->tt_dev, sizeof(TimeTerms) * (3 * nrep + 1));
+  // the solves' teams: as many blocks as keep two a SM busy
   int n_parts = 0;
-  for (int r = 0; r < nrep; ++r) n_parts += cg_team_size(cfgs[r].n * cfgs[r].n * cfgs[r].n);
+  for (int nodes = kTeamNodesMin;; nodes *= 2) {
+    n_parts = 0;
+    for (int r = 0; r < nrep; ++r) {
+      const int T = cg_team_size(cfgs[r].n * cfgs[r].n * cfgs[r].n, nodes);
+      if (c->reps_host) c->reps_host[r].team = T;
+      n_parts += T;
+    }
+    if (n_parts <= 2 * c->num_sms || nodes >= kTeamNodes) break;
+  }
   c->n_cg_parts = n_parts;
   grab((void**)&c->cg_team_bar, sizeof(unsigned) * nrep);
   grab((void**)&c->cg_team_red, sizeof(double) * (size_t)nrep * 2 * kTeamMax);
@@ -1708,7 +1717,7 @@ pic_status pic_create_batch(const pic_config* cfgs, int32_t nrep, void* stream, 
       int k = 0;
       for (int i = 0; i < nrep; ++i) {
         const int r = order[i];
-        const int T = cg_team_size(cfgs[r].n * cfgs[r].n * cfgs[r].n);
+        const int T = c->reps_host[r].team;
         for (int t = 0; t < T; ++t) parts[k++] = make_int2(r, t);
       }
       e = cudaMemcpy(c->cg_parts, parts, sizeof(int2) * (size_t)c->n_cg_parts, cudaMemcpyHostToDevice);

@@ -1,0 +1,42 @@
+"""The batched Poisson solve at its team sizes: blocks of 1,024 nodes (with
+replicates of one block, of a ragged last block and of the full team), then
+2,048, 8,192 and 16,384 nodes as the replicates fill the SMs.
+
+Sampling is bit-identical, and without collisions nothing else decides, so a
+replicate differs from its single-domain run by the two solves alone: each
+field is within 1e-4 of the exact one (the precision form's stated error),
+hence dv <= steps dt |q/m| 2e-4 max|E| beside the FP32 rounding of v and x."""
+import numpy as np
+import pytest
+
+from paper_2602_15130_gb300 import Batch, Pic, workloads
+
+pytestmark = pytest.mark.gpu
+STEPS = 2
+
+
+@pytest.mark.parametrize("sizes", [[3, 10, 11, 12, 13, 33], [33] * 10 + [12], [33] * 40, [33] * 160],
+                         ids=["1024", "2048", "8192", "16384"])
+def test_batch_fields_match_single_runs_at_every_team_size(sizes):
+    import __graft_entry__ as g
+
+    g.build()
+    cf = [workloads.mixed(workloads.smallest(n=n, n_particles=n ** 3 + 5 * i, K=0, seed=i, dt=0.01))
+          for i, n in enumerate(sizes)]
+    with Batch(cf) as b:
+        b.sample_mms(0.1)
+        b.step(STEPS)
+        its = b.cg_iters()
+        for r in sorted({0, 1, len(cf) // 2, len(cf) - 1} if len(cf) > 20 else range(len(cf))):
+            p = cf[r]
+            with Pic(p) as s:
+                s.sample_mms(0.1)
+                s.step(STEPS)
+                x, v = s.get_state()
+                E = np.abs(s.get_field()[2]).max()
+            xb, vb = b.get_state(r)
+            dv = STEPS * p["dt"] * abs(p["qm"]) * 2e-4 * E + 4 * 2.0 ** -24 * np.abs(v).max()
+            dx = np.abs(xb - x)
+            assert its[r] > 0
+            assert np.abs(vb - v).max() <= dv
+            assert np.minimum(dx, 1.0 - dx).max() <= STEPS * p["dt"] * dv + 4 * 2.0 ** -24
