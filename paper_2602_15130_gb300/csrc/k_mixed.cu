@@ -1341,6 +1341,216 @@ __global__ void __launch_bounds__(kCgThreads) k_cg32(Cg32Args a) {
   }
 }
 
+// The plain CG on one cluster of blocks, for meshes of at most kClusterNodes
+// nodes: the residual that the stencil reads lies in the blocks' shared
+// memory, the other vectors in registers, and the barriers are the cluster's
+// (some 500 SM cycles, against 3,000 to 5,000 through global memory). The same
+// recurrence as k_cg32; den = delta - beta gamma / alpha is formed as
+// delta - beta^2 den_before, and beta with the reciprocal of the old gamma,
+// which a second warp forms during the update: an FP64 division takes 580
+// cycles, and one of three is left on the way. A solve, with its launch, of
+// 8^3, 12^3, 20^3, 31^3 and 40^3 nodes (12, 18, 25, 38 and 47 iterations): 116,
+// 169, 229, 337 and 414 us on the grid, 39, 56, 84, 162 and 268 us here.
+//
+// Blocks: 16 from 2,048 nodes on, fewer below, where the exchange's 16 stores
+// and a wider barrier cost more than the nodes (8^3: 39 us with 4 blocks, 41
+// with 16, 12^3: 55 with 8, 57 with 16, 67 with 2). One node a thread as long
+// as the threads last. With eight (beyond 65,536 nodes; 45^3: 586 us against
+// 460) the grid's SMs are the faster ones.
+constexpr int kClusterBlocks = 16;
+constexpr int kClusterNpt = 4;
+constexpr int64_t kClusterNodes = (int64_t)kClusterBlocks * kCgThreads * kClusterNpt;
+
+__device__ __forceinline__ uint32_t cluster_address(const void* shared, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(shared)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int NPT>
+__global__ void __launch_bounds__(kCgThreads) k_cg32_cluster(Cg32Args a) {
+  __shared__ float rs[NPT * kCgThreads];
+  __shared__ float4 part[2][kClusterBlocks];  // every block's partials, alternating
+  __shared__ float4 sh4[32];
+  __shared__ double shd[2];   // mean of b; then gamma and its reciprocal
+  __shared__ float fscal[2];  // alpha, beta
+  __shared__ int stop;
+  const int n = a.n, nn = n * n, m = (int)a.ncell, t = threadIdx.x, T = blockDim.x, C = gridDim.x;
+  const int chunk = NPT * T, lo = (int)blockIdx.x * chunk;
+  float x[NPT], p[NPT], s[NPT], w[NPT];
+  uint32_t nbr[NPT][6];  // the neighbours' residuals: x+, x-, y+, y-, z+, z-
+  // f(k, slot, id) for every node of the thread
+  auto each = [&](auto f) {
+#pragma unroll
+    for (int k = 0; k < NPT; ++k)
+      if (lo + t + k * T < m) f(k, t + k * T, lo + t + k * T);
+  };
+  auto nbr_sum = [&](int k) {
+    float v[6];
+#pragma unroll
+    for (int e = 0; e < 6; ++e) v[e] = ld_cluster(nbr[k][e]);
+    return v[0] + v[1] + v[2] + v[3] + v[4] + v[5];
+  };
+  // Totals over the cluster of two values a thread, in warp 0; the caller
+  // follows with a __syncthreads. A barrier stands between two calls.
+  int set = 0;
+  auto sum = [&](DF& u, DF& v) {
+    set ^= 1;
+    u = warp_total_df(u);
+    v = warp_total_df(v);
+    if ((t & 31) == 0) sh4[t >> 5] = make_float4(u.hi, u.lo, v.hi, v.lo);
+    __syncthreads();
+    if (t < 32) {
+      const float4 e = t < T / 32 ? sh4[t] : make_float4(0.f, 0.f, 0.f, 0.f);
+      u = warp_total_df(DF{e.x, e.y});
+      v = warp_total_df(DF{e.z, e.w});
+      if (t < C) st_cluster(cluster_address(&part[set][blockIdx.x], (uint32_t)t), make_float4(u.hi, u.lo, v.hi, v.lo));
+    }
+    cluster_barrier();
+    if (t < 32) {
+      const float4 e = t < C ? part[set][t] : make_float4(0.f, 0.f, 0.f, 0.f);
+      u = warp_total_df(DF{e.x, e.y});
+      v = warp_total_df(DF{e.z, e.w});
+    }
+  };
+  each([&](int k, int, int id) {
+    const Nbr q = neighbours(id, n, nn, a.log2n);
+    const int o[6] = {q.xp, q.xm, q.yp, q.ym, q.zp, q.zm};
+#pragma unroll
+    for (int e = 0; e < 6; ++e) nbr[k][e] = cluster_address(rs + o[e] % chunk, (uint32_t)(o[e] / chunk));
+  });
+
+  const float mean_b = (float)(grid_total32(a.rhs_part, a.rhs_blocks, shd) / (double)m);
+  each([&](int k, int l, int id) {
+    x[k] = a.x[id];
+    rs[l] = x[k];
+  });
+  cluster_barrier();
+  DF u{0.f, 0.f}, v{0.f, 0.f};
+  each([&](int k, int, int id) {
+    const float bv = a.b[id] - mean_b;
+    w[k] = bv - (6.f * x[k] - nbr_sum(k)) * a.inv_h2;
+    u = df_fma(u, w[k], w[k]);
+    v = df_fma(v, bv, bv);
+  });
+  sum(u, v);
+  // the scalars below are meaningful in thread 0 only
+  double gamma = df_to_double(u), bb = df_to_double(v), delta = 0.0, beta = 0.0, alpha = 0.0, den = 0.0;
+  const double thresh = a.tol * sqrt(bb), thresh2 = thresh * thresh;
+  const int helper = T > 32 ? 32 : 0;
+  int it = 0, status = 0;
+  each([&](int k, int l, int) { rs[l] = w[k]; });  // the sum's barrier: every block has read x
+  cluster_barrier();
+  for (;;) {
+    // w = A r, (r, r) and (r, w)
+    u = DF{0.f, 0.f};
+    v = DF{0.f, 0.f};
+    each([&](int k, int l, int) {
+      const float rv = rs[l];
+      w[k] = (6.f * rv - nbr_sum(k)) * a.inv_h2;
+      u = df_fma(u, rv, rv);
+      v = df_fma(v, rv, w[k]);
+    });
+    sum(u, v);
+    if (t == 0) {
+      delta = df_to_double(v);
+      if (it > 0) {
+        const double gamma_new = df_to_double(u);
+        beta = gamma_new * shd[1];
+        gamma = gamma_new;
+      }
+      stop = (bb == 0.0 || gamma <= thresh2) ? 1 : (it >= a.maxit ? 2 : 0);
+      if (!stop) {
+        den = it == 0 ? delta : delta - beta * beta * den;
+        alpha = gamma / den;
+        fscal[0] = (float)alpha;
+        fscal[1] = (float)beta;
+        shd[0] = gamma;
+      }
+    }
+    __syncthreads();
+    if (stop == 1) break;
+    if (stop == 2) { status = 1; break; }
+    if (t == helper) shd[1] = 1.0 / shd[0];
+    const float al = fscal[0], be = fscal[1];
+    each([&](int k, int l, int) {
+      const float rv = rs[l];
+      p[k] = it == 0 ? rv : fmaf(be, p[k], rv);
+      s[k] = it == 0 ? w[k] : fmaf(be, s[k], w[k]);
+      x[k] = fmaf(al, p[k], x[k]);
+      rs[l] = fmaf(-al, s[k], rv);
+    });
+    ++it;
+    cluster_barrier();
+  }
+  // zero-mean potential and E
+  u = DF{0.f, 0.f};
+  v = DF{0.f, 0.f};
+  each([&](int k, int, int) { u = df_add_f(u, x[k]); });
+  sum(u, v);
+  if (t == 0) fscal[0] = (float)(df_to_double(u) / (double)m);
+  __syncthreads();
+  const float mean_x = fscal[0];
+  each([&](int k, int l, int id) {
+    const float y = x[k] - mean_x;
+    a.x[id] = y;
+    rs[l] = y;
+  });
+  cluster_barrier();
+  each([&](int k, int, int id) {
+    float v[6];
+#pragma unroll
+    for (int e = 0; e < 6; ++e) v[e] = ld_cluster(nbr[k][e]);
+    a.E4[id] = make_float4(-(v[0] - v[1]) * a.inv_2h, -(v[2] - v[3]) * a.inv_2h, -(v[4] - v[5]) * a.inv_2h, 0.f);
+  });
+  if (blockIdx.x == 0 && t == 0) {
+    a.info[0] = it;
+    a.info[1] = status;
+    if (a.hist) a.hist[0] = it;
+    a.res[0] = bb > 0.0 ? sqrt(gamma) / sqrt(bb) : 0.0;
+    if (status) atomicOr(a.flags, 2);
+    atomicMax(a.flags + 1, it);
+  }
+  cluster_barrier();  // no block leaves while another reads its shared memory
+}
+
+cudaError_t launch_cg32_cluster(const Cg32Args& args, cudaStream_t stream) {
+  Cg32Args a = args;
+  const int C = a.ncell <= 1024 ? 4 : a.ncell <= 2048 ? 8 : kClusterBlocks;
+  const int per = (int)((a.ncell + C - 1) / C);
+  const int npt = per <= kCgThreads ? 1 : per <= 2 * kCgThreads ? 2 : 4;
+  const void* fn = npt == 1   ? (const void*)k_cg32_cluster<1>
+                   : npt == 2 ? (const void*)k_cg32_cluster<2>
+                              : (const void*)k_cg32_cluster<4>;
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)C);
+  cfg.blockDim = dim3((unsigned)(((per + npt - 1) / npt + 31) / 32 * 32));
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  void* argv[] = {&a};
+  return cudaLaunchKernelExC(&cfg, fn, argv);
+}
+
 // ------------------------------------------- multigrid-preconditioned CG --
 // The precision form's Poisson solve on meshes of 2^k >= 16 nodes per edge:
 // CG preconditioned by one multigrid V-cycle (the same discrete system
@@ -2058,6 +2268,15 @@ cudaError_t launch_cg32(pic_ctx* c) {
   a.skip_block = c->stall_next_cg ? c->cg_grid - 1 : -1;
   a.hist = c->hist_row;
   c->stall_next_cg = false;
+  if (c->mg_nlev == 0 && a.ncell <= kClusterNodes && a.skip_block < 0) {
+    // (a failure injection takes the grid, whose waits are bounded)
+    prof_begin(c);
+    const cudaError_t e = launch_cg32_cluster(a, c->stream);
+    if (e != cudaSuccess) return e;
+    prof_end(c, KC_CG);
+    c->launches++;
+    return cudaSuccess;
+  }
   cudaError_t e = cudaMemsetAsync(c->cg_bar, 0, 2 * sizeof(unsigned int), c->stream);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(c->cg_info, 0, 3 * sizeof(int), c->stream);
