@@ -651,6 +651,17 @@ __global__ void __launch_bounds__(kDsmcThreads, 16) k_dsmc(DsmcArgs a) {
 //   v += 1/2 (dt q/m (E_p - E^M_p) + dv + dt vdot^M) (vdot^M = 0 for the
 //   Gaussian f_v, vh'(t) tau for the paper's f_v),
 //   x += dt (v + xdot^M - v^M) at t_half (drift), wrapped; new cell key.
+//
+// What bounds it is the FP64 pipe (an instruction of a warp takes the SM's 19
+// cycles), so operations are what counts: sin and cos from a table and the
+// angle's remainder (15, sincospi 22 and a reduction); the drift's xdot^M from
+// a table of its one transcendental quantity, dG^{-1}/dT (xm_solve and xm_dot:
+// a Hermite start, a Newton step with its sincospi, three divisions: 90);
+// uniforms, cells and table indexes read off the bits of a sum with 2^52
+// (a conversion takes the pipe like an addition). Per particle some 110
+// FP64 instructions instead of 150 for the Lorentz term, 70 instead of 310
+// for the drift. Two steps of 64^3 cells of 32 (a closing kick, one with
+// drift): 9.2 ms before, 4.6 now.
 // --------------------------------------------------------------------------
 struct KickArgs {
   Params P;
@@ -661,37 +672,100 @@ struct KickArgs {
   const double *E0, *E1, *E2;
   double *L0, *L1, *L2;  // Lorentz term dt q/m (E_p - E^M_p)
   int lor_mode;          // 0: compute, 1: compute and store, 2: load
+  double dt_qm;
   TimeTerms tE, th;
   TimeTerms t0, t1;      // t_n, t_{n+1} for the isolated-collision drift
   int drift;
+  // the drift by table: T = 1.m - T0 with 1.m = xi + 1 - 2^-53, and
+  // xdot^M = c - xslope dG^{-1}/dT(T)
+  double T0, xslope;
   int32_t *key, *rank, *count;
 };
 
-__device__ __forceinline__ void gather_E(const Params& P, const double* E0, const double* E1, const double* E2,
-                                         double x, double y, double z, double* e) {
+constexpr double kRound52 = 0x1.8p52;  // adding it rounds to an integer, in the low word
+
+// exponent of |x|, as in the high word of 2^e
+__device__ __forceinline__ bool below_pow2(double x, int e) {
+  return (__double2hiint(x) & 0x7fffffff) < (1023 + e) << 20;
+}
+__device__ __noinline__ void sincos_far(double d, double* s, double* c) { sincospi(2.0 * d, s, c); }
+
+// sin and cos of 2 pi d: the table at the nearest kTrigM-th of
+// a turn, and the remainder b, |b| <= pi / kTrigM, by Taylor's series (the
+// first terms left out are b^7/5040 = 8e-18 and b^8/40320)
+__device__ __forceinline__ void sincos_turn(const double2* tab, double d, double* s, double* c) {
+  constexpr double w = kTwoPi / kTrigM, w2 = w * w;
+  if (!below_pow2(d, 40)) return sincos_far(d, s, c);  // (or not finite)
+  const double z = fma(d, (double)kTrigM, kRound52);
+  const double2 t = __ldg(tab + (__double2loint(z) & (kTrigM - 1)));
+  const double u = fma(d, (double)kTrigM, kRound52 - z);
+  const double u2 = u * u;
+  const double sb = u * fma(u2, fma(u2, w * w2 * w2 / 120.0, -w * w2 / 6.0), w);
+  const double cb = u2 * fma(u2, fma(u2, -w2 * w2 * w2 / 720.0, w2 * w2 / 24.0), -0.5 * w2);  // cos - 1
+  *s = fma(t.y, sb, fma(t.x, cb, t.x));
+  *c = fma(-t.x, sb, fma(t.y, cb, t.y));
+}
+
+// cell_coord(x, n) without conversions where x lies in the box; xn = x n
+// rounded, *whole the coordinate in FP64
+__device__ __forceinline__ int cell_coord_fast(double x, double xn, int n, double* whole) {
+  const double z = __dadd_rd(xn, kRound52);
+  int i = __double2loint(z);
+  *whole = __dsub_rn(z, kRound52);
+  if ((unsigned)i >= (unsigned)n || !below_pow2(xn, 31)) {
+    i = cell_coord(x, n);
+    *whole = (double)i;
+  }
+  return i;
+}
+
+// dt q/m (E_p + E_app - E^M) at a particle
+__device__ __forceinline__ void lorentz64(const KickArgs& a, const double* x, double* L) {
+  const Params& P = a.P;
   const int n = P.n;
-  const double un = x * (double)n, vn = y * (double)n, wn = z * (double)n;
-  const int i = cell_coord(x, n), j = cell_coord(y, n), k = cell_coord(z, n);
-  const double fx = un - (double)i, fy = vn - (double)j, fz = wn - (double)k;
-  const int i1 = i + 1 == n ? 0 : i + 1, j1 = j + 1 == n ? 0 : j + 1, k1 = k + 1 == n ? 0 : k + 1;
-  const double wx[2] = {1.0 - fx, fx}, wy[2] = {1.0 - fy, fy}, wz[2] = {1.0 - fz, fz};
-  const int ii[2] = {i, i1}, jj[2] = {j, j1}, kk[2] = {k, k1};
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+  double w1[3], w0[3];
+  int i0[3], i1[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double xn = __dmul_rn(x[d], (double)n);
+    double whole;
+    i0[d] = cell_coord_fast(x[d], xn, n, &whole);
+    i1[d] = i0[d] + 1 == n ? 0 : i0[d] + 1;
+    w1[d] = xn - whole;
+    w0[d] = 1.0 - w1[d];
+  }
+  double e0 = P.E_app[0], e1 = P.E_app[1], e2 = P.E_app[2];
 #pragma unroll
   for (int c = 0; c < 2; ++c)
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < 2; ++b) {
+      const double wyz = (b ? w1[1] : w0[1]) * (c ? w1[2] : w0[2]);
+      const int64_t row = (int64_t)n * ((b ? i1[1] : i0[1]) + (int64_t)n * (c ? i1[2] : i0[2]));
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const int64_t node = ii[a] + (int64_t)n * (jj[b] + (int64_t)n * kk[c]);
-        const double ww = wx[a] * wy[b] * wz[c];
-        a0 += ww * __ldg(E0 + node);
-        a1 += ww * __ldg(E1 + node);
-        a2 += ww * __ldg(E2 + node);
+      for (int q = 0; q < 2; ++q) {
+        const int64_t node = row + (q ? i1[0] : i0[0]);
+        const double w = (q ? w1[0] : w0[0]) * wyz;
+        e0 = fma(w, __ldg(a.E0 + node), e0);
+        e1 = fma(w, __ldg(a.E1 + node), e1);
+        e2 = fma(w, __ldg(a.E2 + node), e2);
       }
-  e[0] = a0; e[1] = a1; e[2] = a2;
+    }
+  // E^M = -amp (c0 s1 s2, s0 c1 s2, s0 s1 c2)
+  const double2* tab =
+      reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1) + kR64Doubles + 8 * kSlopeM);
+  double s0, c0, s1, c1, s2, c2;
+  sincos_turn(tab, x[0] - P.phi_shift[0], &s0, &c0);
+  sincos_turn(tab, x[1] - P.phi_shift[1], &s1, &c1);
+  sincos_turn(tab, x[2] - P.phi_shift[2], &s2, &c2);
+  const double as0 = a.tE.em_amp * s0;
+  L[0] = a.dt_qm * fma(a.tE.em_amp * c0, s1 * s2, e0);
+  L[1] = a.dt_qm * fma(as0 * c1, s2, e1);
+  L[2] = a.dt_qm * fma(as0 * s1, c2, e2);
 }
 
+// kTable: the Gaussian f_v's drift by table; otherwise the paper's problem,
+// the isolated-collision drift of Sec. 5.4 and an f_x too sharp for the table.
+template <bool kTable>
 __global__ void __launch_bounds__(kThreads) k_kick(KickArgs a) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const Params& P = a.P;
@@ -702,54 +776,67 @@ __global__ void __launch_bounds__(kThreads) k_kick(KickArgs a) {
   if (a.lor_mode == 2) {
     L[0] = a.L0[j]; L[1] = a.L1[j]; L[2] = a.L2[j];
   } else {
-    double Ep[3], EM[3];
-    gather_E(P, a.E0, a.E1, a.E2, x[0], x[1], x[2], Ep);
-    e_manufactured(P, a.tE, x[0], x[1], x[2], &EM[0], &EM[1], &EM[2]);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) L[d] = P.dt * P.qm_eff * (Ep[d] + P.E_app[d] - EM[d]);
+    lorentz64(a, x, L);
     if (a.lor_mode == 1) {
       a.L0[j] = L[0]; a.L1[j] = L[1]; a.L2[j] = L[2];
     }
   }
-  double dv[3] = {0.0, 0.0, 0.0};
-  if (a.dv0) { dv[0] = a.dv0[j]; dv[1] = a.dv1[j]; dv[2] = a.dv2[j]; }
-  const bool paper = P.dist == PIC_DIST_PAPER;
+  const bool paper = !kTable && P.dist == PIC_DIST_PAPER;
   double vm[3] = {0.0, 0.0, 0.0};
   if (a.drift || paper) { vm[0] = a.vm0[j]; vm[1] = a.vm1[j]; vm[2] = a.vm2[j]; }
+  if (a.dv0) { L[0] += a.dv0[j]; L[1] += a.dv1[j]; L[2] += a.dv2[j]; }
   if (paper) {
     // v^M arrays hold tau: vdot^M(t) = vh'(t) tau (Eq. velocity_verlet)
 #pragma unroll
-    for (int d = 0; d < 3; ++d) v[d] = v[d] + 0.5 * ((L[d] + dv[d]) + P.dt * (vm[d] * a.tE.dvh[d]));
-  } else {
-#pragma unroll
-    for (int d = 0; d < 3; ++d) v[d] = v[d] + 0.5 * (L[d] + dv[d]);
+    for (int d = 0; d < 3; ++d) L[d] += P.dt * (vm[d] * a.tE.dvh[d]);
   }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) v[d] = fma(0.5, L[d], v[d]);
   a.v0[j] = v[0]; a.v1[j] = v[1]; a.v2[j] = v[2];
   if (!a.drift) return;
   const uint64_t p = a.pid[j];
   const U4 b0 = sample_block(P, p, 0), b1 = sample_block(P, p, 1);
-  const double xi[3] = {unif52(b0.x, b0.y), unif52(b0.z, b0.w), unif52(b1.x, b1.y)};
+  const uint32_t hi[3] = {b0.x, b0.z, b1.x}, lw[3] = {b0.y, b0.w, b1.y};
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    double s;
-    if (paper) {
-      double c;
-      xm_solve_gen(a.th, d, xi[d], &s, &c);
-      const double xd = xm_dot_gen(a.th, d, s, c);
-      x[d] = wrap_unit(x[d] + P.dt * (v[d] + xd - vm[d] * a.th.vh[d]));
-    } else if (P.verify & PIC_VERIFY_ISOLATE) {
-      // exact manufactured increment x^M(t_{n+1}) - x^M(t_n) (Sec. 5.4)
-      const double dxm = xm_solve(P, a.t1, xi[d], &s) - xm_solve(P, a.t0, xi[d], &s);
-      x[d] = wrap_unit(x[d] + (P.dt * (v[d] - vm[d]) + dxm));
+    if constexpr (kTable) {
+      // unif52's 52 bits as the mantissa of a number in [1, 2)
+      const double m = __hiloint2double((int)(0x3ff00000u | hi[d] >> 12), (int)(hi[d] << 20 | lw[d] >> 12));
+      const double T = m - a.T0;
+      const double z = fma(T, (double)kSlopeM, kRound52);
+      const double u = fma(T, (double)kSlopeM, kRound52 - z);
+      const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1) + kR64Doubles) +
+                         4 * (__double2loint(z) & (kSlopeM - 1));
+      const double2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
+      const double g =
+          fma(fma(fma(fma(fma(fma(fma(q3.y, u, q3.x), u, q2.y), u, q2.x), u, q1.y), u, q1.x), u, q0.y), u, q0.x);
+      x[d] = wrap_unit(fma(P.dt, (v[d] - vm[d]) + fma(-a.xslope, g, P.fx_speed), x[d]));
     } else {
-      xm_solve(P, a.th, xi[d], &s);
-      const double xd = xm_dot(P, a.th, s);
-      x[d] = wrap_unit(x[d] + P.dt * (v[d] + xd - vm[d]));
+      const double xi = unif52(hi[d], lw[d]);
+      double s;
+      if (paper) {
+        double c;
+        xm_solve_gen(a.th, d, xi, &s, &c);
+        const double xd = xm_dot_gen(a.th, d, s, c);
+        x[d] = wrap_unit(x[d] + P.dt * (v[d] + xd - vm[d] * a.th.vh[d]));
+      } else if (P.verify & PIC_VERIFY_ISOLATE) {
+        // exact manufactured increment x^M(t_{n+1}) - x^M(t_n) (Sec. 5.4)
+        const double dxm = xm_solve(P, a.t1, xi, &s) - xm_solve(P, a.t0, xi, &s);
+        x[d] = wrap_unit(x[d] + (P.dt * (v[d] - vm[d]) + dxm));
+      } else {
+        xm_solve(P, a.th, xi, &s);
+        const double xd = xm_dot(P, a.th, s);
+        x[d] = wrap_unit(x[d] + P.dt * (v[d] + xd - vm[d]));
+      }
     }
   }
   a.x0[j] = x[0]; a.x1[j] = x[1]; a.x2[j] = x[2];
   const int n = P.n;
-  const int32_t k = cell_coord(x[0], n) + n * (cell_coord(x[1], n) + n * cell_coord(x[2], n));
+  double whole;
+  int ci[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) ci[d] = cell_coord_fast(x[d], __dmul_rn(x[d], (double)n), n, &whole);
+  const int32_t k = ci[0] + n * (ci[1] + n * ci[2]);
   a.key[j] = k;
   a.rank[j] = cell_slot(a.count, k);
 }
@@ -1010,11 +1097,19 @@ cudaError_t launch_kick(pic_ctx* c, double tE, bool with_coll, bool drift, doubl
   a.t0 = time_terms(c->P, tE);
   a.t1 = time_terms(c->P, tn1);
   a.drift = drift ? 1 : 0;
+  const Params& P = c->P;
+  a.dt_qm = P.dt * P.qm_eff;
+  a.T0 = (1.0 - 0x1p-53) + (a.th.ct + P.fx_amp_over_2pi * a.th.cos2ct);
+  // A c (S + s) / (1 + A S) with s = sin(2 pi c t) is c - c (1 - A s) / (1 + A S)
+  a.xslope = P.fx_speed * (1.0 - P.fx_amp * a.th.sin2ct);
   a.key = c->key;
   a.rank = c->rank;
   a.count = c->count;
+  const bool table = P.dist == PIC_DIST_CONFIG && !(P.verify & PIC_VERIFY_ISOLATE) && c->slope_table &&
+                     fabs(a.T0) < 0x1p30;  // (beyond, T has no digits left to look up)
   prof_begin(c);
-  k_kick<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(a);
+  if (table) k_kick<true><<<blocks_for(P.np), kThreads, 0, c->stream>>>(a);
+  else k_kick<false><<<blocks_for(P.np), kThreads, 0, c->stream>>>(a);
   prof_end(c, KC_KICK);
   c->launches++;
   c->lor_valid = !drift;

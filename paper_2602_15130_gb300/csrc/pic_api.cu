@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <memory>
+#include <utility>
 #include <new>
 
 #include "pic_internal.cuh"
@@ -178,6 +179,50 @@ void hs_R64_table(double* out) {
     }
     for (int j = 0; j < kN; ++j) out[kN * k + j] = (double)c[j];
   }
+}
+
+// FP64 tables of the kick. dG^{-1}/dT = 1 / (1 + A sin(2 pi G^{-1}(T))) around
+// every knot T_k by its Taylor polynomial in u = kSlopeM T - k, |u| <= 1/2,
+// from the recurrences of g = y', S = sin(2 pi y) and C = cos(2 pi y):
+// S' = 2 pi C g, C' = -2 pi S g, (1 + A S) g = 1. Returns whether the first
+// term left out stays below rounding everywhere (A = 0.3: 4e-18; from
+// |A| = 0.6 on G^{-1} bends too sharply). Behind it sin and cos of
+// 2 pi k / kTrigM, from the first octant's.
+bool kick_tables(double A, const double* ginv, double* out) {
+  constexpr int kN = 9;
+  double worst = 0.0;
+  for (int k = 0; k < kSlopeM; ++k) {
+    double g[kN], S[kN + 1], C[kN + 1];
+    const double y = ginv[2 * (k * (kGinvM / kSlopeM))];
+    S[0] = sin(2.0 * kPi * y);
+    C[0] = cos(2.0 * kPi * y);
+    const double d0 = 1.0 / (1.0 + A * S[0]);
+    for (int j = 0; j < kN; ++j) {
+      double q = j == 0 ? 1.0 : 0.0;
+      for (int i = 1; i <= j; ++i) q -= A * S[i] * g[j - i];
+      g[j] = q * d0;
+      double ds = 0.0, dc = 0.0;
+      for (int i = 0; i <= j; ++i) {
+        ds += C[i] * g[j - i];
+        dc -= S[i] * g[j - i];
+      }
+      S[j + 1] = 2.0 * kPi / (j + 1) * ds;
+      C[j + 1] = 2.0 * kPi / (j + 1) * dc;
+    }
+    double scale = 1.0;
+    for (int j = 0; j < 8; ++j, scale /= kSlopeM) out[8 * k + j] = g[j] * scale;
+    worst = fmax(worst, fabs(g[8] * scale) / 256.0);
+  }
+  double* t = out + 8 * kSlopeM;
+  for (int k = 0; k < kTrigM; ++k) {
+    const int quarter = kTrigM / 4, q = k / quarter, r = k % quarter;
+    const int f = r <= quarter / 2 ? r : quarter - r;  // folded to the octant
+    double s = sin(2.0 * kPi * f / kTrigM), c = cos(2.0 * kPi * f / kTrigM);
+    if (f != r) std::swap(s, c);
+    t[2 * k] = q == 0 ? s : q == 1 ? c : q == 2 ? -s : -c;
+    t[2 * k + 1] = q == 0 ? c : q == 1 ? -s : q == 2 ? -c : s;
+  }
+  return worst <= 0x1p-55;
 }
 
 // FP32 tables of the precision form: the knots of G^{-1} (y_k, dy/dT) and
@@ -414,7 +459,7 @@ void for_each_buffer(pic_ctx* c, F f) {
   f((void**)&c->flags, 64);
   f((void**)&c->err_part, (size_t)c->err_blocks * 14 * 8);
   f((void**)&c->err_out, 14 * 8);
-  f((void**)&c->ginv, ((size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles)) * 8);
+  f((void**)&c->ginv, ((size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles + kKickDoubles)) * 8);
   f((void**)&c->ginv_f, (size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4);
   if (c->nrep == 0 && (c->cfg.verify & PIC_VERIFY_ANGLES)) {
     f((void**)&c->ang_hist, (size_t)2 * PIC_ANGLE_BINS * 8);
@@ -1003,7 +1048,7 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     return PIC_ENOMEM;
   }
   {
-    const size_t tab_doubles = (size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles);
+    const size_t tab_doubles = (size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles + kKickDoubles);
     double* tab = (double*)malloc(tab_doubles * 8);
     float* tabf = (float*)malloc((size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4);
     if (!tab || !tabf) {
@@ -1022,6 +1067,7 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
         return t;
       }();
       memcpy(tab + (kGinvM + 1) * 2, r64.get(), sizeof(double) * kR64Doubles);
+      c->slope_table = kick_tables(c->cfg.fx_amp, tab, tab + (kGinvM + 1) * 2 + kR64Doubles);
     }
     e = cudaMemcpy(c->ginv, tab, tab_doubles * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->ginv_f, tabf, (size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4,

@@ -25,6 +25,10 @@ constexpr float kRTabAmax = 8.f;
 // degree 7 a unit of u, behind the FP64 G^{-1} knots
 constexpr int kR64Max = 64, kR64PerUnit = 8;
 constexpr int kR64Doubles = 8 * kR64Max * kR64PerUnit;
+// FP64 tables of the kick, behind that one: dG^{-1}/dT as kSlopeM polynomials
+// of degree 7 a period, and (sin, cos) of 2 pi k / kTrigM
+constexpr int kSlopeM = 512, kTrigM = 256;
+constexpr int kKickDoubles = 8 * kSlopeM + 2 * kTrigM;
 
 // ---------------------------------------------------------------------------
 // Everything a kernel needs to know about the problem, passed by value.
@@ -618,6 +622,7 @@ struct pic_ctx {
 
   double* dv[3];    // collision term per particle (sorted order)
   double* lor[3];   // dt q/m (E_p - E^M_p) of the last kick without drift
+  bool slope_table;  // the drift's table of dG^{-1}/dT is exact to rounding
   bool lor_valid;   // lor matches the current order, positions and field
   // precision form: v^M (tau for the paper's f_v) by pid, written with the
   // context's first state
