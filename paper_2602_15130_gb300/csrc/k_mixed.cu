@@ -673,6 +673,80 @@ __host__ __device__ constexpr size_t dsmc32_smem_words(int bm_words) {
   return (size_t)32 * bm_words + (size_t)kList * 32 * 4 + 32;
 }
 
+// Add to acc what the outcomes of the set bits, lanes of the warp whose lists
+// are given, have changed of particle jj, in ascending order.
+__device__ __forceinline__ void add_changes(uint32_t mine, int jj, const float4* wlist, const int* wlen,
+                                            const float* wov, int max_ppc, float w0, float w1, float w2,
+                                            float* acc) {
+  while (mine) {
+    const int L = __ffs(mine) - 1;
+    mine &= mine - 1u;
+    // lane L's working velocity of particle jj: its list, else its overlay
+    const int k = wl_find(wlist + L, wlen[L], jj);
+    float W0, W1, W2;
+    if (k >= 0) {
+      const float4 e = wlist[32 * k + L];
+      W0 = e.x; W1 = e.y; W2 = e.z;
+    } else {
+      const float* W = wov + ((size_t)L * max_ppc + jj) * 3;
+      W0 = W[0]; W1 = W[1]; W2 = W[2];
+    }
+    acc[0] += W0 - w0;
+    acc[1] += W1 - w1;
+    acc[2] += W2 - w2;
+  }
+}
+
+// The averages of particle j of a cell of cc, from its summed changes.
+__device__ __forceinline__ void dsmc_finish32(const Dsmc32Args& a, int32_t j, int cc, float w0, float w1, float w2,
+                                              const float* acc, float invK) {
+  const ParamsF& P = a.P;
+  // analytic <Delta v^M> (hard spheres: f m with m = mu - v)
+  float sm[3];
+  if (P.n_sigma == 0) {
+    const float mx = P.vmean[0] - w0, my = P.vmean[1] - w1, mz = P.vmean[2] - w2;
+    const float am = sqrtf(fmaf(mx, mx, fmaf(my, my, mz * mz))) * P.inv_vsig;
+    const float f = P.src_pref * (float)(cc - 1) * P.vsig * hs_R_f(P, am);
+    sm[0] = f * mx; sm[1] = f * my; sm[2] = f * mz;
+  } else {
+    odd_source_f(P, a.vh, w0, w1, w2, cc, sm);
+  }
+  if (a.m0 != nullptr) {
+    a.dv0[j] = acc[0] * invK; a.dv1[j] = acc[1] * invK; a.dv2[j] = acc[2] * invK;
+    a.m0[j] = sm[0]; a.m1[j] = sm[1]; a.m2[j] = sm[2];
+  } else {
+    // inside a step: the velocity with this call's half kick of
+    // Eq. velocity_verlet applied, v + (<dv> - <dv^M>)/2, so that
+    // the kick that follows reads one array instead of two
+    a.dv0[j] = fmaf(0.5f, fmaf(acc[0], invK, -sm[0]), w0);
+    a.dv1[j] = fmaf(0.5f, fmaf(acc[1], invK, -sm[1]), w1);
+    a.dv2[j] = fmaf(0.5f, fmaf(acc[2], invK, -sm[2]), w2);
+  }
+}
+
+// the warp's counts onto the context's and the step's
+__device__ __forceinline__ void add_counts(const Dsmc32Args& a, Counts32 cnt, int lane) {
+  for (int off = 16; off > 0; off >>= 1) {
+    cnt.cand += __shfl_down_sync(0xffffffffu, cnt.cand, off);
+    cnt.coll += __shfl_down_sync(0xffffffffu, cnt.coll, off);
+    cnt.gmax += __shfl_down_sync(0xffffffffu, cnt.gmax, off);
+    cnt.tie += __shfl_down_sync(0xffffffffu, cnt.tie, off);
+    cnt.ftie += __shfl_down_sync(0xffffffffu, cnt.ftie, off);
+  }
+  if (lane == 0) {
+    if (cnt.cand) atomicAdd(a.counters + 0, cnt.cand);
+    if (cnt.coll) atomicAdd(a.counters + 1, cnt.coll);
+    if (cnt.gmax) atomicAdd(a.counters + 2, cnt.gmax);
+    if (cnt.tie) atomicAdd(a.counters + 3, cnt.tie);
+    if (cnt.ftie) atomicAdd(a.counters + 4, cnt.ftie);
+    if (a.hist) {
+      if (cnt.cand) atomicAdd((unsigned long long*)a.hist + 1, cnt.cand);
+      if (cnt.coll) atomicAdd((unsigned long long*)a.hist + 2, cnt.coll);
+      if (cnt.gmax) atomicAdd((unsigned long long*)a.hist + 3, cnt.gmax);
+    }
+  }
+}
+
 template <bool kVerify>
 __global__ void __launch_bounds__(kDsmcThreads, 6) k_dsmc32(Dsmc32Args a) {
   extern __shared__ uint32_t smem[];
@@ -692,10 +766,7 @@ __global__ void __launch_bounds__(kDsmcThreads, 6) k_dsmc32(Dsmc32Args a) {
   for (int i = 0; i < a.bm_words; ++i) bm[i] = 0u;
   __syncwarp();
   Counts32 cnt = {0, 0, 0, 0, 0};
-  const bool separate = a.m0 != nullptr;
   const float invK = 1.f / (float)P.K;
-  const float mu0 = P.vmean[0], mu1 = P.vmean[1], mu2 = P.vmean[2];
-  const float vs = P.vsig, ivs = P.inv_vsig, pref = P.src_pref;
 
   int64_t gbase = 0;
   int gk = a.chunk;
@@ -750,49 +821,13 @@ __global__ void __launch_bounds__(kDsmcThreads, 6) k_dsmc32(Dsmc32Args a) {
           uint32_t mine = tw & (kseg << (cl * a.Kc));
           const int32_t j = cs + jj;
           const float w0 = a.v0[j], w1 = a.v1[j], w2 = a.v2[j];
-          float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f;
-          if (ch > 0) { acc0 = a.dv0[j]; acc1 = a.dv1[j]; acc2 = a.dv2[j]; }
-          while (mine) {
-            const int L = __ffs(mine) - 1;
-            mine &= mine - 1u;
-            // lane L's working velocity of particle jj: its list, else its overlay
-            const int k = wl_find(wlist + L, wlen[L], jj);
-            float W0, W1, W2;
-            if (k >= 0) {
-              const float4 e = wlist[32 * k + L];
-              W0 = e.x; W1 = e.y; W2 = e.z;
-            } else {
-              const float* W = wov + ((size_t)L * a.max_ppc + jj) * 3;
-              W0 = W[0]; W1 = W[1]; W2 = W[2];
-            }
-            acc0 += W0 - w0;
-            acc1 += W1 - w1;
-            acc2 += W2 - w2;
-          }
+          float acc[3] = {0.f, 0.f, 0.f};
+          if (ch > 0) { acc[0] = a.dv0[j]; acc[1] = a.dv1[j]; acc[2] = a.dv2[j]; }
+          add_changes(mine, jj, wlist, wlen, wov, a.max_ppc, w0, w1, w2, acc);
           if (!last) {
-            a.dv0[j] = acc0; a.dv1[j] = acc1; a.dv2[j] = acc2;
+            a.dv0[j] = acc[0]; a.dv1[j] = acc[1]; a.dv2[j] = acc[2];
           } else {
-            // analytic <Delta v^M> (hard spheres: f m with m = mu - v)
-            float sm[3];
-            if (P.n_sigma == 0) {
-              const float mx = mu0 - w0, my = mu1 - w1, mz = mu2 - w2;
-              const float am = sqrtf(fmaf(mx, mx, fmaf(my, my, mz * mz))) * ivs;
-              const float f = pref * (float)(cc - 1) * vs * hs_R_f(P, am);
-              sm[0] = f * mx; sm[1] = f * my; sm[2] = f * mz;
-            } else {
-              odd_source_f(P, a.vh, w0, w1, w2, cc, sm);
-            }
-            if (separate) {
-              a.dv0[j] = acc0 * invK; a.dv1[j] = acc1 * invK; a.dv2[j] = acc2 * invK;
-              a.m0[j] = sm[0]; a.m1[j] = sm[1]; a.m2[j] = sm[2];
-            } else {
-              // inside a step: the velocity with this call's half kick of
-              // Eq. velocity_verlet applied, v + (<dv> - <dv^M>)/2, so that
-              // the kick that follows reads one array instead of two
-              a.dv0[j] = fmaf(0.5f, fmaf(acc0, invK, -sm[0]), w0);
-              a.dv1[j] = fmaf(0.5f, fmaf(acc1, invK, -sm[1]), w1);
-              a.dv2[j] = fmaf(0.5f, fmaf(acc2, invK, -sm[2]), w2);
-            }
+            dsmc_finish32(a, j, cc, w0, w1, w2, acc, invK);
           }
         }
       }
@@ -802,25 +837,82 @@ __global__ void __launch_bounds__(kDsmcThreads, 6) k_dsmc32(Dsmc32Args a) {
       __syncwarp();
     }
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    cnt.cand += __shfl_down_sync(0xffffffffu, cnt.cand, off);
-    cnt.coll += __shfl_down_sync(0xffffffffu, cnt.coll, off);
-    cnt.gmax += __shfl_down_sync(0xffffffffu, cnt.gmax, off);
-    cnt.tie += __shfl_down_sync(0xffffffffu, cnt.tie, off);
-    cnt.ftie += __shfl_down_sync(0xffffffffu, cnt.ftie, off);
-  }
-  if (lane == 0) {
-    if (cnt.cand) atomicAdd(a.counters + 0, cnt.cand);
-    if (cnt.coll) atomicAdd(a.counters + 1, cnt.coll);
-    if (cnt.gmax) atomicAdd(a.counters + 2, cnt.gmax);
-    if (cnt.tie) atomicAdd(a.counters + 3, cnt.tie);
-    if (cnt.ftie) atomicAdd(a.counters + 4, cnt.ftie);
-    if (a.hist) {
-      if (cnt.cand) atomicAdd((unsigned long long*)a.hist + 1, cnt.cand);
-      if (cnt.coll) atomicAdd((unsigned long long*)a.hist + 2, cnt.coll);
-      if (cnt.gmax) atomicAdd((unsigned long long*)a.hist + 3, cnt.gmax);
+  add_counts(a, cnt, lane);
+}
+
+// The same with the warps of a block sharing a cell, for several chunks of
+// outcomes: the two or four warps take a chunk each, and then, with the
+// chunks' lists side by side in shared memory, every second or fourth word of
+// 32 particles, whose changes they add chunk by chunk in the same ascending
+// order (bit for bit the sums of k_dsmc32). What bounded the launches it is
+// for was the chain of a cell's chunks in one warp: 12^3 cells of 101, K = 243,
+// 11 warps an SM and a last wave of stragglers, 342 us a call, 134 now.
+template <bool kVerify, int kWarps>
+__global__ void __launch_bounds__(32 * kWarps, 24 / kWarps) k_dsmc32_team(Dsmc32Args a) {
+  extern __shared__ uint32_t smem[];
+  __shared__ unsigned long long next;
+  const ParamsF& P = a.P;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const size_t words = dsmc32_smem_words(a.bm_words);
+  uint32_t* bm = smem + wib * words + (size_t)lane * a.bm_words;
+  float4* wl = reinterpret_cast<float4*>(smem + wib * words + 32 * a.bm_words) + lane;
+  const size_t wov_words = (size_t)32 * a.max_ppc * 3;
+  const float* block_ov = a.overlay + (size_t)blockIdx.x * kWarps * wov_words;
+  float* ov = a.overlay + ((size_t)blockIdx.x * kWarps + wib) * wov_words + (size_t)lane * a.max_ppc * 3;
+  for (int i = 0; i < a.bm_words; ++i) bm[i] = 0u;
+  Counts32 cnt = {0, 0, 0, 0, 0};
+  const float invK = 1.f / (float)P.K;
+  for (;;) {
+    if (threadIdx.x == 0) next = atomicAdd(a.queue, 1ull);
+    __syncthreads();
+    const int64_t cell = (int64_t)next;
+    if (cell >= a.ngroups) break;  // block-uniform
+    const int32_t s = a.start[cell], c = a.start[cell + 1] - s;
+    const int wmax = (c + 31) / 32;
+    const bool fits = c <= a.max_ppc;
+    if (!fits && threadIdx.x == 0) atomicOr(a.flags, 1);
+    for (int ch0 = 0; ch0 < a.nchunks; ch0 += kWarps) {
+      const int ch = ch0 + wib;
+      const int o = ch * 32 + lane;
+      const bool run = ch < a.nchunks && o < P.K && c >= 2 && fits;
+      int t = 0;
+      if (run)
+        ntc_outcome_f<kVerify>(P, a.c0, (uint32_t)cell, (uint32_t)o, c, a.v0 + s, a.v1 + s, a.v2 + s, bm, wl, t, ov,
+                               cnt, a.lg);
+      reinterpret_cast<int*>(smem + wib * words + 32 * a.bm_words + kList * 128)[lane] = t;
+      __syncthreads();
+      const bool last = ch0 + kWarps >= a.nchunks;
+      for (int w = wib; w < wmax; w += kWarps) {
+        const int jj = 32 * w + lane;
+        const int32_t j = s + jj;
+        const bool there = jj < c;
+        float w0 = 0.f, w1 = 0.f, w2 = 0.f, acc[3] = {0.f, 0.f, 0.f};
+        if (there) {
+          w0 = a.v0[j]; w1 = a.v1[j]; w2 = a.v2[j];
+          if (ch0 > 0) { acc[0] = a.dv0[j]; acc[1] = a.dv1[j]; acc[2] = a.dv2[j]; }
+        }
+        for (int k = 0; k < kWarps && ch0 + k < a.nchunks; ++k) {
+          const uint32_t* wk = smem + k * words;
+          const uint32_t tw = warp_transpose32(w < a.bm_words ? wk[(size_t)lane * a.bm_words + w] : 0u, lane);
+          const float4* lists = reinterpret_cast<const float4*>(wk + 32 * a.bm_words);
+          if (there)
+            add_changes(tw, jj, lists, reinterpret_cast<const int*>(lists + 32 * kList), block_ov + k * wov_words,
+                        a.max_ppc, w0, w1, w2, acc);
+        }
+        if (there) {
+          if (!last) {
+            a.dv0[j] = acc[0]; a.dv1[j] = acc[1]; a.dv2[j] = acc[2];
+          } else {
+            dsmc_finish32(a, j, c, w0, w1, w2, acc, invK);
+          }
+        }
+      }
+      __syncthreads();
+      if (run)
+        for (int i = 0; i < wmax; ++i) bm[i] = 0u;
     }
   }
+  add_counts(a, cnt, lane);
 }
 
 // ------------------------------------------------------------ kick/drift --
@@ -2124,9 +2216,12 @@ cudaError_t launch_gather32(pic_ctx* c) {
 }
 
 const void* sort_big32_kernel_ptr() { return (const void*)k_sort_big32; }
-int dsmc32_threads() { return kDsmcThreads; }
-size_t dsmc32_smem_bytes(int bm_words) { return (size_t)(kDsmcThreads / 32) * dsmc32_smem_words(bm_words) * 4; }
-const void* dsmc32_kernel_ptr(bool verify) {
+// team: warps of a block that share a cell, or 0
+int dsmc32_threads(int team) { return team > 0 ? 32 * team : kDsmcThreads; }
+size_t dsmc32_smem_bytes(int bm_words, int threads) { return (size_t)(threads / 32) * dsmc32_smem_words(bm_words) * 4; }
+const void* dsmc32_kernel_ptr(bool verify, int team) {
+  if (team == 4) return verify ? (const void*)k_dsmc32_team<true, 4> : (const void*)k_dsmc32_team<false, 4>;
+  if (team == 2) return verify ? (const void*)k_dsmc32_team<true, 2> : (const void*)k_dsmc32_team<false, 2>;
   return verify ? (const void*)k_dsmc32<true> : (const void*)k_dsmc32<false>;
 }
 int cg32_threads() { return kCgThreads; }
@@ -2166,10 +2261,11 @@ cudaError_t launch_dsmc32(pic_ctx* c, uint32_t c0, bool separate, double t_src) 
   prof_begin(c);
   const cudaError_t eq = cudaMemsetAsync(c->dsmc_queue, 0, 8, c->stream);
   if (eq != cudaSuccess) return eq;
-  if (c->P.verify || a.lg.mode == PIC_DLOG_ALL)
-    k_dsmc32<true><<<c->dsmc_grid, kDsmcThreads, c->dsmc_smem, c->stream>>>(a);
-  else
-    k_dsmc32<false><<<c->dsmc_grid, kDsmcThreads, c->dsmc_smem, c->stream>>>(a);
+  const bool verify = c->P.verify || a.lg.mode == PIC_DLOG_ALL;
+  void* argv[] = {&a};
+  const cudaError_t el = cudaLaunchKernel(dsmc32_kernel_ptr(verify, c->dsmc_team), dim3(c->dsmc_grid),
+                                          dim3(c->dsmc_block), argv, c->dsmc_smem, c->stream);
+  if (el != cudaSuccess) return el;
   prof_end(c, KC_DSMC);
   c->launches++;
   return cudaGetLastError();

@@ -22,9 +22,9 @@ size_t cg_slot_bytes(int grid);
 int64_t scan_blocks_needed(int64_t ncell);
 int rhs_blocks_needed(int64_t ncell);
 int err_blocks_needed(int64_t np, int64_t ncell);
-int dsmc32_threads();
-size_t dsmc32_smem_bytes(int bm_words);
-const void* dsmc32_kernel_ptr(bool verify);
+int dsmc32_threads(int team);
+size_t dsmc32_smem_bytes(int bm_words, int threads);
+const void* dsmc32_kernel_ptr(bool verify, int team);
 int batch_dsmc_threads();
 const void* batch_dsmc_kernel_ptr();
 const void* sort_big_kernel_ptr();
@@ -979,10 +979,26 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
   c->dsmc_G = K < 32 ? 32 / K : 1;
   c->dsmc_groups = (c->P.ncell + c->dsmc_G - 1) / c->dsmc_G;
   c->bm_words = c->cfg.max_ppc / 32;
-  c->dsmc_block = c->mixed ? dsmc32_threads() : dsmc_threads();
-  const void* dsmc_fn = c->mixed ? dsmc32_kernel_ptr(c->P.verify != 0) : dsmc_kernel_ptr(c->P.verify != 0);
+  // precision form, several chunks of outcomes: how many warps share a cell.
+  // With fewer than three cells a resident warp (24 an SM) whole cells leave
+  // the last warps running alone, or SMs idle: two or four. With more, sharing
+  // pays by the velocities that a block's warps find in L1, from two words of
+  // 32 particles on: two, four from seven chunks. us a call by one, two and
+  // four warps a cell: 12^3 cells of 101, K = 243: 342, 191, 134; 16^3 of 320,
+  // K = 1,024: 3,600, 2,200, 1,640; 8^3 of 16, K = 40: 28, 18, 20; 32^3 of 128,
+  // K = 192: 602, 501, 536; 24^3 of 100, K = 200: 309, 280, 257; and of 32
+  // particles 32^3, K = 96: 124, 140, 153; 48^3, K = 64: 246, 260, 387.
+  const int chunks = (K + 31) / 32;
+  c->dsmc_team = 0;
+  if (c->mixed && chunks > 1) {
+    if (c->P.ncell < (int64_t)72 * c->num_sms) c->dsmc_team = chunks == 2 ? 2 : 4;
+    else if (c->P.np > 48 * c->P.ncell) c->dsmc_team = chunks < 7 ? 2 : 4;
+  }
+  c->dsmc_block = c->mixed ? dsmc32_threads(c->dsmc_team) : dsmc_threads();
+  const void* dsmc_fn =
+      c->mixed ? dsmc32_kernel_ptr(c->P.verify != 0, c->dsmc_team) : dsmc_kernel_ptr(c->P.verify != 0);
   if (c->mixed) {
-    c->dsmc_smem = dsmc32_smem_bytes(c->bm_words);
+    c->dsmc_smem = dsmc32_smem_bytes(c->bm_words, c->dsmc_block);
   } else {
     // the FP32 copy of a group's velocities: room for twice its mean; larger
     // groups are tested from their FP64 velocities
@@ -994,7 +1010,7 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
   if (c->dsmc_smem > 48 * 1024) {
     e = cudaFuncSetAttribute(dsmc_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dsmc_smem);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(c->mixed ? dsmc32_kernel_ptr(true) : dsmc_kernel_ptr(true),
+      e = cudaFuncSetAttribute(c->mixed ? dsmc32_kernel_ptr(true, c->dsmc_team) : dsmc_kernel_ptr(true),
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dsmc_smem);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -1032,7 +1048,7 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     while (parts > 1 && (size_t)parts * 24 * (size_t)c->P.np > kDsmcPartialBytes) --parts;
     c->dsmc_parts = parts < 1 ? 1 : (int)parts;
   }
-  int64_t dgrid = (c->dsmc_groups * c->dsmc_parts + wpb - 1) / wpb;
+  int64_t dgrid = c->dsmc_team ? c->dsmc_groups : (c->dsmc_groups * c->dsmc_parts + wpb - 1) / wpb;
   if (dgrid > (int64_t)docc * c->num_sms) dgrid = (int64_t)docc * c->num_sms;
   c->dsmc_grid = (int)(dgrid < 1 ? 1 : dgrid);
   if (c->cfg.K == 0) c->dsmc_grid = 1;

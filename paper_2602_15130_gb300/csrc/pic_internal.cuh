@@ -693,6 +693,7 @@ struct pic_ctx {
   double* overlay;  // per-lane working velocities
   int dsmc_grid, dsmc_block, dsmc_G, dsmc_Kc, bm_words;
   int dsmc_stage;   // FP64 form: particles of a cell group staged in shared memory
+  int dsmc_team;    // precision form: warps of a block that share a cell (k_dsmc32_team), or 0
   int dsmc_parts;   // FP64 form: warps that share a group's outcomes, and their sums [parts][3][N_p]
   double* dsmc_partial;
   int64_t dsmc_groups;
