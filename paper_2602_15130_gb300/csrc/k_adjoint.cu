@@ -29,6 +29,7 @@ struct AdjointBuffers {
   int seg = 0, ncp = 0, max_rec = 0;
   size_t np3 = 0, nc = 0, mu_len = 0, rec_len = 0;
   double *lam_x = nullptr, *lam_v = nullptr, *carry = nullptr, *G = nullptr, *lamL = nullptr;
+  double* vm = nullptr;  // v^M by pid, of the running call
   double *tx = nullptr, *tv = nullptr, *tvh = nullptr, *tE = nullptr;
   double* ck = nullptr;
   double *corner24 = nullptr, *lamE = nullptr, *badj = nullptr, *mu = nullptr, *Etmp = nullptr, *seedE = nullptr;
@@ -45,7 +46,7 @@ inline int nblk(int64_t n) { return (int)((n + kT - 1) / kT < 1 ? 1 : (n + kT - 
 template <class F>
 void each_buffer(AdjointBuffers& B, F f) {
   const size_t np3 = B.np3, nc = B.nc;
-  f(&B.lam_x, np3); f(&B.lam_v, np3); f(&B.carry, np3); f(&B.G, np3); f(&B.lamL, np3);
+  f(&B.lam_x, np3); f(&B.lam_v, np3); f(&B.carry, np3); f(&B.G, np3); f(&B.lamL, np3); f(&B.vm, np3);
   f(&B.tx, (size_t)(B.seg + 1) * np3); f(&B.tv, (size_t)B.seg * np3); f(&B.tvh, (size_t)B.seg * np3);
   f(&B.tE, (size_t)B.seg * 3 * nc);
   f(&B.ck, (size_t)B.ncp * (2 * np3 + 4 * nc));
@@ -72,13 +73,6 @@ __device__ double block_sum_d(double v, double* sh) {
   return t;
 }
 
-__device__ __forceinline__ void vM_of(const Params& P, uint64_t p, double* vm) {
-  const U4 b1 = sample_block(P, p, 1), b2 = sample_block(P, p, 2);
-  vm[0] = P.vmean[0] + P.vsig * normcdfinv(unif52(b1.z, b1.w));
-  vm[1] = P.vmean[1] + P.vsig * normcdfinv(unif52(b2.x, b2.y));
-  vm[2] = P.vmean[2] + P.vsig * normcdfinv(unif52(b2.z, b2.w));
-}
-
 // sorted buffers -> pid-ordered AoS
 __global__ void __launch_bounds__(kT) k_adj_store(int64_t np, const double* x0, const double* x1, const double* x2,
                                                    const double* v0, const double* v1, const double* v2,
@@ -90,31 +84,29 @@ __global__ void __launch_bounds__(kT) k_adj_store(int64_t np, const double* x0, 
   if (V) { V[3 * p] = v0[j]; V[3 * p + 1] = v1[j]; V[3 * p + 2] = v2[j]; }
 }
 
-// pid-ordered AoS -> the current buffers (slot = pid), with v^M of each pid
-__global__ void __launch_bounds__(kT) k_adj_load(Params P, const double* X, const double* V, double* x0, double* x1,
-                                                  double* x2, double* v0, double* v1, double* v2, double* m0,
-                                                  double* m1, double* m2, uint32_t* pid) {
+// pid-ordered AoS -> the current buffers (slot = pid). v^M comes from the
+// call's array: three inverse normals a particle, every time a state of the
+// sweep is loaded, were 100 us of a load of 262,144 particles.
+__global__ void __launch_bounds__(kT) k_adj_load(int64_t np, const double* X, const double* V, const double* M,
+                                                  double* x0, double* x1, double* x2, double* v0, double* v1,
+                                                  double* v2, double* m0, double* m1, double* m2, uint32_t* pid) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= P.np) return;
-  double vm[3];
-  vM_of(P, (uint64_t)i, vm);
-  m0[i] = vm[0]; m1[i] = vm[1]; m2[i] = vm[2];
+  if (i >= np) return;
+  m0[i] = M[3 * i]; m1[i] = M[3 * i + 1]; m2[i] = M[3 * i + 2];
   x0[i] = X[3 * i]; x1[i] = X[3 * i + 1]; x2[i] = X[3 * i + 2];
   v0[i] = V[3 * i]; v1[i] = V[3 * i + 1]; v2[i] = V[3 * i + 2];
   pid[i] = (uint32_t)i;
 }
 
 // lam_v = (2/N_p)(v - v^M), lam_x = carry = 0; block partials of |v - v^M|^2
-__global__ void __launch_bounds__(kT) k_adj_seed(Params P, const double* V, double* lam_v, double* lam_x,
-                                                  double* carry, double* part) {
+__global__ void __launch_bounds__(kT) k_adj_seed(Params P, const double* V, const double* M, double* lam_v,
+                                                  double* lam_x, double* carry, double* part) {
   __shared__ double sh[32];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double e2 = 0.0;
   if (i < P.np) {
-    double vm[3];
-    vM_of(P, (uint64_t)i, vm);
     for (int d = 0; d < 3; ++d) {
-      const double e = V[3 * i + d] - vm[d];
+      const double e = V[3 * i + d] - M[3 * i + d];
       e2 += e * e;
       if (lam_v) {
         lam_v[3 * i + d] = 2.0 / (double)P.np * e;
@@ -375,7 +367,7 @@ __global__ void __launch_bounds__(kT) k_adj_sum3(int64_t np, const double* v, do
 //   d = n . (mu_p' - mu_q') / 2.
 // The K outcomes average in ascending order; the analytic source adds
 //   -(d<dv^M>/dv)^T lam = pref (c-1) [s_v R(a) lam + (R'(a)/a)(m.lam) m/s_v]
-// with m = mu_v - v, a = |m|/s_v (R'(a)/a by its series below a = 0.3).
+// with m = mu_v - v, a = |m|/s_v.
 // ------------------------------------------------------------------------
 struct ListRec {
   double* r;
@@ -397,17 +389,78 @@ struct ListRec {
   }
 };
 
-__device__ __forceinline__ double hs_Rp_over_a(const Params& P, double a) {
-  if (a < 0.3) {
-    double acc = 2.0 * (kSeriesTerms - 1) * P.R_series[kSeriesTerms - 1];
-    for (int j = kSeriesTerms - 2; j >= 1; --j) acc = fma(acc, a * a, 2.0 * j * P.R_series[j]);
-    return acc;
+// Algorithm 1 for one (cell, outcome) lane in FP64, in the forward kernel's
+// arithmetic. The lane's working velocities live in a private overlay ov, valid
+// where the lane's bitmap bm has the particle's bit; untouched particles are
+// read from v. rec receives every accepted pair before its update.
+//
+// The accept test U < g / g_max is taken on the squares, apart by more than
+// 4e-12 g_max^2 (the near-tie bound, which covers the rounding of both sides
+// a thousand times), or else as the forward kernel decides it: an FP64 square
+// root and a division a candidate were most of this function. With the source by
+// table, a call of 16^3 cells of 64, K = 8: 290 us before, 120 now.
+__device__ __forceinline__ void load_vel(int p, const uint32_t* bm, const double* ov, const double* v0,
+                                         const double* v1, const double* v2, double* o) {
+  if ((bm[p >> 5] >> (p & 31)) & 1u) {
+    o[0] = ov[3 * p]; o[1] = ov[3 * p + 1]; o[2] = ov[3 * p + 2];
+  } else {
+    o[0] = v0[p]; o[1] = v1[p]; o[2] = v2[p];
   }
-  const double ia = 1.0 / a, ia2 = ia * ia;
-  const double sq2pi = 0.79788456080286535588;
-  const double rp = sq2pi * exp(-0.5 * a * a) * (ia - 3.0 * ia2 * ia) +
-                    (1.0 - 2.0 * ia2 + 3.0 * ia2 * ia2) * erf(a * 0.70710678118654752440);
-  return rp * ia;
+}
+
+__device__ void ntc_outcome(const Params& P, uint32_t c0, uint32_t cell, uint32_t o, int c, const double* v0,
+                            const double* v1, const double* v2, uint32_t* bm, double* ov, ListRec& rec) {
+  // the chi stream (c0, cell, slot, (o << 8) | 1): word 0 of slot 0 is the
+  // N_pairs uniform, word (s + 1) mod 4 of slot (s + 1) / 4 the chi of
+  // candidate s
+  U4 bchi = philox(c0, cell, 0u, (o << 8) | 1u, P.key0, P.key1);
+  long long chi_group = 0;
+  const double base = __dmul_rn(__dmul_rn((double)((long long)c * (long long)(c - 1)), P.pmax), 0.5);
+  const long long npairs = (long long)floor(__dadd_rn(base, unif32(bchi.x)));
+  const double gmax2 = P.gmax * P.gmax, margin = 4e-12 * gmax2, near = gmax2 * (1.0 - 4e-12);
+  // candidate s: block (c0, cell, s, o << 8) = (p, q, accept, epsilon);
+  // its chi block is formed when an accepted candidate needs it
+  for (long long s = 0; s < npairs; ++s) {
+    const U4 b0 = philox(c0, cell, (uint32_t)s, o << 8, P.key0, P.key1);
+    const uint32_t p = draw_index(b0.x, (uint32_t)c);
+    // q uniform over the other c - 1 particles: the distribution of
+    // drawing again until q != p
+    uint32_t q = draw_index(b0.y, (uint32_t)(c - 1));
+    q += q >= p ? 1u : 0u;
+    double vp[3], vq[3];
+    load_vel((int)p, bm, ov, v0, v1, v2, vp);
+    load_vel((int)q, bm, ov, v0, v1, v2, vq);
+    const double dx = __dsub_rn(vp[0], vq[0]), dy = __dsub_rn(vp[1], vq[1]), dz = __dsub_rn(vp[2], vq[2]);
+    const double g2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    // U = (2 w + 1) 2^-33 from the bits of 1 + U - 2^-33
+    const double U = __hiloint2double((int)(0x3ff00000u | b0.z >> 12), (int)(b0.z << 20)) - (1.0 - 0x1p-33);
+    const double ug = U * P.gmax, d = fma(ug, ug, -g2);
+    const bool accept =
+        fabs(d) > margin && g2 < near ? d < 0.0 : (ntc_decide64(P, b0.z, dx, dy, dz) & 1) != 0;
+    if (!accept) continue;
+    const long long js = s + 1;
+    if ((js >> 2) != chi_group) {
+      chi_group = js >> 2;
+      bchi = philox(c0, cell, (uint32_t)chi_group, (o << 8) | 1u, P.key0, P.key1);
+    }
+    const uint32_t wchi = (js & 3) == 0 ? bchi.x : (js & 3) == 1 ? bchi.y : (js & 3) == 2 ? bchi.z : bchi.w;
+    const double g = __dsqrt_rn(g2);
+    double se, ce;
+    sincospi(2.0 * unif32(b0.w), &se, &ce);
+    const double cchi = __dsub_rn(1.0, __dmul_rn(2.0, unif32(wchi)));
+    const double schi = __dsqrt_rn(__dsub_rn(1.0, __dmul_rn(cchi, cchi)));
+    const double nv[3] = {__dmul_rn(ce, schi), __dmul_rn(se, schi), cchi};
+    rec(p, q, vp, vq, nv, g);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const double gp = __dmul_rn(g, nv[e]);
+      const double cm = __dmul_rn(__dadd_rn(vp[e], vq[e]), 0.5);
+      ov[3 * p + e] = fma(gp, 0.5, cm);
+      ov[3 * q + e] = fma(gp, -0.5, cm);
+    }
+    bm[p >> 5] |= 1u << (p & 31);
+    bm[q >> 5] |= 1u << (q & 31);
+  }
 }
 
 struct DsmcAdjArgs {
@@ -441,7 +494,7 @@ __global__ void __launch_bounds__(kAdjDsmcThreads) k_dsmc_adj(DsmcAdjArgs a) {
   double* rec = a.rec + ((size_t)gwarp * 32 + lane) * a.max_rec * 12;
   for (int i = 0; i < a.bm_words; ++i) bm[i] = 0u;
   __syncwarp();
-  LaneCounts cnt = {0, 0, 0, 0};
+  const double invK = 1.0 / (double)P.K;
   for (int64_t grp = gwarp; grp < a.ngroups; grp += nwarps) {
     const int64_t cell0 = grp * a.Gc;
     const int ncl = (int)min((int64_t)a.Gc, P.ncell - cell0);
@@ -462,8 +515,7 @@ __global__ void __launch_bounds__(kAdjDsmcThreads) k_dsmc_adj(DsmcAdjArgs a) {
       }
       if (run) {
         ListRec R{rec, a.max_rec, 0, false};
-        ntc_outcome<false>(P, a.c0, (uint32_t)(cell0 + mycl), (uint32_t)o, c, a.v0 + s, a.v1 + s, a.v2 + s, bm, ov,
-                           cnt, R);
+        ntc_outcome(P, a.c0, (uint32_t)(cell0 + mycl), (uint32_t)o, c, a.v0 + s, a.v1 + s, a.v2 + s, bm, ov, R);
         if (R.overflow) atomicOr(a.flags, 1);
         for (int w = 0; w < (c + 31) / 32; ++w) {
           uint32_t bits = bm[w];
@@ -518,15 +570,15 @@ __global__ void __launch_bounds__(kAdjDsmcThreads) k_dsmc_adj(DsmcAdjArgs a) {
         if (!last) {
           a.G[3 * pj] = acc0; a.G[3 * pj + 1] = acc1; a.G[3 * pj + 2] = acc2;
         } else {
-          const double K = (double)P.K;
           const double m[3] = {P.vmean[0] - a.v0[j], P.vmean[1] - a.v1[j], P.vmean[2] - a.v2[j]};
-          const double am = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) * P.inv_vsig;
+          double R, Rp;
+          hs_R64_both(P, (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) * (P.inv_vsig * P.inv_vsig), &R, &Rp);
           const double pc = P.src_pref * (double)(cc - 1);
-          const double f1 = pc * P.vsig * hs_R(P, am);
-          const double f2 = pc * hs_Rp_over_a(P, am) * P.inv_vsig * (m[0] * l0 + m[1] * l1 + m[2] * l2);
-          a.G[3 * pj] = acc0 / K + f1 * l0 + f2 * m[0];
-          a.G[3 * pj + 1] = acc1 / K + f1 * l1 + f2 * m[1];
-          a.G[3 * pj + 2] = acc2 / K + f1 * l2 + f2 * m[2];
+          const double f1 = pc * P.vsig * R;
+          const double f2 = pc * Rp * P.inv_vsig * (m[0] * l0 + m[1] * l1 + m[2] * l2);
+          a.G[3 * pj] = acc0 * invK + f1 * l0 + f2 * m[0];
+          a.G[3 * pj + 1] = acc1 * invK + f1 * l1 + f2 * m[1];
+          a.G[3 * pj + 2] = acc2 * invK + f1 * l2 + f2 * m[2];
         }
       }
       __syncwarp();
@@ -621,9 +673,9 @@ cudaError_t store_xv(pic_ctx* c, double* X, double* V) {
 // pid-ordered (X, V) into the context, sorted by (cell, pid)
 cudaError_t load_sorted(pic_ctx* c, const double* X, const double* V) {
   const int b = c->cur;
-  k_adj_load<<<nblk(c->P.np), kT, 0, c->stream>>>(c->P, X, V, c->x[b][0], c->x[b][1], c->x[b][2], c->v[b][0],
-                                                  c->v[b][1], c->v[b][2], c->vm[b][0], c->vm[b][1], c->vm[b][2],
-                                                  c->pid[b]);
+  k_adj_load<<<nblk(c->P.np), kT, 0, c->stream>>>(c->P.np, X, V, c->adj->vm, c->x[b][0], c->x[b][1], c->x[b][2],
+                                                  c->v[b][0], c->v[b][1], c->v[b][2], c->vm[b][0], c->vm[b][1],
+                                                  c->vm[b][2], c->pid[b]);
   c->launches++;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemsetAsync(c->count, 0, (size_t)c->P.ncell * 4, c->stream);
@@ -728,6 +780,13 @@ extern "C" pic_status pic_adjoint_gradient(pic_ctx* c, int32_t nsteps, int32_t e
   } reset{c};
   // initial state: x^M(0), and v^M(0) or the given velocities
   AS(pic_sample_mms(c, 0.0));
+  {
+    const int b = c->cur;
+    k_adj_store<<<nblk(P.np), kT, 0, c->stream>>>(P.np, nullptr, nullptr, nullptr, c->vm[b][0], c->vm[b][1],
+                                                  c->vm[b][2], c->pid[b], nullptr, B.vm);
+    c->launches++;
+    AK(cudaGetLastError());
+  }
   if (v0) {
     AK(store_xv(c, B.tx, nullptr));
     AK(cudaMemcpyAsync(B.tv, v0, np3 * sizeof(double), cudaMemcpyDefault, c->stream));
@@ -754,7 +813,7 @@ extern "C" pic_status pic_adjoint_gradient(pic_ctx* c, int32_t nsteps, int32_t e
   // objective
   AK(store_xv(c, nullptr, B.tv));
   const int nbp = nblk(P.np), nbc = nblk(P.ncell);
-  k_adj_seed<<<nbp, kT, 0, c->stream>>>(P, B.tv, grad ? B.lam_v : nullptr, B.lam_x, B.carry, B.part);
+  k_adj_seed<<<nbp, kT, 0, c->stream>>>(P, B.tv, B.vm, grad ? B.lam_v : nullptr, B.lam_x, B.carry, B.part);
   k_adj_final<<<1, kT, 0, c->stream>>>(B.part, nbp, 1, B.acc + 8, 1.0 / (double)P.np, 0);
   k_adj_energy<<<nbc, kT, 0, c->stream>>>(P.ncell, c->E[0], c->E[1], c->E[2], B.part);
   k_adj_final<<<1, kT, 0, c->stream>>>(B.part, nbc, 1, B.acc + 9, 0.5 * P.eps0 * P.dV, 0);

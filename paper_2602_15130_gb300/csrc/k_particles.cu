@@ -224,17 +224,6 @@ __device__ __forceinline__ int list_find(const ListEntry* wl, int t, int p) {
   return k;
 }
 
-// The accept decision of one candidate in FP64, as the paper writes it
-// (U < sigma(g) g / (sigma g)_max), with the near-tie and g > g_max flags.
-__device__ __noinline__ int ntc_decide64(const Params& P, uint32_t w, double dx, double dy, double dz) {
-  const double g2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-  const double g = __dsqrt_rn(g2);
-  const double ratio = P.n_sigma == 0 ? __ddiv_rn(__dmul_rn(P.sigma0, g), P.sg_max)
-                                      : __ddiv_rn(sigma_g(P, g2), P.sg_max);
-  const double U = unif32(w);
-  return (U < ratio ? 1 : 0) | (fabs(U - ratio) < 1e-12 ? 2 : 0) | (g > P.gmax ? 4 : 0);
-}
-
 // FP32 constants of the test
 struct Test32 {
   float gmax, gmax2, sgmax, s0, s1, s2;
@@ -269,18 +258,6 @@ __device__ __forceinline__ int ntc_test32(const Test32& T, uint32_t w, const flo
   }
   if (fabsf(lhs - rhs) > margin && g2 + e2 < T.gmax2) return lhs < rhs ? 1 : 0;
   return -1;
-}
-
-// R(a) of hs_R at u = a^2: polynomials of degree 7 on intervals of 1/8 up to
-// kR64Max (interpolation error below 1e-17), the closed form beyond.
-__device__ __forceinline__ double hs_R64(const Params& P, double u) {
-  if (!(u < (double)kR64Max)) return hs_R(P, sqrt(u));
-  const double t = u * (double)kR64PerUnit;
-  const double r = floor_small(t);
-  const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1)) + 4 * (int)r;
-  const double x = t - r - 0.5;
-  const double2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
-  return fma(fma(fma(fma(fma(fma(fma(q3.y, x, q3.x), x, q2.y), x, q2.x), x, q1.y), x, q1.x), x, q0.y), x, q0.x);
 }
 
 // Algorithm 1 for the warp's (cell, outcome) lanes: outcome o of cell `cell`
