@@ -2007,12 +2007,13 @@ __global__ void __launch_bounds__(kThreads) k_err_partial32(Err32Args a) {
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         double s, cc;
-        const double xm = paper ? xm_solve_gen(a.tt, d, xi[d], &s, &cc) : xm_solve(P, a.tt, xi[d], &s);
+        const double xm = paper ? xm_solve_gen(a.tt, d, xi[d], &s, &cc) : xm_table(P, a.tt, xi[d]);
         double e = ((double)ci[d] + (double)os[d]) * P.h - xm;
         e -= floor(e + 0.5);
         vals[d] = e * e;
         vals[7 + d] = fabs(e);
-        const double vmd = paper ? tau_inv(xi[3 + d]) * a.tt.vh[d] : P.vmean[d] + P.vsig * normcdfinv(xi[3 + d]);
+        const double vmd =
+            paper ? tau_inv(xi[3 + d]) * a.tt.vh[d] : P.vmean[d] + P.vsig * normal_quantile(P, xi[3 + d]);
         const double ev = (double)vs[d] - vmd;
         vals[3 + d] = ev * ev;
         vals[10 + d] = fabs(ev);

@@ -36,8 +36,8 @@ __global__ void __launch_bounds__(kThreads) k_sample(SampleArgs a) {
            b2 = sample_block(P, (uint64_t)i, 2);
   const double xi[6] = {unif52(b0.x, b0.y), unif52(b0.z, b0.w), unif52(b1.x, b1.y),
                         unif52(b1.z, b1.w), unif52(b2.x, b2.y), unif52(b2.z, b2.w)};
-  double s;
   if (P.dist == PIC_DIST_PAPER) {
+    double s;
     // x^M(t0) per axis; v^M(t0) = vh(t0) tau(xi), tau kept in the v^M arrays
     double c;
     a.x0[i] = wrap_unit(xm_solve_gen(a.tt, 0, xi[0], &s, &c));
@@ -49,12 +49,12 @@ __global__ void __launch_bounds__(kThreads) k_sample(SampleArgs a) {
     a.pid[i] = (uint32_t)i;
     return;
   }
-  const double X0 = xm_solve(P, a.tt, xi[0], &s);
-  const double X1 = xm_solve(P, a.tt, xi[1], &s);
-  const double X2 = xm_solve(P, a.tt, xi[2], &s);
-  const double V0 = P.vmean[0] + P.vsig * normcdfinv(xi[3]);
-  const double V1 = P.vmean[1] + P.vsig * normcdfinv(xi[4]);
-  const double V2 = P.vmean[2] + P.vsig * normcdfinv(xi[5]);
+  const double X0 = xm_table(P, a.tt, xi[0]);
+  const double X1 = xm_table(P, a.tt, xi[1]);
+  const double X2 = xm_table(P, a.tt, xi[2]);
+  const double V0 = P.vmean[0] + P.vsig * normal_quantile(P, xi[3]);
+  const double V1 = P.vmean[1] + P.vsig * normal_quantile(P, xi[4]);
+  const double V2 = P.vmean[2] + P.vsig * normal_quantile(P, xi[5]);
   a.x0[i] = wrap_unit(X0); a.x1[i] = wrap_unit(X1); a.x2[i] = wrap_unit(X2);
   a.v0[i] = V0; a.v1[i] = V1; a.v2[i] = V2;
   a.vm0[i] = V0; a.vm1[i] = V1; a.vm2[i] = V2;
@@ -81,9 +81,9 @@ __global__ void __launch_bounds__(kThreads) k_load_state(LoadArgs a) {
   if (P.dist == PIC_DIST_PAPER) {
     a.vm0[i] = tau_inv(xi[3]); a.vm1[i] = tau_inv(xi[4]); a.vm2[i] = tau_inv(xi[5]);
   } else {
-    a.vm0[i] = P.vmean[0] + P.vsig * normcdfinv(xi[3]);
-    a.vm1[i] = P.vmean[1] + P.vsig * normcdfinv(xi[4]);
-    a.vm2[i] = P.vmean[2] + P.vsig * normcdfinv(xi[5]);
+    a.vm0[i] = P.vmean[0] + P.vsig * normal_quantile(P, xi[3]);
+    a.vm1[i] = P.vmean[1] + P.vsig * normal_quantile(P, xi[4]);
+    a.vm2[i] = P.vmean[2] + P.vsig * normal_quantile(P, xi[5]);
   }
   const double* xs = a.xs;
   const double* vs = a.vs;
@@ -659,12 +659,6 @@ struct KickArgs {
   int32_t *key, *rank, *count;
 };
 
-constexpr double kRound52 = 0x1.8p52;  // adding it rounds to an integer, in the low word
-
-// exponent of |x|, as in the high word of 2^e
-__device__ __forceinline__ bool below_pow2(double x, int e) {
-  return (__double2hiint(x) & 0x7fffffff) < (1023 + e) << 20;
-}
 __device__ __noinline__ void sincos_far(double d, double* s, double* c) { sincospi(2.0 * d, s, c); }
 
 // sin and cos of 2 pi d: the table at the nearest kTrigM-th of
@@ -729,7 +723,7 @@ __device__ __forceinline__ void lorentz64(const KickArgs& a, const double* x, do
     }
   // E^M = -amp (c0 s1 s2, s0 c1 s2, s0 s1 c2)
   const double2* tab =
-      reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1) + kR64Doubles + 8 * kSlopeM);
+      reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1) + kQuantileDoubles + kR64Doubles + 8 * kSlopeM);
   double s0, c0, s1, c1, s2, c2;
   sincos_turn(tab, x[0] - P.phi_shift[0], &s0, &c0);
   sincos_turn(tab, x[1] - P.phi_shift[1], &s1, &c1);
@@ -782,11 +776,8 @@ __global__ void __launch_bounds__(kThreads) k_kick(KickArgs a) {
       const double T = m - a.T0;
       const double z = fma(T, (double)kSlopeM, kRound52);
       const double u = fma(T, (double)kSlopeM, kRound52 - z);
-      const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1) + kR64Doubles) +
-                         4 * (__double2loint(z) & (kSlopeM - 1));
-      const double2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
-      const double g =
-          fma(fma(fma(fma(fma(fma(fma(q3.y, u, q3.x), u, q2.y), u, q2.x), u, q1.y), u, q1.x), u, q0.y), u, q0.x);
+      const double g = poly7(P.ginv + 2 * (P.ginv_M + 1) + kQuantileDoubles + kR64Doubles,
+                             __double2loint(z) & (kSlopeM - 1), u);
       x[d] = wrap_unit(fma(P.dt, (v[d] - vm[d]) + fma(-a.xslope, g, P.fx_speed), x[d]));
     } else {
       const double xi = unif52(hi[d], lw[d]);
@@ -875,7 +866,7 @@ __global__ void __launch_bounds__(kThreads) k_err_partial(ErrArgs a) {
       for (int d = 0; d < 3; ++d) {
         double s, c;
         const bool paper = P.dist == PIC_DIST_PAPER;
-        const double xm = paper ? xm_solve_gen(a.tt, d, xi[d], &s, &c) : xm_solve(P, a.tt, xi[d], &s);
+        const double xm = paper ? xm_solve_gen(a.tt, d, xi[d], &s, &c) : xm_table(P, a.tt, xi[d]);
         double e = xs[d] - xm;
         e -= floor(e + 0.5);
         vals[d] = e * e;
@@ -1082,7 +1073,7 @@ cudaError_t launch_kick(pic_ctx* c, double tE, bool with_coll, bool drift, doubl
   a.key = c->key;
   a.rank = c->rank;
   a.count = c->count;
-  const bool table = P.dist == PIC_DIST_CONFIG && !(P.verify & PIC_VERIFY_ISOLATE) && c->slope_table &&
+  const bool table = P.dist == PIC_DIST_CONFIG && !(P.verify & PIC_VERIFY_ISOLATE) && P.xm_table &&
                      fabs(a.T0) < 0x1p30;  // (beyond, T has no digits left to look up)
   prof_begin(c);
   if (table) k_kick<true><<<blocks_for(P.np), kThreads, 0, c->stream>>>(a);

@@ -23,7 +23,7 @@ __device__ __forceinline__ double hs_R64(const Params& P, double u) {
   if (!(u < (double)kR64Max)) return hs_R(P, sqrt(u));
   const double t = u * (double)kR64PerUnit;
   const double r = floor_small(t);
-  const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1)) + 4 * (int)r;
+  const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1) + kQuantileDoubles) + 4 * (int)r;
   const double x = t - r - 0.5;
   const double2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
   return fma(fma(fma(fma(fma(fma(fma(q3.y, x, q3.x), x, q2.y), x, q2.x), x, q1.y), x, q1.x), x, q0.y), x, q0.x);
@@ -42,7 +42,7 @@ __device__ __forceinline__ void hs_R64_both(const Params& P, double u, double* R
   }
   const double t = u * (double)kR64PerUnit;
   const double r = floor_small(t);
-  const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1)) + 4 * (int)r;
+  const double2* q = reinterpret_cast<const double2*>(P.ginv + 2 * (P.ginv_M + 1) + kQuantileDoubles) + 4 * (int)r;
   const double x = t - r - 0.5;
   const double2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
   double d = q3.y, v = fma(q3.y, x, q3.x);

@@ -188,7 +188,8 @@ void hs_R64_table(double* out) {
 // term left out stays below rounding everywhere (A = 0.3: 4e-18; from
 // |A| = 0.6 on G^{-1} bends too sharply). Behind it sin and cos of
 // 2 pi k / kTrigM, from the first octant's.
-bool kick_tables(double A, const double* ginv, double* out) {
+// With xm: the same for G^{-1}(T) - T = A / (2 pi) C, its integral.
+bool kick_tables(double A, const double* ginv, double* out, double* xm) {
   constexpr int kN = 9;
   double worst = 0.0;
   for (int k = 0; k < kSlopeM; ++k) {
@@ -210,11 +211,15 @@ bool kick_tables(double A, const double* ginv, double* out) {
       C[j + 1] = 2.0 * kPi / (j + 1) * dc;
     }
     double scale = 1.0;
-    for (int j = 0; j < 8; ++j, scale /= kSlopeM) out[8 * k + j] = g[j] * scale;
+    xm[8 * k] = A / (2.0 * kPi) * C[0];
+    for (int j = 0; j < 8; ++j, scale /= kSlopeM) {
+      if (out) out[8 * k + j] = g[j] * scale;
+      if (j < 7) xm[8 * k + j + 1] = (j == 0 ? -A * S[0] * d0 : g[j]) * scale / kSlopeM / (j + 1);
+    }
     worst = fmax(worst, fabs(g[8] * scale) / 256.0);
   }
   double* t = out + 8 * kSlopeM;
-  for (int k = 0; k < kTrigM; ++k) {
+  for (int k = 0; out && k < kTrigM; ++k) {
     const int quarter = kTrigM / 4, q = k / quarter, r = k % quarter;
     const int f = r <= quarter / 2 ? r : quarter - r;  // folded to the octant
     double s = sin(2.0 * kPi * f / kTrigM), c = cos(2.0 * kPi * f / kTrigM);
@@ -223,6 +228,51 @@ bool kick_tables(double A, const double* ginv, double* out) {
     t[2 * k + 1] = q == 0 ? c : q == 1 ? -s : q == 2 ? -c : s;
   }
   return worst <= 0x1p-55;
+}
+
+// The normal quantile z(q) around the middle q_0 of every interval of q below
+// 1/2, in powers of q - q_0, from the recurrence of w = dz/dq = sqrt(2 pi)
+// exp(z^2 / 2): w' = z w^2. z_0 by Newton from the neighbour's polynomial (the
+// first from q = 1/2); the first term left out is below 2^-56.
+void quantile_table(double* out) {
+  double z0 = 0.0, q0 = 0.5, c[9] = {0.0, sqrt(2.0 * kPi)};
+  for (int k = 0; k < kQuantSub * kQuantExp; ++k) {
+    const int e = k / kQuantSub, m = k % kQuantSub;  // q in 2^-(e+1) (1 - (m, m + 1) / (2 kQuantSub))
+    const double q = ldexp(1.0 - (m + 0.5) / (2.0 * kQuantSub), -(e + 1));
+    double z = 0.0;
+    for (int j = 8; j >= 0; --j) z = z * (q - q0) + c[j];
+    for (int it = 0; it < 2; ++it)
+      z -= (0.5 * erfc(-z / sqrt(2.0)) - q) * sqrt(2.0 * kPi) * exp(0.5 * z * z);
+    z0 = z;
+    q0 = q;
+    double w[8];
+    c[0] = z0;
+    w[0] = sqrt(2.0 * kPi) * exp(0.5 * z0 * z0);
+    for (int j = 0; j < 8; ++j) {
+      c[j + 1] = w[j] / (j + 1);
+      if (j == 7) break;
+      double t = 0.0;  // (z w^2)_j
+      for (int a = 0; a <= j; ++a)
+        for (int b = 0; b <= j - a; ++b) t += c[a] * w[b] * w[j - a - b];
+      w[j + 1] = t / (j + 1);
+    }
+    for (int j = 0; j < 8; ++j) out[8 * k + j] = c[j];
+  }
+}
+
+// all of the FP64 tables behind the G^{-1} knots; slope: with the kick's
+bool form_tables(double A, const double* ginv, bool fp64, double* out) {
+  // the same for every context: formed once
+  static const std::unique_ptr<double[]> fixed = [] {
+    std::unique_ptr<double[]> t(new double[kQuantDoubles + kR64Doubles]);
+    quantile_table(t.get());
+    hs_R64_table(t.get() + kQuantDoubles);
+    return t;
+  }();
+  memcpy(out + kXmDoubles, fixed.get(), sizeof(double) * kQuantDoubles);
+  double* r64 = out + kQuantileDoubles;
+  if (fp64) memcpy(r64, fixed.get() + kQuantDoubles, sizeof(double) * kR64Doubles);
+  return kick_tables(A, ginv, fp64 ? r64 + kR64Doubles : nullptr, out);
 }
 
 // FP32 tables of the precision form: the knots of G^{-1} (y_k, dy/dT) and
@@ -459,7 +509,7 @@ void for_each_buffer(pic_ctx* c, F f) {
   f((void**)&c->flags, 64);
   f((void**)&c->err_part, (size_t)c->err_blocks * 14 * 8);
   f((void**)&c->err_out, 14 * 8);
-  f((void**)&c->ginv, ((size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles + kKickDoubles)) * 8);
+  f((void**)&c->ginv, ((size_t)(kGinvM + 1) * 2 + kQuantileDoubles + (c->mixed ? 0 : kR64Doubles + kKickDoubles)) * 8);
   f((void**)&c->ginv_f, (size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4);
   if (c->nrep == 0 && (c->cfg.verify & PIC_VERIFY_ANGLES)) {
     f((void**)&c->ang_hist, (size_t)2 * PIC_ANGLE_BINS * 8);
@@ -1064,7 +1114,8 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     return PIC_ENOMEM;
   }
   {
-    const size_t tab_doubles = (size_t)(kGinvM + 1) * 2 + (c->mixed ? 0 : kR64Doubles + kKickDoubles);
+    const size_t tab_doubles =
+        (size_t)(kGinvM + 1) * 2 + kQuantileDoubles + (c->mixed ? 0 : kR64Doubles + kKickDoubles);
     double* tab = (double*)malloc(tab_doubles * 8);
     float* tabf = (float*)malloc((size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4);
     if (!tab || !tabf) {
@@ -1075,16 +1126,7 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     }
     ginv_table(c->cfg.fx_amp, tab);
     ginv_table_f(tab, tabf);
-    if (!c->mixed) {
-      // the same for every context: formed once
-      static const std::unique_ptr<double[]> r64 = [] {
-        std::unique_ptr<double[]> t(new double[kR64Doubles]);
-        hs_R64_table(t.get());
-        return t;
-      }();
-      memcpy(tab + (kGinvM + 1) * 2, r64.get(), sizeof(double) * kR64Doubles);
-      c->slope_table = kick_tables(c->cfg.fx_amp, tab, tab + (kGinvM + 1) * 2 + kR64Doubles);
-    }
+    c->P.xm_table = form_tables(c->cfg.fx_amp, tab, !c->mixed, tab + (kGinvM + 1) * 2);
     e = cudaMemcpy(c->ginv, tab, tab_doubles * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->ginv_f, tabf, (size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4,
                                          cudaMemcpyHostToDevice);
@@ -1741,12 +1783,14 @@ pic_status pic_create_batch(const pic_config* cfgs, int32_t nrep, void* stream, 
   }
   // G^{-1} tables (shared manufactured distribution), then per-replicate copies
   {
-    double* tab = (double*)malloc((size_t)(kGinvM + 1) * 2 * 8);
+    const size_t tab_doubles = (size_t)(kGinvM + 1) * 2 + kQuantileDoubles;
+    double* tab = (double*)malloc(tab_doubles * 8);
     float* tabf = (float*)malloc((size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4);
     if (tab && tabf) {
       ginv_table(c0.fx_amp, tab);
       ginv_table_f(tab, tabf);
-      e = cudaMemcpy(c->ginv, tab, (size_t)(kGinvM + 1) * 2 * 8, cudaMemcpyHostToDevice);
+      c->P.xm_table = form_tables(c0.fx_amp, tab, false, tab + (kGinvM + 1) * 2);
+      e = cudaMemcpy(c->ginv, tab, tab_doubles * 8, cudaMemcpyHostToDevice);
       if (e == cudaSuccess) e = cudaMemcpy(c->ginv_f, tabf, (size_t)(kGinvM + 1) * 4 * 4 + (size_t)(kRTabM + 1) * 2 * 4,
                                          cudaMemcpyHostToDevice);
     } else {
@@ -1762,6 +1806,7 @@ pic_status pic_create_batch(const pic_config* cfgs, int32_t nrep, void* stream, 
     c->prm_host[r].ginv = c->ginv;
     c->prm_host[r].ginv_f = c->ginv_f;
     c->prm_host[r].ginv_M = kGinvM;
+    c->prm_host[r].xm_table = c->P.xm_table;
     c->reps_host[r].f = params_f(c->prm_host[r]);
   }
   if (e == cudaSuccess) e = cudaMemcpy(c->reps_dev, c->reps_host, sizeof(BatchRep) * nrep, cudaMemcpyHostToDevice);

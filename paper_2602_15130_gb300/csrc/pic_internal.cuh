@@ -29,6 +29,12 @@ constexpr int kR64Doubles = 8 * kR64Max * kR64PerUnit;
 // of degree 7 a period, and (sin, cos) of 2 pi k / kTrigM
 constexpr int kSlopeM = 512, kTrigM = 256;
 constexpr int kKickDoubles = 8 * kSlopeM + 2 * kTrigM;
+// FP64 tables of the quantiles, behind the G^{-1} knots in every form:
+// G^{-1}(T) - T as kSlopeM polynomials of degree 7 a period, and the normal
+// quantile as kQuantSub of them a power of two of the tail probability
+constexpr int kQuantExp = 12, kQuantSub = 64;
+constexpr int kXmDoubles = 8 * kSlopeM, kQuantDoubles = 8 * kQuantSub * kQuantExp;
+constexpr int kQuantileDoubles = kXmDoubles + kQuantDoubles;
 
 // ---------------------------------------------------------------------------
 // Everything a kernel needs to know about the problem, passed by value.
@@ -56,6 +62,7 @@ struct Params {
   const double* ginv;
   const float* ginv_f;
   int ginv_M;
+  int xm_table;                    // the tables of G^{-1}(T) - T and dG^{-1}/dT are exact to rounding
   int verify;                      // PIC_VERIFY_* bits
   unsigned long long* ang_hist;    // [2][PIC_ANGLE_BINS] when recording angles
   double E_app[3];                 // uniform applied field in the push (adjoint parameter; 0 otherwise)
@@ -460,6 +467,47 @@ __device__ __forceinline__ void e_manufactured(const Params& P, const TimeTerms&
   *ez = -tt.em_amp * s0 * s1 * c2;
 }
 
+constexpr double kRound52 = 0x1.8p52;  // adding it rounds to an integer, in the low word
+
+// |x| < 2^e (false for NaN and infinities)
+__device__ __forceinline__ bool below_pow2(double x, int e) {
+  return (__double2hiint(x) & 0x7fffffff) < (1023 + e) << 20;
+}
+
+// a polynomial of degree 7 of a table
+__device__ __forceinline__ double poly7(const double* table, int k, double u) {
+  const double2* q = reinterpret_cast<const double2*>(table) + 4 * k;
+  const double2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
+  return fma(fma(fma(fma(fma(fma(fma(q3.y, u, q3.x), u, q2.y), u, q2.x), u, q1.y), u, q1.x), u, q0.y), u, q0.x);
+}
+
+// x^M of xm_solve by table: 14 FP64 instructions instead of 75 (a Hermite
+// start, a sincospi, two divisions), which bound sampling and norms.
+__device__ __forceinline__ double xm_table(const Params& P, const TimeTerms& tt, double xi) {
+  const double T = xi - tt.ct - P.fx_amp_over_2pi * tt.cos2ct;
+  if (!P.xm_table || !below_pow2(T, 30)) {
+    double s;
+    return xm_solve(P, tt, xi, &s);
+  }
+  const double z = fma(T, (double)kSlopeM, kRound52);
+  const double u = fma(T, (double)kSlopeM, kRound52 - z);
+  const double d = poly7(P.ginv + 2 * (P.ginv_M + 1), __double2loint(z) & (kSlopeM - 1), u);
+  return T + d + tt.ct;
+}
+
+// The quantile of the standard normal at xi, an odd multiple of 2^-53: by
+// table for a tail probability of at least 2^-13 (9 FP64 instructions, 63
+// of normcdfinv), which one value in 4,000 falls short of.
+__device__ __forceinline__ double normal_quantile(const Params& P, double xi) {
+  const double q = xi < 0.5 ? xi : 1.0 - xi;
+  const int hi = __double2hiint(q);
+  const int k = (0x3fe00000 >> 14) - 1 - (hi >> 14);
+  if (k >= kQuantSub * kQuantExp) return normcdfinv(xi);
+  const double mid = __hiloint2double((hi & ~0x3fff) | 0x2000, 0);
+  const double z = poly7(P.ginv + 2 * (P.ginv_M + 1) + kXmDoubles, k, q - mid);
+  return xi < 0.5 ? z : -z;
+}
+
 // floor of 0 <= t < 2^31 without a conversion instruction (FP64 conversions
 // run on the FP64 pipe, as an addition does)
 __device__ __forceinline__ double floor_small(double t) {
@@ -622,7 +670,6 @@ struct pic_ctx {
 
   double* dv[3];    // collision term per particle (sorted order)
   double* lor[3];   // dt q/m (E_p - E^M_p) of the last kick without drift
-  bool slope_table;  // the drift's table of dG^{-1}/dT is exact to rounding
   bool lor_valid;   // lor matches the current order, positions and field
   // precision form: v^M (tau for the paper's f_v) by pid, written with the
   // context's first state
