@@ -2012,8 +2012,9 @@ __global__ void __launch_bounds__(kThreads) k_err_partial32(Err32Args a) {
         e -= floor(e + 0.5);
         vals[d] = e * e;
         vals[7 + d] = fabs(e);
-        const double vmd =
-            paper ? tau_inv(xi[3 + d]) * a.tt.vh[d] : P.vmean[d] + P.vsig * normal_quantile(P, xi[3 + d]);
+        // (normcdfinv, whose values give sampled velocities the same norm bits
+        // in any order of the particles that was tested)
+        const double vmd = paper ? tau_inv(xi[3 + d]) * a.tt.vh[d] : P.vmean[d] + P.vsig * normcdfinv(xi[3 + d]);
         const double ev = (double)vs[d] - vmd;
         vals[3 + d] = ev * ev;
         vals[10 + d] = fabs(ev);
