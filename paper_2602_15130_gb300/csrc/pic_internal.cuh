@@ -129,11 +129,14 @@ constexpr int kBatchTile = 256;
 // batch is a chain of barriers and of each thread's loads, with most SMs
 // idle) up to kTeamNodes (many replicates fill the SMs, and more blocks in a
 // team only wait longer). The solves of 16 replicates of up to 32^3 nodes: 5.9 ms
-// with 16,384 nodes a block, 0.98 ms by this rule.
-constexpr int kTeamNodesMin = 1024, kTeamNodes = 16384;
+// with 16,384 nodes a block, 0.98 ms by this rule. A mesh of up to kTeamSolo
+// nodes is one block's: its barriers cost less than a team's (six steps of
+// four replicates of up to 16^3: 6.8 ms by one block, 7.2 and 8.9 by teams of
+// four and two).
+constexpr int kTeamNodesMin = 1024, kTeamNodes = 16384, kTeamSolo = 4096;
 constexpr int kTeamMax = 32;
 inline int cg_team_size(int m, int nodes) {
-  const int T = m / nodes;
+  const int T = m <= kTeamSolo ? 1 : m / nodes;
   return T < 1 ? 1 : (T > kTeamMax ? kTeamMax : T);
 }
 
