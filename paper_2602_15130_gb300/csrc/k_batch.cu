@@ -62,30 +62,23 @@ __global__ void __launch_bounds__(kThreads) kb_sample(BSampleArgs a) {
            b2 = sample_block(P, (uint64_t)loc, 2);
   const double xi[6] = {unif52(b0.x, b0.y), unif52(b0.z, b0.w), unif52(b1.x, b1.y),
                         unif52(b1.z, b1.w), unif52(b2.x, b2.y), unif52(b2.z, b2.w)};
-  double x[3], v[3], vm[3];
+  const int n = P.n;
+  int ci[3];
+  float off[3], v[3], vm[3];
   for (int d = 0; d < 3; ++d) {
-    double s;
-    vm[d] = P.vmean[d] + P.vsig * normcdfinv(xi[3 + d]);
+    vm[d] = vm_sample32(P, d, xi[3 + d]);
     if (a.xv) {
-      x[d] = a.xv[3 * i + d];
-      v[d] = a.xv[3 * a.np + 3 * i + d];
+      ci[d] = cell_offset32(a.xv[3 * i + d], n, &off[d]);
+      v[d] = (float)a.xv[3 * a.np + 3 * i + d];
     } else {
-      x[d] = wrap_unit(xm_solve(P, a.tt[3 * r], xi[d], &s));
+      ci[d] = xm_sample32(P, a.tt[3 * r], xi[d], &off[d]);
       v[d] = vm[d];
     }
   }
-  const int n = P.n;
-  int ci[3];
-  float off[3];
-  for (int d = 0; d < 3; ++d) {
-    ci[d] = cell_coord(x[d], n);
-    const float o = (float)(x[d] * (double)n - (double)ci[d]);
-    off[d] = o >= 1.f ? 0x1.fffffep-1f : (o < 0.f ? 0.f : o);
-  }
   a.cell[i] = (int32_t)(a.reps[r].coff + ci[0] + n * (ci[1] + n * ci[2]));
   a.o0[i] = off[0]; a.o1[i] = off[1]; a.o2[i] = off[2];
-  a.v0[i] = (float)v[0]; a.v1[i] = (float)v[1]; a.v2[i] = (float)v[2];
-  a.m0[i] = (float)vm[0]; a.m1[i] = (float)vm[1]; a.m2[i] = (float)vm[2];
+  a.v0[i] = v[0]; a.v1[i] = v[1]; a.v2[i] = v[2];
+  a.m0[i] = vm[0]; a.m1[i] = vm[1]; a.m2[i] = vm[2];
   a.pid[i] = (uint32_t)loc;
 }
 

@@ -99,22 +99,28 @@ __global__ void __launch_bounds__(kThreads) k_sample32(Sample32Args a) {
   const double xi[6] = {unif52(b0.x, b0.y), unif52(b0.z, b0.w), unif52(b1.x, b1.y),
                         unif52(b1.z, b1.w), unif52(b2.x, b2.y), unif52(b2.z, b2.w)};
   const bool paper = P.dist == PIC_DIST_PAPER;
-  double vm[3];
-  for (int d = 0; d < 3; ++d) vm[d] = paper ? tau_inv(xi[3 + d]) : P.vmean[d] + P.vsig * normcdfinv(xi[3 + d]);
-  const float4 m = make_float4((float)vm[0], (float)vm[1], (float)vm[2], 0.f);
-  a.vm[i] = m;
-  if (!a.state) return;
-  const int n = P.n;
   int ci[3];
   float off[3], vf[3];
-  for (int d = 0; d < 3; ++d) {
-    double s, cc;
-    const double x = wrap_unit(paper ? xm_solve_gen(a.tt, d, xi[d], &s, &cc) : xm_solve(P, a.tt, xi[d], &s));
-    vf[d] = (float)(paper ? vm[d] * a.tt.vh[d] : vm[d]);
-    ci[d] = cell_coord(x, n);
-    const float o = (float)fma(x, (double)n, -(double)ci[d]);
-    off[d] = o >= 1.f ? 0x1.fffffep-1f : (o < 0.f ? 0.f : o);
+  float4 m;
+  if (!paper) {
+    m = make_float4(vm_sample32(P, 0, xi[3]), vm_sample32(P, 1, xi[4]), vm_sample32(P, 2, xi[5]), 0.f);
+    a.vm[i] = m;
+    if (!a.state) return;
+    for (int d = 0; d < 3; ++d) ci[d] = xm_sample32(P, a.tt, xi[d], &off[d]);
+    vf[0] = m.x; vf[1] = m.y; vf[2] = m.z;
+  } else {
+    double tau[3];
+    for (int d = 0; d < 3; ++d) tau[d] = tau_inv(xi[3 + d]);
+    m = make_float4((float)tau[0], (float)tau[1], (float)tau[2], 0.f);
+    a.vm[i] = m;
+    if (!a.state) return;
+    for (int d = 0; d < 3; ++d) {
+      double s, c;
+      ci[d] = cell_offset32(wrap_unit(xm_solve_gen(a.tt, d, xi[d], &s, &c)), P.n, &off[d]);
+      vf[d] = (float)(tau[d] * a.tt.vh[d]);
+    }
   }
+  const int n = P.n;
   put32(a.put, i, ci[0] + n * (ci[1] + n * ci[2]), off, vf, m);
 }
 

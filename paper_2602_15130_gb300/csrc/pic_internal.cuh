@@ -484,6 +484,15 @@ __device__ __forceinline__ double poly7(const double* table, int k, double u) {
   return fma(fma(fma(fma(fma(fma(fma(q3.y, u, q3.x), u, q2.y), u, q2.x), u, q1.y), u, q1.x), u, q0.y), u, q0.x);
 }
 
+__device__ __forceinline__ double wrap_unit(double x) {
+  double y = x - floor(x);
+  return y >= 1.0 ? 0.0 : y;
+}
+
+// More than a value of xm_table, or of normal_quantile in units of its size
+// and one, is off that of the general path: 14e-15, ten times their errors.
+constexpr double kTableTol = 0x1p-46;
+
 // x^M of xm_solve by table: 14 FP64 instructions instead of 75 (a Hermite
 // start, a sincospi, two divisions), which bound sampling and norms.
 __device__ __forceinline__ double xm_table(const Params& P, const TimeTerms& tt, double xi) {
@@ -509,6 +518,41 @@ __device__ __forceinline__ double normal_quantile(const Params& P, double xi) {
   const double mid = __hiloint2double((hi & ~0x3fff) | 0x2000, 0);
   const double z = poly7(P.ginv + 2 * (P.ginv_M + 1) + kXmDoubles, k, q - mid);
   return xi < 0.5 ? z : -z;
+}
+
+// Sampling of the precision form, the general path's floats bit for bit: the
+// tables' value where every value within their error rounds to the same float
+// (all but one in a million), else the general path.
+//
+// (float)(mean + sigma Phi^{-1}(xi))
+__device__ __forceinline__ float vm_sample32(const Params& P, int d, double xi) {
+  const double z = normal_quantile(P, xi);
+  const double v = fma(P.vsig, z, P.vmean[d]), tol = kTableTol * fma(P.vsig, fabs(z), fabs(P.vmean[d]) + P.vsig);
+  const float a = (float)(v - tol), b = (float)(v + tol);
+  return a == b ? a : (float)(P.vmean[d] + P.vsig * normcdfinv(xi));
+}
+// cell and offset, in cells, of x in [0, 1)
+__device__ __forceinline__ int cell_offset32(double x, int n, float* off) {
+  const int c = cell_coord(x, n);
+  const float o = (float)fma(x, (double)n, -(double)c);
+  *off = o >= 1.f ? 0x1.fffffep-1f : (o < 0.f ? 0.f : o);
+  return c;
+}
+// those of x^M
+__device__ __forceinline__ int xm_sample32(const Params& P, const TimeTerms& tt, double xi, float* off) {
+  const int n = P.n;
+  const double x = xm_table(P, tt, xi);
+  const double f = x - floor(x);
+  const double u = f * (double)n, c = floor(u), o = u - c;
+  // x n carries the error n times, and its rounding
+  const double tol = kTableTol * (double)n * (1.0 + fabs(tt.ct));
+  const float a = (float)(o - tol), b = (float)(o + tol);
+  if (a == b && o > tol && o + tol < 1.0) {
+    *off = a >= 1.f ? 0x1.fffffep-1f : a;
+    return (int)c;
+  }
+  double s;
+  return cell_offset32(wrap_unit(xm_solve(P, tt, xi, &s)), n, off);
 }
 
 // floor of 0 <= t < 2^31 without a conversion instruction (FP64 conversions
@@ -629,11 +673,6 @@ __device__ __forceinline__ int32_t cell_slot(int32_t* count, int32_t key) {
   if (lane == leader) base = atomicAdd(count + key, __popc(peers));
   base = __shfl_sync(act, base, leader);
   return base + __popc(peers & ((1u << lane) - 1u));
-}
-
-__device__ __forceinline__ double wrap_unit(double x) {
-  double y = x - floor(x);
-  return y >= 1.0 ? 0.0 : y;
 }
 
 }  // namespace pic

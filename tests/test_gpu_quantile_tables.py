@@ -58,3 +58,34 @@ def test_sample_and_norms(A, c, t0):
     dv = vm - v
     want = np.concatenate([np.sqrt((dx ** 2).mean(0)), np.sqrt((dv ** 2).mean(0))])
     assert np.all(np.abs(em[:6] - want) <= 1e-6 * want + 4 * bound)
+
+
+@pytest.mark.parametrize("n,N,A,t0,mean", [(8, 200000, 0.3, 0.0, 0.2), (7, 200000, 0.3, 3.3, 0.0), (96, 400000, -0.3, 0.7, 0.2),
+                                           (16, 100000, 0.9, 0.1, 0.2)])
+def test_precision_sample_is_the_rounded_quantile(n, N, A, t0, mean):
+    """The precision form samples cell and FP32 offset of x^M and the FP32 v^M:
+    what rounding the FP64 form's values (equal to 1e-14) gives, to within one
+    rounding wherever that difference can decide it."""
+    import __graft_entry__ as g
+
+    g.build()
+    p = workloads.base(n, N, 0.01, 0, 1.0, fx_amp=A, seed=3, v_mean=(mean,) * 3, max_ppc=2048)
+    with Pic(p) as s:
+        s.sample_mms(t0)
+        x, v = s.get_state()
+    with Pic(workloads.mixed(p)) as s:
+        s.sample_mms(t0)
+        xm, vm = s.get_state()
+    tol = 2e-14
+    lo, hi = (v - tol * (1 + np.abs(v))).astype(np.float32), (v + tol * (1 + np.abs(v))).astype(np.float32)
+    assert np.all((vm >= lo) & (vm <= hi))
+    u = x * n
+    c = np.floor(u)
+    o = u - c
+    inside = (o > 1e-9) & (o < 1 - 1e-7)
+    lo, hi = (o - tol * n).astype(np.float32), (o + tol * n).astype(np.float32)
+    om = xm * n - c
+    # the state is the cell plus the offset times h: three roundings at most
+    slack = 4 * U * n
+    assert np.all(((om >= lo.astype(float) - slack) & (om <= hi.astype(float) + slack))[inside])
+    assert inside.mean() > 0.999
