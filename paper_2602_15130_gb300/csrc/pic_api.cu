@@ -1037,11 +1037,15 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
   // four warps a cell: 12^3 cells of 101, K = 243: 342, 191, 134; 16^3 of 320,
   // K = 1,024: 3,600, 2,200, 1,640; 8^3 of 16, K = 40: 28, 18, 20; 32^3 of 128,
   // K = 192: 602, 501, 536; 24^3 of 100, K = 200: 309, 280, 257; and of 32
-  // particles 32^3, K = 96: 124, 140, 153; 48^3, K = 64: 246, 260, 387.
+  // particles 32^3, K = 96: 124, 140, 153; 48^3, K = 64: 246, 260, 387. Three
+  // chunks leave one of two warps idle in every second round: four warps, from
+  // three words on (24^3, K = 75, cells of 107: 150, 149, 135; 28^3 of 64: 130,
+  // 140, 137).
   const int chunks = (K + 31) / 32;
   c->dsmc_team = 0;
   if (c->mixed && chunks > 1) {
     if (c->P.ncell < (int64_t)72 * c->num_sms) c->dsmc_team = chunks == 2 ? 2 : 4;
+    else if (chunks == 3) c->dsmc_team = c->P.np > 96 * c->P.ncell ? 4 : 0;
     else if (c->P.np > 48 * c->P.ncell) c->dsmc_team = chunks < 7 ? 2 : 4;
   }
   c->dsmc_block = c->mixed ? dsmc32_threads(c->dsmc_team) : dsmc_threads();
