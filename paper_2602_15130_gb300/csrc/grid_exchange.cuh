@@ -12,7 +12,9 @@
 // hops), 11.8 us with an atomic counter and 8.4 us by inboxes.
 //
 // kData: the exchange also orders the blocks' global writes before it ahead
-// of the others' reads after it (2,000 of its 7,000 SM cycles).
+// of the others' reads after it (2,000 of its 7,000 SM cycles). Without it an
+// exchange still orders a block's reads before it ahead of the others' writes
+// after it where the values read went into the sum.
 //
 // The inboxes alternate between two sets: a block can be one exchange ahead
 // of another, never two. Waits are bounded (4e9 SM cycles, about 2 s): then
@@ -90,10 +92,10 @@ struct GridExchange {
         mine[q] = (unsigned long long)__double_as_longlong(warp_sum_d(s));
       }
     }
-    if (kData) {
-      if (t == 0) fence_gpu();
-      __syncwarp();
-    }
+    // Every publishing lane fences for itself: a release is a fence and the
+    // store that follows it in the same thread (lane t's slots are what the
+    // blocks t, t + 32, ... read).
+    if (kData) fence_gpu();
 #pragma unroll
     for (int q = 0; q < kV; ++q)
       for (int i = t; i < G; i += 32) slot_put(set + ((size_t)q * G + i) * G + blockIdx.x, mine[q], number);
