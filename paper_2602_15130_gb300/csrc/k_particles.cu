@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(kThreads) k_store_dv(StoreDvArgs a) {
 // What bounds it is the FP64 pipe (two lanes an SM and clock), so as little
 // as possible runs there, and that by full warps:
 //  - the accept test runs in FP32 on a copy of the group's velocities in
-//    shared memory, with a bound on its error; the one candidate in a
-//    million it cannot decide is decided in FP64 as the paper writes it
-//    (ntc_decide64), so every decision is the FP64 one;
+//    shared memory, free of units, with a bound on its error; the one
+//    candidate in a million it cannot decide is decided in FP64 as the paper
+//    writes it (ntc_decide64), so every decision is the FP64 one;
 //  - one candidate in eight is accepted: the lanes only test their
 //    candidates and put the accepted pairs into a queue of the warp, which is
 //    scattered 32 pairs at a time, whichever lanes they came from. A
@@ -156,8 +156,38 @@ __global__ void __launch_bounds__(kThreads) k_store_dv(StoreDvArgs a) {
 // bytes of its list's indices (0xff: unused), so that in cells of up to 255
 // particles an entry is found by one zero-byte search.
 // --------------------------------------------------------------------------
+// Constants of the FP32 accept test (ntc_test32)
+struct Test32 {
+  double scale;         // of the velocities: 1, or a power of two
+  int scaled;           // it is not 1
+  float inv_gmax2;      // 1 / (scale g_max)^2
+  float err;            // 2^-19 of it
+  float tie;            // what a near tie (1e-12 in U) amounts to where U is below 1e-6
+  float c0, c1, c2;     // sigma_k g_max^2k / (sigma g)_max
+  int n_sigma;
+};
+
+// The velocities keep their units while g_max lies within 2^+-32; beyond, a power
+// of two brings it there.
+Test32 test32_of(const Params& P) {
+  Test32 T;
+  const int e = ilogb(P.gmax);
+  T.scaled = abs(e) > 32;
+  T.scale = T.scaled ? ldexp(1.0, -e) : 1.0;
+  const double g = P.gmax * T.scale, g2 = P.gmax * P.gmax;
+  T.inv_gmax2 = (float)(1.0 / (g * g));
+  T.err = 0x1p-19f * T.inv_gmax2;
+  T.n_sigma = P.n_sigma;
+  T.tie = P.n_sigma == 0 ? 2e-18f : 2e-12f;
+  T.c0 = (float)(P.sigma_n[0] / P.sg_max);
+  T.c1 = (float)(P.sigma_n[1] * g2 / P.sg_max);
+  T.c2 = (float)(P.sigma_n[2] * (g2 * g2) / P.sg_max);
+  return T;
+}
+
 struct DsmcArgs {
   Params P;
+  Test32 T;
   const double *v0, *v1, *v2;
   const int32_t* start;
   uint32_t c0;
@@ -224,48 +254,60 @@ __device__ __forceinline__ int list_find(const ListEntry* wl, int t, int p) {
   return k;
 }
 
-// FP32 constants of the test
-struct Test32 {
-  float gmax, gmax2, sgmax, s0, s1, s2;
-  float tie;  // what a near tie (1e-12 in U) amounts to where U is below 1e-6
-  int n_sigma;
-};
-
-// The same decision from FP32 velocities (each the FP64 one rounded): 0 or
-// 1, or -1 where FP64 has to decide. With S = sum (v_p^2 + v_q^2) the
-// components' differences are off by at most 2^-23 (|v_p| + |v_q|), g^2 by
-// less than 2^-20 S, and the squared threshold by less than 2^-20 of itself;
-// the margin is twice both. g^2 near or above g_max^2 is left to FP64 too
-// (its flag), and so is anything not finite (no comparison with it holds).
-// Odd-power sigma: the same through its derivative.
+// The same decision from FP32 velocities (each the FP64 one, in units of
+// 1 / T.scale, rounded): 0 or 1, or -1 where FP64 has to decide. The test is
+// on y = g^2 / g_max^2: U^2 < y, or for the odd-power sigma U < c0 + c1 y +
+// c2 y^2. With S = sum (v_p^2 + v_q^2) the components' differences are off by at
+// most 2^-23 (|v_p| + |v_q|), so y by less than 2^-19 S / g_max^2, the
+// margin, and U^2 by less than 2^-20 of itself. y near or above one is left to
+// FP64 too (its flag), and so is anything not finite (no comparison with it
+// holds). Odd-power sigma: the same through its derivative.
+//
+// Nothing that matters lies below FP32's normal range whatever the units: U,
+// y and c_k are numbers near one, g_max is within 2^+-32 of one in the units
+// of the velocities (test32_of), so a subnormal square is 2^-85 of
+// g_max^2 or less, and the near-tie term covers that.
 __device__ __forceinline__ int ntc_test32(const Test32& T, uint32_t w, const float4& a, const float4& b) {
   const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
-  const float g2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float S = a.w + b.w;  // |v_p|^2 + |v_q|^2
+  const float y = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) * T.inv_gmax2;
   const float U = fmaf((float)w, 0x1p-32f, 0x1p-33f);
-  const float e2 = fmaf(0x1p-19f, S, T.tie);
+  const float e = fmaf(T.err, a.w + b.w, T.tie);  // (|v_p|^2 + |v_q|^2)
   float lhs, rhs, margin;
   if (T.n_sigma == 0) {
-    const float ug = U * T.gmax;
-    lhs = ug * ug;
-    rhs = g2;
-    margin = fmaf(0x1p-19f, lhs, e2);
+    lhs = U * U;
+    rhs = y;
+    margin = fmaf(0x1p-19f, lhs, e);
   } else {
-    lhs = U * T.sgmax;
-    rhs = fmaf(fmaf(T.s2, g2, T.s1), g2, T.s0);
-    const float d = fmaf(2.f * fabsf(T.s2), g2 + e2, fabsf(T.s1));
-    margin = fmaf(d, e2, fmaf(0x1p-19f, lhs + fabsf(T.s0) + g2 * d, T.tie));
+    lhs = U;
+    rhs = fmaf(fmaf(T.c2, y, T.c1), y, T.c0);
+    const float d = fmaf(2.f * fabsf(T.c2), y + e, fabsf(T.c1));
+    margin = fmaf(d, e, fmaf(0x1p-19f, lhs + fabsf(T.c0) + y * d, T.tie));
   }
-  if (fabsf(lhs - rhs) > margin && g2 + e2 < T.gmax2) return lhs < rhs ? 1 : 0;
+  if (fabsf(lhs - rhs) > margin && y + e < 1.f) return lhs < rhs ? 1 : 0;
   return -1;
+}
+
+// An FP64 velocity as the test takes it. The scaling is a call: in line, the
+// multiplications take the FP64 pipe, predicated off as they are, also where
+// there is none to do (12^3 cells of 101, K = 243: 1.37 ms a call, 1.19 so).
+__device__ __noinline__ float4 rounded_scaled(double s, double x, double y, double z) {
+  float4 f = make_float4((float)(x * s), (float)(y * s), (float)(z * s), 0.f);
+  f.w = fmaf(f.x, f.x, fmaf(f.y, f.y, f.z * f.z));
+  return f;
+}
+__device__ __forceinline__ float4 rounded(const Test32& T, double x, double y, double z) {
+  if (T.scaled) return rounded_scaled(T.scale, x, y, z);
+  float4 f = make_float4((float)x, (float)y, (float)z, 0.f);
+  f.w = fmaf(f.x, f.x, fmaf(f.y, f.y, f.z * f.z));
+  return f;
 }
 
 // Algorithm 1 for the warp's (cell, outcome) lanes: outcome o of cell `cell`
 // (particles off .. off + c - 1) where run is set.
 template <bool kVerify>
-__device__ __forceinline__ void ntc_warp64(const DsmcArgs& a, const Test32& T, uint32_t cell, uint32_t o, int off,
-                                           int c, bool run, int lane, Warp64& W, const float4* stage, int gs,
-                                           uint32_t* mask, double* wov, Counts64& cnt) {
+__device__ __forceinline__ void ntc_warp64(const DsmcArgs& a, uint32_t cell, uint32_t o, int off, int c, bool run,
+                                           int lane, Warp64& W, const float4* stage, int gs, uint32_t* mask,
+                                           double* wov, Counts64& cnt) {
   const Params& P = a.P;
   const DLog& lg = a.lg;
   const uint32_t c0 = a.c0;
@@ -325,11 +367,6 @@ __device__ __forceinline__ void ntc_warp64(const DsmcArgs& a, const Test32& T, u
       const double* e = k < kList ? W.list[32 * k + l].v : wov + ((size_t)l * a.max_ppc + x) * 3;
       v[0] = e[0]; v[1] = e[1]; v[2] = e[2];
     }
-  };
-  auto rounded = [](const double* v) {
-    float4 f = make_float4((float)v[0], (float)v[1], (float)v[2], 0.f);
-    f.w = fmaf(f.x, f.x, fmaf(f.y, f.y, f.z * f.z));
-    return f;
   };
   for (;;) {
     const bool go = s < np && !stuck;
@@ -419,12 +456,12 @@ __device__ __forceinline__ void ntc_warp64(const DsmcArgs& a, const Test32& T, u
         if (s < np) b0 = philox(c0, cell, (uint32_t)s, o << 8, P.key0, P.key1);
         int d = -1;
         if (stage && kp < 0 && kq < 0) {
-          d = ntc_test32(T, wz, stage[off - gs + (int)p], stage[off - gs + (int)q]);
+          d = ntc_test32(a.T, wz, stage[off - gs + (int)p], stage[off - gs + (int)q]);
         } else {
           double vp[3], vq[3];
           velocity((int)p, kp, lane, off, vp);
           velocity((int)q, kq, lane, off, vq);
-          d = ntc_test32(T, wz, rounded(vp), rounded(vq));
+          d = ntc_test32(a.T, wz, rounded(a.T, vp[0], vp[1], vp[2]), rounded(a.T, vq[0], vq[1], vq[2]));
         }
         if (d < 0) {
           double vp[3], vq[3];
@@ -529,9 +566,6 @@ __global__ void __launch_bounds__(kDsmcThreads, 16) k_dsmc(DsmcArgs a) {
   __syncwarp();
   Counts64 cnt = {0u, 0u, 0u, 0u};
   const double invK = 1.0 / (double)P.K;
-  const Test32 T = {(float)P.gmax, (float)(P.gmax * P.gmax), (float)P.sg_max, (float)P.sigma_n[0],
-                    (float)P.sigma_n[1], (float)P.sigma_n[2],
-                    P.n_sigma == 0 ? (float)(2e-18 * P.gmax * P.gmax) : (float)(2e-12 * P.sg_max), P.n_sigma};
 
   for (int64_t take = blockIdx.x;; take += gridDim.x) {
     int64_t item = take;
@@ -565,10 +599,7 @@ __global__ void __launch_bounds__(kDsmcThreads, 16) k_dsmc(DsmcArgs a) {
     const bool use_stage = gn <= a.stage;
     __syncwarp();
     if (use_stage)
-      for (int i = lane; i < gn; i += 32) {
-        const float x = (float)a.v0[gs + i], y = (float)a.v1[gs + i], z = (float)a.v2[gs + i];
-        staged[i] = make_float4(x, y, z, fmaf(x, x, fmaf(y, y, z * z)));
-      }
+      for (int i = lane; i < gn; i += 32) staged[i] = rounded(a.T, a.v0[gs + i], a.v1[gs + i], a.v2[gs + i]);
     __syncwarp();
     for (int ch = ch0; ch < ch1; ++ch) {
       const int o = ch * a.Kc + lane % a.Kc;
@@ -577,7 +608,7 @@ __global__ void __launch_bounds__(kDsmcThreads, 16) k_dsmc(DsmcArgs a) {
         atomicOr(a.flags, 1);
         run = false;
       }
-      ntc_warp64<kVerify>(a, T, (uint32_t)(cell0 + mycl), (uint32_t)o, s, c, run, lane, W,
+      ntc_warp64<kVerify>(a, (uint32_t)(cell0 + mycl), (uint32_t)o, s, c, run, lane, W,
                           use_stage ? staged : nullptr, gs, mask, wov, cnt);
       // sum this chunk's changes per particle in ascending outcome order
       const bool last = ch == a.nchunks - 1 && a.parts == 1;
@@ -1010,6 +1041,7 @@ cudaError_t launch_dsmc(pic_ctx* c, uint32_t c0, bool separate, double t_src) {
   a.Kc = c->dsmc_Kc;
   a.nchunks = (c->P.K + c->dsmc_Kc - 1) / c->dsmc_Kc;
   a.stage = c->dsmc_stage;
+  a.T = test32_of(c->P);
   a.ngroups = c->dsmc_groups;
   a.parts = c->dsmc_parts;
   a.partial = c->dsmc_partial;
