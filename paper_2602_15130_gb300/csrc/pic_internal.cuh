@@ -290,12 +290,41 @@ __device__ __forceinline__ double xm_dot(const Params& P, const TimeTerms& tt, d
 // PIC_DIST_PAPER: x_d^M(t) solves F_{x_d}(x, t) = xi for f_{x_d} = 1 + A
 // sin(2 pi (x - s)), A and s varying in time. With y = x - s the equation
 // is G(y) = y - A/(2 pi) cos(2 pi y) = T, T = xi - s - A/(2 pi) cos(2 pi s)
-// (G' = 1 + A sin >= 1 - |A| > 0, root within |A|/(2 pi) of T). y - T is
-// found in FP32 first: Newton inside a bracket that every step narrows, to
-// about 1e-8. One FP64 Newton step leaves 2 pi A (1e-8)^2, and a second one
-// with sin and cos carried over to the new point by their Taylor expansions
-// (dy^3 < 1e-23) leaves rounding: one FP64 sincospi where Newton from y = T
-// took seven. Returns x^M = y + s, with sin and cos of 2 pi y.
+// (G' = 1 + A sin >= 1 - |A|, root within |A|/(2 pi) of T).
+
+// Newton in FP64 from y, kept inside a bracket that every step narrows
+// (bisection where a step leaves it), to rounding.
+static __device__ __noinline__ double xm_newton(double A, double T, double y, double* sy, double* cy) {
+  const double a2p = A * (1.0 / kTwoPi), r = fabs(a2p);
+  double lo = T - r, hi = T + r;
+  for (int it = 0; it < 64; ++it) {
+    double s, c;
+    sincospi(2.0 * y, &s, &c);
+    const double G = y - a2p * c - T;
+    if (G == 0.0) break;
+    if (G < 0.0) lo = y; else hi = y;
+    double yn = y - G / (1.0 + A * s);
+    if (!(yn > lo && yn < hi)) yn = 0.5 * (lo + hi);
+    const bool done = fabs(yn - y) <= 0x1p-52;
+    y = yn;
+    if (done) break;
+  }
+  sincospi(2.0 * y, sy, cy);
+  return y;
+}
+
+// y - T is found in FP32 first: Newton inside a narrowing bracket, to some
+// 1e-7 / G'. One FP64 Newton step leaves its square, and a second one with sin
+// and cos carried over to the new point by their Taylor expansions leaves
+// rounding: one FP64 sincospi where Newton from y = T took seven. Where the
+// steps are too long for that (the first above 1e-6, whose cube is the
+// expansions' error, or the second above 1e-9, whose square is what remains),
+// and for |A| >= 1 (G not monotone), xm_newton takes over. Emulated on the CPU,
+// the result is off by at most 1.4 times 2^-52 / G' for A up to 0.999999; xm_newton
+// is needed by no value up to A = 0.8 and half of those close to the flattest
+// point at 0.999, where the two steps alone left 3,000 times that.
+//
+// Returns x^M = y + s, with sin and cos of 2 pi y.
 __device__ __forceinline__ double xm_solve_gen(const TimeTerms& tt, int d, double xi, double* sy, double* cy) {
   const double A = tt.fA[d], a2p = A * (1.0 / kTwoPi);
   const double T = xi - tt.fs[d] - a2p * tt.fcs[d];
@@ -319,15 +348,19 @@ __device__ __forceinline__ double xm_solve_gen(const TimeTerms& tt, int d, doubl
   }
   double s, c;
   sincospi(2.0 * y, &s, &c);
+  bool near = fabs(A) < 1.0;
+  const double y0 = near ? y : T;
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const double dy = (y - a2p * c - T) / (1.0 + A * s);
+    near = near && fabs(dy) <= (it == 0 ? 0x1p-20 : 0x1p-30);
     y -= dy;
     const double e = -kTwoPi * dy, e2 = 0.5 * e * e;
     const double s1 = fma(c, e, s) - e2 * s;
     c = fma(-s, e, c) - e2 * c;
     s = s1;
   }
+  if (!near) y = xm_newton(A, T, y0, &s, &c);
   *sy = s;
   *cy = c;
   return y + tt.fs[d];
