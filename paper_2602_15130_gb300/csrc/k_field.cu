@@ -175,7 +175,15 @@ __device__ __forceinline__ Nbr neighbours(int id, int i, int j, int k, int n, in
 // over every SM, one block each, with as few threads as hold them (32 at
 // least), npt nodes a thread in registers (1, 2, 4 or 8; 0: more than that,
 // the vectors stay in memory).
+//
+// With the vectors in memory (n >= 86 on 152 SMs) a solve is bound by L2: 1,024
+// threads for the loads in flight, and the grid's threads on consecutive nodes,
+// so that the blocks' stencils meet in L2 at the same time. us an iteration at
+// 86^3, 100^3, 128^3 and 144^3: 27.3, 34.8, 59.1, 88.4; with 512 threads and a
+// contiguous range a block 28.1, 38.4, 70.6, 117; with 1,024 and ranges 26.6,
+// 34.3, 60.7, 95.1. Loads through L1 made no difference.
 constexpr int kCgThreads = 512;
+constexpr int kCgThreadsMem = 1024;
 
 struct CgShape {
   int npt, threads, grid;
@@ -186,7 +194,7 @@ inline CgShape cg_shape(int64_t m, int sms) {
   const int64_t per = (m + sms - 1) / sms;  // nodes an SM
   s.npt = per <= kCgThreads ? 1 : per <= 2 * kCgThreads ? 2 : per <= 4 * kCgThreads ? 4 : per <= 8 * kCgThreads ? 8 : 0;
   if (s.npt == 0) {
-    s.threads = kCgThreads;
+    s.threads = kCgThreadsMem;
     s.grid = sms;
     return s;
   }
@@ -220,10 +228,10 @@ __device__ __forceinline__ bool done(double bb, double rr, double thresh, double
 }
 
 template <int NPT>
-__global__ void __launch_bounds__(kCgThreads) k_cg(CgArgs a) {
+__global__ void __launch_bounds__(NPT > 0 ? kCgThreads : kCgThreadsMem) k_cg(CgArgs a) {
   constexpr bool kRegs = NPT > 0, kRecompute = NPT == 1;
   constexpr int kN = kRegs ? NPT : 1;
-  __shared__ double sh[2 * kCgThreads];
+  __shared__ double sh[2 * (kRegs ? kCgThreads : kCgThreadsMem)];
   __shared__ double scal[2];  // scalars formed once per block by thread 0
   __shared__ int stop, ok_sh;
   // the others then wait for an arrival that never comes, until the bound
@@ -231,9 +239,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg(CgArgs a) {
   const int n = a.n, nn = a.n * a.n;
   const int m = (int)a.ncell;
   const int t = threadIdx.x, T = blockDim.x, G = gridDim.x;
-  const int chunk = kRegs ? NPT * T : (m + G - 1) / G;
-  const int64_t lo64 = (int64_t)blockIdx.x * chunk;
-  const int lo = (int)(lo64 < m ? lo64 : m), hi = lo64 + chunk < m ? (int)(lo64 + chunk) : m;
+  const int64_t lo64 = (int64_t)blockIdx.x * (NPT * T);  // (in registers: the block's nodes)
+  const int lo = (int)(lo64 < m ? lo64 : m), hi = lo64 + NPT * T < m ? (int)(lo64 + NPT * T) : m;
   GridExchange X{a.slots, G, a.launch, 0u, a.info + 2, a.flags, &ok_sh};
   double xr[kN], rr_[kN], pr[kN], qr[kN];
   int ijk[kN];  // the node's coordinates, 10 bits each
@@ -247,7 +254,10 @@ __global__ void __launch_bounds__(kCgThreads) k_cg(CgArgs a) {
         if (id < hi) f(k, id, ijk[k] & 1023, (ijk[k] >> 10) & 1023, ijk[k] >> 20);
       }
     } else {
-      for (int id = lo + t; id < hi; id += T) f(0, id, id % n, (id / n) % n, id / nn);
+      for (int64_t i = (int64_t)blockIdx.x * T + t; i < m; i += G * T) {
+        const int id = (int)i;
+        f(0, id, id % n, (id / n) % n, id / nn);
+      }
     }
   };
   if constexpr (kRegs) {
