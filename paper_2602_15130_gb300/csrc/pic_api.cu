@@ -408,9 +408,29 @@ pic_status cuda_status(cudaError_t e) {
   return PIC_ECUDA;
 }
 
+// Device memory, aligned to kAlign bytes: the widest load or store of the
+// kernels. A caller's allocator may hand out smaller granules: each of its
+// blocks has room to round the start up, and where that moves it the
+// allocator's own address is kept for the release.
+constexpr size_t kAlign = 32;
+
 void* dev_alloc(pic_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 16;
-  if (c->have_alloc) return c->alloc.alloc(c->alloc.user, (uint64_t)bytes);
+  if (c->have_alloc) {
+    void* raw = c->alloc.alloc(c->alloc.user, (uint64_t)(bytes + kAlign));
+    void* p = (void*)(((uintptr_t)raw + kAlign - 1) / kAlign * kAlign);
+    if (p == raw) return p;  // (or nullptr)
+    void** moved = (void**)realloc(c->moved, sizeof(void*) * 2 * (size_t)(c->n_moved + 1));
+    if (!moved) {
+      c->alloc.free(c->alloc.user, raw);
+      return nullptr;
+    }
+    c->moved = moved;
+    c->moved[2 * c->n_moved] = p;
+    c->moved[2 * c->n_moved + 1] = raw;
+    c->n_moved++;
+    return p;
+  }
   void* p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -421,8 +441,19 @@ void* dev_alloc(pic_ctx* c, size_t bytes) {
 
 void dev_free(pic_ctx* c, void* p) {
   if (!p) return;
-  if (c->have_alloc) c->alloc.free(c->alloc.user, p);
-  else cudaFree(p);
+  if (c->have_alloc) {
+    for (int i = 0; i < c->n_moved; ++i) {
+      if (c->moved[2 * i] != p) continue;
+      p = c->moved[2 * i + 1];
+      c->n_moved--;
+      c->moved[2 * i] = c->moved[2 * c->n_moved];
+      c->moved[2 * i + 1] = c->moved[2 * c->n_moved + 1];
+      break;
+    }
+    c->alloc.free(c->alloc.user, p);
+  } else {
+    cudaFree(p);
+  }
 }
 
 #define CK(expr)                                   \
@@ -967,6 +998,7 @@ void pic_destroy(pic_ctx* c) {
   for (int i = 0; i < 2 * c->ev_cap; ++i) cudaEventDestroy(c->ev_pool[i]);
   free(c->ev_pool);
   free(c->ev_class);
+  free(c->moved);
   delete c;
 }
 

@@ -725,6 +725,8 @@ struct pic_ctx {
   int device, num_sms;
   pic_allocator alloc;
   bool have_alloc;
+  void** moved;     // blocks of it whose start was rounded up: (our address, its own)
+  int n_moved;
 
   bool mixed;       // precision form (PIC_MIXED)
 
