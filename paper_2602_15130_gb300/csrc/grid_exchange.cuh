@@ -1,4 +1,5 @@
-// Sums over the blocks of a co-resident grid, for the CG kernels.
+// Sums over the blocks of a co-resident grid, and launches of one cluster, for
+// the CG kernels.
 //
 // One exchange is a reduction and a grid barrier in one: warp 0 of a block
 // writes the block's partial, with the exchange's number in the same 16-byte
@@ -140,6 +141,36 @@ struct GridExchange {
       }
       *ok = good ? 1 : 0;
     }
+  }
+};
+
+// A launch of one thread-block cluster.
+struct ClusterLaunch {
+  cudaLaunchAttribute at = {};
+  cudaLaunchConfig_t cfg = {};
+  ClusterLaunch(int blocks, int threads, cudaStream_t stream) {
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)blocks;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+  }
+  ClusterLaunch(const ClusterLaunch&) = delete;
+
+  // Whether the SMs that this process and stream may use hold it. Sixteen
+  // blocks need most of a GPC; where a process gets a share of the SMs they may
+  // not fit, and the solve takes the grid.
+  bool fits(const void* fn) const {
+    int n = 0;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
+    if (e == cudaSuccess) return n > 0;
+    cudaGetLastError();
+    return false;
   }
 };
 

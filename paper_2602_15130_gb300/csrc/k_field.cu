@@ -609,29 +609,17 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_cluster(CgArgs a) {
   cluster_barrier();  // no block leaves while another reads its shared memory
 }
 
-// Launch the solve: one cluster where the mesh is small, else a cooperative
+int cluster_threads(int64_t m) { return (int)(((m + kClusterBlocks - 1) / kClusterBlocks + 31) / 32 * 32); }
+
+// Launch the solve: on one cluster (cg_cluster_fits), else on a cooperative
 // grid over the SMs (always with a failure injection, whose wait is bounded
 // there).
-cudaError_t launch_solve(const CgArgs& args, int sms, cudaStream_t stream) {
+cudaError_t launch_solve(const CgArgs& args, bool cluster, int sms, cudaStream_t stream) {
   CgArgs a = args;
   void* argv[] = {&a};
-  if (a.ncell <= kClusterNodes && a.skip_block < 0) {
-    const int64_t per = (a.ncell + kClusterBlocks - 1) / kClusterBlocks;
-    const void* fn = (const void*)k_cg_cluster;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kClusterBlocks;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kClusterBlocks);
-    cfg.blockDim = dim3((unsigned)((per + 31) / 32 * 32));
-    cfg.stream = stream;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, fn, argv);
+  if (cluster && a.skip_block < 0) {
+    const ClusterLaunch l(kClusterBlocks, cluster_threads(a.ncell), stream);
+    return cudaLaunchKernelExC(&l.cfg, (const void*)k_cg_cluster, argv);
   }
   const CgShape s = cg_shape(a.ncell, sms);
   return cudaLaunchCooperativeKernel(cg_kernel(s.npt), dim3(s.grid), dim3(s.threads), argv, 0, stream);
@@ -693,6 +681,9 @@ cudaError_t launch_rhs(pic_ctx* c, double t) {
   return cudaGetLastError();
 }
 
+bool cg_cluster_fits(int64_t m, cudaStream_t stream) {
+  return m <= kClusterNodes && ClusterLaunch(kClusterBlocks, cluster_threads(m), stream).fits((const void*)k_cg_cluster);
+}
 int cg_blocks(int64_t m, int sms) { return cg_shape(m, sms).grid; }
 // bytes of the exchange inboxes a context of this grid holds
 size_t cg_slot_bytes(int grid) { return exchange_slots((size_t)grid) * sizeof(GridSlot); }
@@ -726,7 +717,7 @@ cudaError_t launch_cg_on(pic_ctx* c, const double* b, double* x, const double* r
   a.hist = c->hist_row;
   c->stall_next_cg = false;
   prof_begin(c);
-  cudaError_t e = launch_solve(a, c->num_sms, c->stream);
+  cudaError_t e = launch_solve(a, c->cg_cluster, c->num_sms, c->stream);
   prof_end(c, KC_CG);
   c->launches++;
   if (e != cudaSuccess) return e;
@@ -864,7 +855,7 @@ extern "C" pic_status pic_poisson_solve_noalloc(int32_t n, const double* b, doub
   a.E2 = E + 2 * m;
   // the array keeps the last call's contents: clear the status words
   cudaError_t e = cudaMemsetAsync(words, 0, 8 * sizeof(int), stream);
-  if (e == cudaSuccess) e = launch_solve(a, sms, stream);
+  if (e == cudaSuccess) e = launch_solve(a, cg_cluster_fits(m, stream), sms, stream);
   int info[3] = {0, 0, 0};
   double r = 0.0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(info, words, sizeof(info), cudaMemcpyDeviceToHost, stream);

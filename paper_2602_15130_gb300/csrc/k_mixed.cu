@@ -9,6 +9,7 @@
 // error-free TwoSum / TwoProd of Knuth and Dekker, relative error about
 // 2^-44) on the FP32 pipe, within and across blocks; the CG's scalar
 // recurrences and the error norms are true FP64.
+#include "grid_exchange.cuh"
 #include "mixed_common.cuh"
 
 namespace pic {
@@ -1624,29 +1625,18 @@ __global__ void __launch_bounds__(kCgThreads) k_cg32_cluster(Cg32Args a) {
   cluster_barrier();  // no block leaves while another reads its shared memory
 }
 
-cudaError_t launch_cg32_cluster(const Cg32Args& args, cudaStream_t stream) {
-  Cg32Args a = args;
-  const int C = a.ncell <= 1024 ? 4 : a.ncell <= 2048 ? 8 : kClusterBlocks;
-  const int per = (int)((a.ncell + C - 1) / C);
+struct Cluster32 {
+  int blocks, threads;
+  const void* fn;
+};
+Cluster32 cg32_cluster(int64_t m) {
+  const int C = m <= 1024 ? 4 : m <= 2048 ? 8 : kClusterBlocks;
+  const int per = (int)((m + C - 1) / C);
   const int npt = per <= kCgThreads ? 1 : per <= 2 * kCgThreads ? 2 : 4;
-  const void* fn = npt == 1   ? (const void*)k_cg32_cluster<1>
-                   : npt == 2 ? (const void*)k_cg32_cluster<2>
-                              : (const void*)k_cg32_cluster<4>;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)C;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)C);
-  cfg.blockDim = dim3((unsigned)(((per + npt - 1) / npt + 31) / 32 * 32));
-  cfg.stream = stream;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  void* argv[] = {&a};
-  return cudaLaunchKernelExC(&cfg, fn, argv);
+  return {C, ((per + npt - 1) / npt + 31) / 32 * 32,
+          npt == 1   ? (const void*)k_cg32_cluster<1>
+          : npt == 2 ? (const void*)k_cg32_cluster<2>
+                     : (const void*)k_cg32_cluster<4>};
 }
 
 // ------------------------------------------- multigrid-preconditioned CG --
@@ -2233,6 +2223,11 @@ const void* dsmc32_kernel_ptr(bool verify, int team) {
   return verify ? (const void*)k_dsmc32<true> : (const void*)k_dsmc32<false>;
 }
 int cg32_threads() { return kCgThreads; }
+bool cg32_cluster_fits(int64_t m, cudaStream_t stream) {
+  if (m > kClusterNodes) return false;
+  const Cluster32 k = cg32_cluster(m);
+  return ClusterLaunch(k.blocks, k.threads, stream).fits(k.fn);
+}
 const void* cg32_kernel_ptr() { return (const void*)k_cg32; }
 
 cudaError_t launch_dsmc32(pic_ctx* c, uint32_t c0, bool separate, double t_src) {
@@ -2372,10 +2367,13 @@ cudaError_t launch_cg32(pic_ctx* c) {
   a.skip_block = c->stall_next_cg ? c->cg_grid - 1 : -1;
   a.hist = c->hist_row;
   c->stall_next_cg = false;
-  if (c->mg_nlev == 0 && a.ncell <= kClusterNodes && a.skip_block < 0) {
+  if (c->cg_cluster && a.skip_block < 0) {
     // (a failure injection takes the grid, whose waits are bounded)
+    const Cluster32 k = cg32_cluster(a.ncell);
+    const ClusterLaunch l(k.blocks, k.threads, c->stream);
+    void* argv[] = {&a};
     prof_begin(c);
-    const cudaError_t e = launch_cg32_cluster(a, c->stream);
+    const cudaError_t e = cudaLaunchKernelExC(&l.cfg, k.fn, argv);
     if (e != cudaSuccess) return e;
     prof_end(c, KC_CG);
     c->launches++;

@@ -19,6 +19,8 @@ size_t dsmc_smem_bytes(int max_ppc, int stage);
 const void* dsmc_kernel_ptr(bool verify);
 int cg_blocks(int64_t m, int sms);
 size_t cg_slot_bytes(int grid);
+bool cg_cluster_fits(int64_t m, cudaStream_t stream);
+bool cg32_cluster_fits(int64_t m, cudaStream_t stream);
 int64_t scan_blocks_needed(int64_t ncell);
 int rhs_blocks_needed(int64_t ncell);
 int err_blocks_needed(int64_t np, int64_t ncell);
@@ -1055,6 +1057,8 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
     size_t wf = 0;
     c->mg_nlev = mg_levels(c->P.n, &c->mg_nlev_grid, &wf);
   }
+  c->cg_cluster = c->mixed ? c->mg_nlev == 0 && cg32_cluster_fits(c->P.ncell, c->stream)
+                           : cg_cluster_fits(c->P.ncell, c->stream);
   // collisions: lanes = (cell in group, outcome); bitmaps in shared memory
   const int K = c->cfg.K > 0 ? c->cfg.K : 1;
   c->dsmc_Kc = K < 32 ? K : 32;

@@ -807,6 +807,7 @@ struct pic_ctx {
   int* cg_info;     // [0] iterations, [1] status (0 ok, 1 noconv), [2] timeout
   double* cg_res;   // relative residual
   int cg_grid;
+  bool cg_cluster;  // the solve runs on one cluster of blocks (small meshes, plain CG)
   bool stall_next_cg;  // failure injection: the next CG launch has one block leave before its first barrier
 
   // G^{-1} knot tables (FP64 and FP32)
