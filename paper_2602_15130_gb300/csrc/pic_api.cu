@@ -7,7 +7,6 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <memory>
 #include <utility>
 #include <new>
 
@@ -262,18 +261,22 @@ void quantile_table(double* out) {
   }
 }
 
-// all of the FP64 tables behind the G^{-1} knots; slope: with the kick's
+// the tables that are the same for every context, formed once (in static
+// memory: nothing is thrown at a C entry)
+struct FixedTables {
+  double quantile[kQuantDoubles], r64[kR64Doubles];
+  FixedTables() {
+    quantile_table(quantile);
+    hs_R64_table(r64);
+  }
+};
+
+// all of the tables behind the G^{-1} knots; fp64: with R and the kick's
 bool form_tables(double A, const double* ginv, bool fp64, double* out) {
-  // the same for every context: formed once
-  static const std::unique_ptr<double[]> fixed = [] {
-    std::unique_ptr<double[]> t(new double[kQuantDoubles + kR64Doubles]);
-    quantile_table(t.get());
-    hs_R64_table(t.get() + kQuantDoubles);
-    return t;
-  }();
-  memcpy(out + kXmDoubles, fixed.get(), sizeof(double) * kQuantDoubles);
+  static const FixedTables fixed;
+  memcpy(out + kXmDoubles, fixed.quantile, sizeof(fixed.quantile));
   double* r64 = out + kQuantileDoubles;
-  if (fp64) memcpy(r64, fixed.get() + kQuantDoubles, sizeof(double) * kR64Doubles);
+  if (fp64) memcpy(r64, fixed.r64, sizeof(fixed.r64));
   return kick_tables(A, ginv, fp64 ? r64 + kR64Doubles : nullptr, out);
 }
 
