@@ -322,12 +322,14 @@ pic_status pic_get_state(pic_ctx* ctx, double* x, double* v);
  * Pinned host and device arrays of the context's GPU are read in place.
  * Memory: in the precision form, the first such load (or pic_sample_mms)
  * allocates per-cell bins of the loaded records, ncell x (four times the
- * mean particles per cell, rounded up to 32) x 64 bytes (about five times
+ * mean particles per cell, rounded up to 32) x 48 bytes (about four times
  * the particle state; 32 bytes when that is too much), when they hold at
  * most eight times the loaded records and take at most a quarter of the free
- * device memory; they stay with the context (released by pic_destroy).
- * Without them, or when a cell holds more particles than its bin, the load
- * sorts the same state by a scatter and a random gather. */
+ * device memory, and the first state v^M by pid, 16 bytes a particle, where
+ * that is at most a quarter; both stay with the context (released by
+ * pic_destroy). Without the bins, or when a cell holds more particles than its
+ * bin, the load sorts the same state by a scatter and a random gather; without
+ * the other, each load forms v^M anew. */
 pic_status pic_set_state(pic_ctx* ctx, const double* x, const double* v, double t0,
                          int64_t step);
 

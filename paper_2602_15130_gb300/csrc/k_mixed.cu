@@ -30,18 +30,18 @@ inline int blocks_for(int64_t n, int t = kThreads) {
 // cell keys and arrival ranks. v^M depends only on the pid: it is kept by pid
 // (m0 m1 m2 -) and joins the particle in the sort.
 //
-// A record is one aligned sector (two with v^M). At 134M particles a load of
-// rows in device memory takes 3.5 ms, bound by the random sectors: records of
-// 48 bytes (which share sectors), written in pid order as well as into the
-// bins, with v^M gathered through the inverse of the old order, took 20.4.
+// A record is one aligned sector. At 134M particles a load of rows in device
+// memory takes 3.5 ms, bound by the random sectors: records of 48 bytes (which
+// share sectors), written in pid order as well as into the bins, with v^M
+// gathered through the inverse of the old order, took 20.4.
 struct Put32 {
   float4* rec;
   float4* bins;
   int64_t bin_cap;
-  int words;      // float4 a binned record: 2, or 4 with v^M
+  int words;      // float4 a binned record: 2, or 3 with v^M
   int* bin_over;
   int32_t *key, *rank, *count;
-  int32_t* cell;  // arrays (rec and bins null)
+  int32_t* cell;  // arrays (rec and bins null); m0 null: v^M is there already
   float *o0, *o1, *o2, *v0, *v1, *v2, *m0, *m1, *m2;
   uint32_t* pid;
 };
@@ -53,6 +53,11 @@ __device__ __forceinline__ void store_record(float4* p, const float4& a, const f
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
                "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
                : "memory");
+}
+
+__device__ __forceinline__ void put_vm32(const Put32& a, int64_t i, const float4& m) {
+  if (!a.m0) return;
+  a.m0[i] = m.x; a.m1[i] = m.y; a.m2[i] = m.z;
 }
 
 __device__ __forceinline__ void put32(const Put32& a, int64_t i, int32_t cell, const float* o, const float* v,
@@ -67,7 +72,12 @@ __device__ __forceinline__ void put32(const Put32& a, int64_t i, int32_t cell, c
         return;
       }
       q = a.bins + a.words * ((int64_t)cell * a.bin_cap + rk);
-      if (a.words == 4) store_record(q + 2, m, make_float4(0.f, 0.f, 0.f, 0.f));
+      if (a.words == 3) {  // 48 bytes: not sectors
+        q[0] = make_float4(o[0], o[1], o[2], v[0]);
+        q[1] = make_float4(v[1], v[2], __uint_as_float((uint32_t)i), 0.f);
+        q[2] = m;
+        return;
+      }
     } else {
       a.key[i] = cell;
       a.rank[i] = rk;
@@ -79,15 +89,15 @@ __device__ __forceinline__ void put32(const Put32& a, int64_t i, int32_t cell, c
   a.cell[i] = cell;
   a.o0[i] = o[0]; a.o1[i] = o[1]; a.o2[i] = o[2];
   a.v0[i] = v[0]; a.v1[i] = v[1]; a.v2[i] = v[2];
-  a.m0[i] = m.x; a.m1[i] = m.y; a.m2[i] = m.z;
   a.pid[i] = (uint32_t)i;
+  put_vm32(a, i, m);
 }
 
 struct Sample32Args {
   Params P;
   TimeTerms tt;
-  float4* vm;      // out: v^M (tau for the paper's f_v) by pid
-  int state;       // 0: v^M only
+  float4* vm;      // out: v^M (tau for the paper's f_v) by pid, or nullptr
+  int state;       // 0: v^M only (also into put's arrays, where it has them)
   Put32 put;
 };
 
@@ -105,16 +115,16 @@ __global__ void __launch_bounds__(kThreads) k_sample32(Sample32Args a) {
   float4 m;
   if (!paper) {
     m = make_float4(vm_sample32(P, 0, xi[3]), vm_sample32(P, 1, xi[4]), vm_sample32(P, 2, xi[5]), 0.f);
-    a.vm[i] = m;
-    if (!a.state) return;
+    if (a.vm) a.vm[i] = m;
+    if (!a.state) return put_vm32(a.put, i, m);
     for (int d = 0; d < 3; ++d) ci[d] = xm_sample32(P, a.tt, xi[d], &off[d]);
     vf[0] = m.x; vf[1] = m.y; vf[2] = m.z;
   } else {
     double tau[3];
     for (int d = 0; d < 3; ++d) tau[d] = tau_inv(xi[3 + d]);
     m = make_float4((float)tau[0], (float)tau[1], (float)tau[2], 0.f);
-    a.vm[i] = m;
-    if (!a.state) return;
+    if (a.vm) a.vm[i] = m;
+    if (!a.state) return put_vm32(a.put, i, m);
     for (int d = 0; d < 3; ++d) {
       double s, c;
       ci[d] = cell_offset32(wrap_unit(xm_solve_gen(a.tt, d, xi[d], &s, &c)), P.n, &off[d]);
@@ -222,7 +232,7 @@ __global__ void __launch_bounds__(kThreads) k_load32(Load32Args a) {
     v[d] = to_f32(svs[3 * threadIdx.x + d]);
   }
   float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (!a.put.rec && !(a.put.bins && a.put.words == 2)) m = a.vm[i];
+  if (a.put.bins ? a.put.words == 3 : a.put.m0 != nullptr) m = a.vm[i];
   put32(a.put, i, ci[0] + a.n * (ci[1] + a.n * ci[2]), off, v, m);
 }
 
@@ -2109,40 +2119,50 @@ static Put32 put_target(pic_ctx* c, LoadTarget target) {
   return a;
 }
 
+// where v^M by pid is written and read: kept, or behind the records
+static float4* vm_area(pic_ctx* c) {
+  return c->vm_by_pid ? c->vm_by_pid : reinterpret_cast<float4*>(c->stage) + 2 * c->P.np;
+}
+
 cudaError_t launch_sample32(pic_ctx* c, double t0, LoadTarget target) {
   Sample32Args a;
   a.P = c->P;
   a.tt = time_terms(c->P, t0);
-  a.vm = c->vm_by_pid;
+  a.vm = vm_area(c);
   a.state = 1;
   a.put = put_target(c, target);
   prof_begin(c);
   k_sample32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(a);
   prof_end(c, KC_SAMPLE);
   c->launches++;
+  c->vm_filled = c->vm_by_pid != nullptr;
   return cudaGetLastError();
 }
 
 cudaError_t launch_load32(pic_ctx* c, const double* x, const double* v, LoadTarget target, bool host) {
-  prof_begin(c);
-  if (!c->sampled) {
-    // the context's first state: v^M of every pid
-    Sample32Args s;
-    s.P = c->P;
-    s.tt = time_terms(c->P, 0.0);
-    s.vm = c->vm_by_pid;
-    s.state = 0;
-    s.put = Put32{};
-    k_sample32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(s);
-    c->launches++;
-  }
   Load32Args a;
   a.n = c->P.n;
   a.np = c->P.np;
   a.xs = x;
   a.vs = v;
-  a.vm = c->vm_by_pid;
+  a.vm = vm_area(c);
   a.put = put_target(c, target);
+  prof_begin(c);
+  if (!c->vm_filled) {
+    // v^M of every pid; rows in the staging area leave it no place there, and
+    // it goes straight into the arrays
+    const bool arrays = target == LoadTarget::kArrays && !c->vm_by_pid;
+    Sample32Args s;
+    s.P = c->P;
+    s.tt = time_terms(c->P, 0.0);
+    s.vm = arrays ? nullptr : vm_area(c);
+    s.state = 0;
+    s.put = arrays ? a.put : Put32{};
+    k_sample32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(s);
+    c->launches++;
+    c->vm_filled = c->vm_by_pid != nullptr;
+    if (arrays) a.put.m0 = nullptr;
+  }
   // v^M in the binned record where the load waits on the host link: 1.3 ms
   // less for the sort at 134M particles, but 2.3 ms more for the load's
   // stores, which only the link hides
@@ -2186,7 +2206,7 @@ cudaError_t launch_gather32(pic_ctx* c) {
   g.spid = c->pid[o];  // written in arrival order by the scatter
   if (c->rec_state) {
     g.rec = c->bin_state ? c->bins : reinterpret_cast<const float4*>(c->stage);
-    g.vm = c->vm_by_pid;
+    g.vm = vm_area(c);
     g.rec_words = c->bin_state ? c->bin_words : 2;
     g.bin_cap = c->bin_state ? c->bin_cap : 0;
     g.spid = nullptr;  // the pids come with the records

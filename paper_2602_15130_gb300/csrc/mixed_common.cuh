@@ -236,7 +236,7 @@ struct Gather32Args {
   int big_lo;             // cells above this count go to the block sort
   const uint32_t* spid;   // optional: pids in arrival order (slot s + e holds perm[s + e]'s pid)
   // optional: the source as records (o0 o1 o2 v0 | v1 v2 pid -) instead of
-  // in[] and pid_in, with v^M (m0 m1 m2 -) behind them (rec_words 4) or by
+  // in[] and pid_in, with v^M (m0 m1 m2 -) behind them (rec_words 3) or by
   // pid in vm (rec_words 2): a random source read so touches two 32-byte
   // sectors a particle instead of nine
   const float4* rec = nullptr;
@@ -255,7 +255,7 @@ __device__ __forceinline__ void gather_load32(const Gather32Args& a, const float
   if constexpr (kRec) {
     const float4* r = rb + a.rec_words * (int64_t)src;
     const float4 r0 = __ldg(r), r1 = __ldg(r + 1);
-    const float4 m = __ldg(a.rec_words == 4 ? r + 2 : a.vm + __float_as_uint(r1.z));
+    const float4 m = __ldg(a.rec_words == 3 ? r + 2 : a.vm + __float_as_uint(r1.z));
     d[0] = r0.x; d[1] = r0.y; d[2] = r0.z; d[3] = r0.w;
     d[4] = r1.x; d[5] = r1.y;
     d[6] = m.x; d[7] = m.y; d[8] = m.z;

@@ -467,6 +467,10 @@ void dev_free(pic_ctx* c, void* p) {
     if (e_ != cudaSuccess) return cuda_status(e_); \
   } while (0)
 
+// the reduction slots of the Poisson solve: the exchange's inboxes (FP64), or two
+// sets of two double-float partials a block
+size_t cg_red_bytes(const pic_ctx* c) { return c->mixed ? (size_t)32 * c->cg_grid : cg_slot_bytes(c->cg_grid); }
+
 // Every device array of the context, in one list for allocation and release.
 template <class F>
 void for_each_buffer(pic_ctx* c, F f) {
@@ -508,7 +512,6 @@ void for_each_buffer(pic_ctx* c, F f) {
       f((void**)&c->dvf[d], np * 4);
       if (c->nrep == 0) f((void**)&c->dvmf[d], np * 4);  // pic_collide_avg only
     }
-    if (c->nrep == 0) f((void**)&c->vm_by_pid, np * 16);
     f((void**)&c->Ef4, nc * 16);
     f((void**)&c->bf, nc * 4);
     f((void**)&c->phif, nc * 4);
@@ -535,7 +538,7 @@ void for_each_buffer(pic_ctx* c, F f) {
   f((void**)&c->corner, 8 * nc * 8);
   f((void**)&c->rho, nc * 8);
   f((void**)&c->rhs_part, (size_t)c->rhs_blocks * 8);
-  f((void**)&c->cg_red, cg_slot_bytes(c->cg_grid));
+  f((void**)&c->cg_red, cg_red_bytes(c));
   f((void**)&c->cg_bar, 64);
   f((void**)&c->cg_info, 64);
   f((void**)&c->cg_res, 64);
@@ -612,6 +615,19 @@ pic_status check_pending(pic_ctx* c) {
   return PIC_OK;
 }
 
+// v^M by pid (vm_by_pid), with the context's first state.
+void ensure_vm(pic_ctx* c) {
+  if (c->vm_tried) return;
+  c->vm_tried = true;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  const size_t bytes = (size_t)c->P.np * 16;
+  if (bytes <= free_b / 4) c->vm_by_pid = (float4*)dev_alloc(c, bytes);
+}
+
 // Bins for the records of a state in pid order, by cell: a capacity of four
 // times the mean particles per cell (a multiple of 32), if that is at most
 // kBigCell (larger cells take the block sort, which reads through perm), the
@@ -633,7 +649,7 @@ void ensure_bins(pic_ctx* c) {
     cudaGetLastError();
     return;
   }
-  c->bin_words_max = records * 64 <= free_b / 4 ? 4 : 2;
+  c->bin_words_max = records * 48 <= free_b / 4 ? 3 : 2;
   const size_t bytes = records * 16 * c->bin_words_max;
   if (bytes > free_b / 4) return;
   c->bins = (float4*)dev_alloc(c, bytes);
@@ -681,6 +697,7 @@ double time_at(const pic_ctx* c, double steps) { return c->t0 + steps * c->cfg.d
 // bins.
 pic_status records_then_sort(pic_ctx* c, double t, const double* xs, const double* vs, bool* binned) {
   ensure_bins(c);
+  ensure_vm(c);
   *binned = false;
   const bool host = xs && (in_host(xs) || in_host(vs));
   auto write = [&](LoadTarget target) -> cudaError_t {
@@ -980,6 +997,7 @@ void pic_destroy(pic_ctx* c) {
   dev_free(c, c->dlog_n);
   dev_free(c, c->bins);
   dev_free(c, c->bin_over);
+  dev_free(c, c->vm_by_pid);
   if (c->aux) {
     cudaStreamSynchronize(c->aux);
     cudaEventDestroy(c->aux_fork);
@@ -1188,7 +1206,7 @@ pic_status pic_create(const pic_config* cfg, void* stream, const pic_allocator* 
   if (e == cudaSuccess) e = cudaMemsetAsync(c->counters, 0, 64, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 0, 64, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->cg_info, 0, 64, c->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->cg_red, 0, cg_slot_bytes(c->cg_grid), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->cg_red, 0, cg_red_bytes(c), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->cg_res, 0, 64, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
@@ -1285,6 +1303,7 @@ pic_status pic_set_state(pic_ctx* c, const double* x, const double* v, double t0
       return check_pending(c);
     }
     c->cur = 0;
+    ensure_vm(c);
     CK(launch_load32(c, xs, vs, LoadTarget::kArrays, false));
   } else {
     c->cur = 0;

@@ -748,9 +748,12 @@ struct pic_ctx {
   double* dv[3];    // collision term per particle (sorted order)
   double* lor[3];   // dt q/m (E_p - E^M_p) of the last kick without drift
   bool lor_valid;   // lor matches the current order, positions and field
-  // precision form: v^M (tau for the paper's f_v) by pid, written with the
-  // context's first state
+  // precision form: v^M (tau for the paper's f_v) by pid, allocated with the
+  // context's first state where it takes at most a quarter of the free memory,
+  // and written then. Without it a state that needs v^M by pid forms it anew, in
+  // the staging area behind the records (vm_area).
   float4* vm_by_pid;
+  bool vm_tried, vm_filled;
   bool rec_state;   // the next sort reads the state from records, in the staging area or the bins
   // Bins for the records of a state in pid order ([ncell][bin_cap]; allocated
   // with the first state that is sampled or read in place, when they fit):
@@ -758,7 +761,7 @@ struct pic_ctx {
   // unless a cell outgrows its bin.
   float4* bins;
   int64_t bin_cap;  // 0: no bins
-  int bin_words, bin_words_max;  // float4 a record (2, or 4 with v^M): of the current ones, and room for
+  int bin_words, bin_words_max;  // float4 a record (2, or 3 with v^M): of the current ones, and room for
   int* bin_over;    // device flag: some cell held more than bin_cap particles
   bool bin_tried;   // the bins' allocation was attempted
   bool bin_state;   // the next sort reads the records from the bins
