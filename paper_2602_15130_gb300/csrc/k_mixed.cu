@@ -26,9 +26,11 @@ inline int blocks_for(int64_t n, int t = kThreads) {
 // Where a state in pid order goes: as arrays into the current buffer, or,
 // for the sort that follows, as 32-byte records (o0 o1 o2 v0 | v1 v2 pid -),
 // either straight into per-cell bins ([ncell][bin_cap], arrival rank r at
-// slot r; a rank at or above bin_cap sets *bin_over) or in pid order with
-// cell keys and arrival ranks. v^M depends only on the pid: it is kept by pid
-// (m0 m1 m2 -) and joins the particle in the sort.
+// slot r) or in pid order with cell keys and arrival ranks. A particle whose
+// rank is bin_cap or more goes to its pid's place among the latter, with its
+// cell in the record, and into a list (pid and rank in key and rank, *bin_over
+// long); k_unbin32 then brings the others there too. v^M depends only on the
+// pid: it is kept by pid (m0 m1 m2 -) and joins the particle in the sort.
 //
 // A record is one aligned sector. At 134M particles a load of rows in device
 // memory takes 3.5 ms, bound by the random sectors: records of 48 bytes (which
@@ -62,28 +64,30 @@ __device__ __forceinline__ void put_vm32(const Put32& a, int64_t i, const float4
 
 __device__ __forceinline__ void put32(const Put32& a, int64_t i, int32_t cell, const float* o, const float* v,
                                       const float4& m) {
-  if (a.rec || a.bins) {
+  if (a.rec) {
     // neighbours in pid order lie in unrelated cells: one atomic each
     const int32_t rk = atomicAdd(a.count + cell, 1);
-    float4* q = a.rec + 2 * i;
+    const float4 r0 = make_float4(o[0], o[1], o[2], v[0]);
+    const float4 r1 = make_float4(v[1], v[2], __uint_as_float((uint32_t)i), __int_as_float(cell));
+    if (a.bins && rk < a.bin_cap) {
+      float4* q = a.bins + a.words * ((int64_t)cell * a.bin_cap + rk);
+      if (a.words == 2) return store_record(q, r0, r1);
+      q[0] = r0; q[1] = r1; q[2] = m;  // 48 bytes: not sectors
+      return;
+    }
+    store_record(a.rec + 2 * i, r0, r1);
     if (a.bins) {
-      if (rk >= a.bin_cap) {
-        *a.bin_over = 1;
-        return;
-      }
-      q = a.bins + a.words * ((int64_t)cell * a.bin_cap + rk);
-      if (a.words == 3) {  // 48 bytes: not sectors
-        q[0] = make_float4(o[0], o[1], o[2], v[0]);
-        q[1] = make_float4(v[1], v[2], __uint_as_float((uint32_t)i), 0.f);
-        q[2] = m;
-        return;
-      }
+      const unsigned there = __activemask();
+      const int lane = threadIdx.x & 31, first = __ffs((int)there) - 1;
+      int32_t k = 0;
+      if (lane == first) k = atomicAdd(a.bin_over, __popc(there));
+      k = __shfl_sync(there, k, first) + __popc(there & ((1u << lane) - 1u));
+      a.key[k] = (int32_t)i;
+      a.rank[k] = rk;
     } else {
       a.key[i] = cell;
       a.rank[i] = rk;
     }
-    store_record(q, make_float4(o[0], o[1], o[2], v[0]),
-                 make_float4(v[1], v[2], __uint_as_float((uint32_t)i), 0.f));
     return;
   }
   a.cell[i] = cell;
@@ -91,6 +95,42 @@ __device__ __forceinline__ void put32(const Put32& a, int64_t i, int32_t cell, c
   a.v0[i] = v[0]; a.v1[i] = v[1]; a.v2[i] = v[2];
   a.pid[i] = (uint32_t)i;
   put_vm32(a, i, m);
+}
+
+// The bins' records to their pids' places and the permutation of all, when some
+// cell holds more than its bin (a cell's span of perm is one store a warp), so
+// that the source is read, or drawn, once. A load of 134M rows, 0.1% of them in
+// one corner of the box: 42.8 ms from pinned memory and 15.3 from device memory
+// (uniform rows 34.4 and 8.7); with a second pass over the rows 72.2 and 16.9.
+// Sampling 1.3M particles of the paper's problem, crowded: 2.7 ms, 4.7 by
+// drawing them twice.
+struct Unbin32Args {
+  int64_t ncell, bin_cap;
+  int words, n_over;
+  const float4* bins;
+  float4* rec;
+  const int32_t *start, *key, *rank;
+  int32_t* perm;
+};
+
+__global__ void __launch_bounds__(kThreads) k_unbin32(Unbin32Args a) {
+  const int lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, T = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t cell = t >> 5; cell < a.ncell; cell += T >> 5) {
+    const int32_t s = a.start[cell];
+    const int64_t c = min((int64_t)(a.start[cell + 1] - s), a.bin_cap);
+    for (int64_t r = lane; r < c; r += 32) {
+      const float4* q = a.bins + a.words * (cell * a.bin_cap + r);
+      const float4 r0 = q[0], r1 = q[1];
+      const uint32_t pid = __float_as_uint(r1.z);
+      a.perm[s + r] = (int32_t)pid;
+      store_record(a.rec + 2 * (int64_t)pid, r0, r1);
+    }
+  }
+  for (int64_t k = t; k < a.n_over; k += T) {
+    const int32_t pid = a.key[k];
+    a.perm[a.start[__float_as_int(a.rec[2 * (int64_t)pid + 1].w)] + a.rank[k]] = pid;
+  }
 }
 
 struct Sample32Args {
@@ -2106,15 +2146,14 @@ static Put32 put_target(pic_ctx* c, LoadTarget target) {
     return a;
   }
   a.count = c->count;
+  a.rec = reinterpret_cast<float4*>(c->stage);
+  a.key = c->key;
+  a.rank = c->rank;
   if (target == LoadTarget::kBins) {
     a.bins = c->bins;
     a.bin_cap = c->bin_cap;
     a.words = c->bin_words = 2;
     a.bin_over = c->bin_over;
-  } else {
-    a.rec = reinterpret_cast<float4*>(c->stage);
-    a.key = c->key;
-    a.rank = c->rank;
   }
   return a;
 }
@@ -2163,12 +2202,33 @@ cudaError_t launch_load32(pic_ctx* c, const double* x, const double* v, LoadTarg
     c->vm_filled = c->vm_by_pid != nullptr;
     if (arrays) a.put.m0 = nullptr;
   }
-  // v^M in the binned record where the load waits on the host link: 1.3 ms
-  // less for the sort at 134M particles, but 2.3 ms more for the load's
-  // stores, which only the link hides
+  // v^M in the binned record where the load waits on the host link, which hides
+  // the stores: 1.3 ms less for the sort at 134M particles (records of 64 bytes,
+  // whole sectors, take the same time and a third more memory)
   if (host && target == LoadTarget::kBins) c->bin_words = a.put.words = c->bin_words_max;
   k_load32<<<blocks_for(c->P.np), kThreads, 0, c->stream>>>(a);
   prof_end(c, KC_OTHER);
+  c->launches++;
+  return cudaGetLastError();
+}
+
+// start holds the cells' offsets; n_over: particles beyond their bins
+cudaError_t launch_unbin32(pic_ctx* c) {
+  Unbin32Args a;
+  a.ncell = c->P.ncell;
+  a.bin_cap = c->bin_cap;
+  a.words = c->bin_words;
+  a.n_over = c->bin_beyond;
+  a.bins = c->bins;
+  a.rec = reinterpret_cast<float4*>(c->stage);
+  a.start = c->start;
+  a.key = c->key;
+  a.rank = c->rank;
+  a.perm = c->perm;
+  const int64_t need = (32 * a.ncell + kThreads - 1) / kThreads, most = 16 * (int64_t)c->num_sms;
+  prof_begin(c);
+  k_unbin32<<<(int)(need < most ? need : most), kThreads, 0, c->stream>>>(a);
+  prof_end(c, KC_SORT);
   c->launches++;
   return cudaGetLastError();
 }
@@ -2230,6 +2290,7 @@ cudaError_t launch_gather32(pic_ctx* c) {
   c->cur = o;
   c->rec_state = false;
   c->bin_state = false;
+  c->bin_beyond = 0;
   return cudaGetLastError();
 }
 

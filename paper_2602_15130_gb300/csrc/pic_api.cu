@@ -673,8 +673,9 @@ pic_status sort_and_field(pic_ctx* c, double t, bool keys_done = false) {
     if (!keys_done) CK(launch_keys32(c));
     // records binned by cell need no permutation: the gather reads each
     // cell's bin
-    if (c->bin_state) CK(launch_scan(c));
+    if (c->bin_state || c->bin_beyond) CK(launch_scan(c));
     else CK(launch_scan_scatter(c));
+    if (c->bin_beyond) CK(launch_unbin32(c));
     CK(launch_gather32(c));
     CK(launch_rhs(c, t));
     CK(launch_cg32(c));
@@ -691,35 +692,34 @@ double time_at(const pic_ctx* c, double steps) { return c->t0 + steps * c->cfg.d
 
 // The precision form's state in pid order (sampled, or a caller's rows used
 // in place) written as records for the sort, and the sort with its field:
-// into the per-cell bins, and again as records in the staging area when a
-// cell outgrows its bin (or straight there without bins), which the sort
-// reads through a scatter and a random gather. *binned: the sort read the
-// bins.
+// into the per-cell bins, or without bins into the staging area, which the
+// sort reads through a scatter and a random gather. Where a cell outgrows its
+// bin the records move from the bins to the staging area. *binned: the sort
+// read the bins.
 pic_status records_then_sort(pic_ctx* c, double t, const double* xs, const double* vs, bool* binned) {
   ensure_bins(c);
   ensure_vm(c);
   *binned = false;
   const bool host = xs && (in_host(xs) || in_host(vs));
-  auto write = [&](LoadTarget target) -> cudaError_t {
-    const cudaError_t e = cudaMemsetAsync(c->count, 0, (size_t)c->P.ncell * 4, c->stream);
-    if (e != cudaSuccess) return e;
-    return xs ? launch_load32(c, xs, vs, target, host) : launch_sample32(c, t, target);
-  };
+  const LoadTarget target = c->bins ? LoadTarget::kBins : LoadTarget::kRecords;
+  CK(cudaMemsetAsync(c->count, 0, (size_t)c->P.ncell * 4, c->stream));
+  if (c->bins) CK(cudaMemsetAsync(c->bin_over, 0, sizeof(int), c->stream));
+  CK(xs ? launch_load32(c, xs, vs, target, host) : launch_sample32(c, t, target));
+  c->bin_beyond = 0;
   if (c->bins) {
-    CK(cudaMemsetAsync(c->bin_over, 0, sizeof(int), c->stream));
-    CK(write(LoadTarget::kBins));
-    int over = 1;
+    int over = 0;
     CK(cudaMemcpyAsync(&over, c->bin_over, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    c->bin_beyond = over;
     *binned = over == 0;
   }
-  if (!*binned) CK(write(LoadTarget::kRecords));
   c->rec_state = true;
   c->bin_state = *binned;
   pic_status s = sort_and_field(c, t, true);
   if (s != PIC_OK) {
     c->rec_state = false;
     c->bin_state = false;
+    c->bin_beyond = 0;
   }
   return s;
 }

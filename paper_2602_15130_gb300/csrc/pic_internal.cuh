@@ -762,7 +762,8 @@ struct pic_ctx {
   float4* bins;
   int64_t bin_cap;  // 0: no bins
   int bin_words, bin_words_max;  // float4 a record (2, or 3 with v^M): of the current ones, and room for
-  int* bin_over;    // device flag: some cell held more than bin_cap particles
+  int* bin_over;    // on the device: particles beyond bin_cap in their cells
+  int bin_beyond;   // that count for the next sort: where it is not zero, the records leave the bins
   bool bin_tried;   // the bins' allocation was attempted
   bool bin_state;   // the next sort reads the records from the bins
   int64_t binned_loads;  // state loads sorted from the bins (pic_stats)
@@ -966,6 +967,7 @@ cudaError_t launch_err_final(pic_ctx* c, int nblocks);
 enum class LoadTarget { kArrays, kBins, kRecords };
 cudaError_t launch_sample32(pic_ctx* c, double t0, LoadTarget target);
 cudaError_t launch_load32(pic_ctx* c, const double* x, const double* v, LoadTarget target, bool host);
+cudaError_t launch_unbin32(pic_ctx* c);       // binned records to their pids' places, and perm
 cudaError_t ensure_aux_stream(pic_ctx* c);    // the auxiliary stream and its events
 // the multigrid levels of an n^3 mesh (n a power of two >= 16, else 0) and
 // the floats their coarse levels need
