@@ -232,9 +232,9 @@ typedef struct {
 
 /* Optional device allocator (e.g. a framework's caching allocator). Both
  * callbacks are called on the creating thread; alloc returns NULL on
- * failure. Blocks may have any alignment: the library asks for 32 bytes more
- * than it uses and rounds their start up to 32 bytes. NULL selects
- * cudaMalloc / cudaFree. */
+ * failure. Blocks may have any alignment: one that does not start on 32 bytes
+ * goes back, and the library asks for 32 bytes more and rounds the start up.
+ * NULL selects cudaMalloc / cudaFree. */
 typedef struct {
   void* (*alloc)(void* user, uint64_t bytes);
   void (*free)(void* user, void* ptr);

@@ -24,13 +24,13 @@ inline int blocks_for(int64_t n, int t = kThreads) {
 
 // ------------------------------------------------- sampling and state load --
 // Where a state in pid order goes: as arrays into the current buffer, or,
-// for the sort that follows, as 32-byte records (o0 o1 o2 v0 | v1 v2 pid -),
-// either straight into per-cell bins ([ncell][bin_cap], arrival rank r at
-// slot r) or in pid order with cell keys and arrival ranks. A particle whose
-// rank is bin_cap or more goes to its pid's place among the latter, with its
-// cell in the record, and into a list (pid and rank in key and rank, *bin_over
-// long); k_unbin32 then brings the others there too. v^M depends only on the
-// pid: it is kept by pid (m0 m1 m2 -) and joins the particle in the sort.
+// for the sort that follows, as 32-byte records (o0 o1 o2 v0 | v1 v2 pid
+// cell), either straight into per-cell bins ([ncell][bin_cap], arrival rank r
+// at slot r) or in pid order with cell keys and arrival ranks. A particle whose
+// rank is bin_cap or more goes to its pid's place among the latter, and into a
+// list (pid and rank in key and rank, *bin_over long); k_unbin32 then brings
+// the others there too. v^M depends only on the pid: it is kept by pid (m0 m1 m2
+// -) and joins the particle in the sort.
 //
 // A record is one aligned sector. At 134M particles a load of rows in device
 // memory takes 3.5 ms, bound by the random sectors: records of 48 bytes (which

@@ -414,17 +414,20 @@ pic_status cuda_status(cudaError_t e) {
 }
 
 // Device memory, aligned to kAlign bytes: the widest load or store of the
-// kernels. A caller's allocator may hand out smaller granules: each of its
-// blocks has room to round the start up, and where that moves it the
-// allocator's own address is kept for the release.
+// kernels. A caller's allocator may hand out smaller granules: where a block
+// does not start on that boundary it is exchanged for one with room to round
+// the start up, and the allocator's own address is kept for the release.
 constexpr size_t kAlign = 32;
 
 void* dev_alloc(pic_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (c->have_alloc) {
-    void* raw = c->alloc.alloc(c->alloc.user, (uint64_t)(bytes + kAlign));
+    void* raw = c->alloc.alloc(c->alloc.user, (uint64_t)bytes);
+    if ((uintptr_t)raw % kAlign == 0) return raw;  // (or nullptr)
+    c->alloc.free(c->alloc.user, raw);
+    raw = c->alloc.alloc(c->alloc.user, (uint64_t)(bytes + kAlign));
     void* p = (void*)(((uintptr_t)raw + kAlign - 1) / kAlign * kAlign);
-    if (p == raw) return p;  // (or nullptr)
+    if (p == raw) return p;
     void** moved = (void**)realloc(c->moved, sizeof(void*) * 2 * (size_t)(c->n_moved + 1));
     if (!moved) {
       c->alloc.free(c->alloc.user, raw);
