@@ -337,14 +337,16 @@ pic_status pic_set_state(pic_ctx* ctx, const double* x, const double* v, double 
  * device wait. Single contexts: the next Poisson solve (of pic_sample_mms,
  * pic_set_state or pic_step) launches one block that leaves before its
  * first grid barrier, so the other blocks wait for an arrival that never
- * comes. Batches: the next pic_step's persistent launch leaves one work
- * item (the first drift-kick tile of a replicate) uncounted, so the items
- * that depend on it wait for a completion that never comes. Either bounded
- * wait (4e9 SM cycles, about 2 s) ends the launch. That call returns
- * PIC_ETIMEOUT, and the field and the state it moves are invalid. The
- * context stays usable: the next pic_sample_mms or pic_set_state starts
- * clean. PIC_EINVAL for a single-context solve of one block (nothing would
- * wait). */
+ * comes; that solve takes the cooperative grid also where the mesh is small
+ * enough for one cluster of blocks, whose hardware barriers wait for nothing
+ * but its own, co-scheduled blocks. Batches: the next pic_step's persistent
+ * launch leaves one work item (the first drift-kick tile of a replicate)
+ * uncounted, so the items that depend on it wait for a completion that never
+ * comes. Either bounded wait (4e9 SM cycles, about 2 s) ends the launch. That
+ * call returns PIC_ETIMEOUT, and the field and the state it moves are
+ * invalid. The context stays usable: the next pic_sample_mms or pic_set_state
+ * starts clean. PIC_EINVAL for a single context of at most 1,024 nodes (n <=
+ * 10). */
 pic_status pic_inject_barrier_stall(pic_ctx* ctx);
 
 /* Copy mesh quantities out (any pointer may be NULL): rho [n^3] (the CIC

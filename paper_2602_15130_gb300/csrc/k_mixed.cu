@@ -2058,8 +2058,9 @@ __global__ void __launch_bounds__(kThreads) k_err_partial32(Err32Args a) {
         e -= floor(e + 0.5);
         vals[d] = e * e;
         vals[7 + d] = fabs(e);
-        // (normcdfinv, whose values give sampled velocities the same norm bits
-        // in any order of the particles that was tested)
+        // normcdfinv, not its table (1.4 ms of 16 replicates' norms): the sums of
+        // the same particles in another order round differently, and with the
+        // table's values the norms of a sampled state did so in the last bit
         const double vmd = paper ? tau_inv(xi[3 + d]) * a.tt.vh[d] : P.vmean[d] + P.vsig * normcdfinv(xi[3 + d]);
         const double ev = (double)vs[d] - vmd;
         vals[3 + d] = ev * ev;

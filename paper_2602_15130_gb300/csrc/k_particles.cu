@@ -144,10 +144,10 @@ __global__ void __launch_bounds__(kThreads) k_store_dv(StoreDvArgs a) {
 //    (hs_R64) instead of an exponential, an error function, a square root
 //    and a division.
 // Before, with the test and the source in FP64 and each lane scattering its
-// own pairs, the FP64 pipe was 85% busy; a call now takes 0.36 ms instead of
-// 1.36 (32^3 cells of 32, K = 16; 168 FP64 instructions per 32 particles,
-// the pipe 95% busy), 0.53 instead of 2.97 (12^3 cells of 101, K = 243) and
-// 98 us instead of 158 (8^3 cells of 8, K = 16: latency of the few warps).
+// own pairs, the FP64 pipe was 85% busy; a call now takes 0.32 ms instead of
+// 1.36 (32^3 cells of 32, K = 16), 0.47 instead of 2.97 (12^3 cells of 101,
+// K = 243) and 93 us instead of 158 (8^3 cells of 8, K = 16: latency of the few
+// warps).
 //
 // Working velocities: bit l of mask[p] says that lane l has changed particle
 // p of its cell. The first kList changed particles of a lane keep their

@@ -554,8 +554,10 @@ __device__ __forceinline__ double normal_quantile(const Params& P, double xi) {
 }
 
 // Sampling of the precision form, the general path's floats bit for bit: the
-// tables' value where every value within their error rounds to the same float
-// (all but one in a million), else the general path.
+// tables' value where every value within their error rounds to the same float,
+// else the general path. That takes one velocity in some 200,000, and one
+// coordinate in 30,000 at n = 8, 3,900 at n = 64 and 2,000 at n = 128, since an
+// offset carries the error n times.
 //
 // (float)(mean + sigma Phi^{-1}(xi))
 __device__ __forceinline__ float vm_sample32(const Params& P, int d, double xi) {
